@@ -273,6 +273,35 @@ __device__ __forceinline__ int activate(const ConvArgs& args, int v, int k) {
   return v;
 }
 
+// The same for NC consecutive output channels kbase .. kbase + NC - 1 of one pixel.  Every lane of the warp
+// needs the same bias values, so what costs is the number of load instructions, not the bytes: a full run of
+// channels whose bias starts on a 16-byte boundary reads four values per load (with one load per channel the
+// 64-channel NHWC int8 layer of 8 x 112 x 112 pixels took 29.1 us, without bias and ReLU 11.3, so 13.6).
+template <int NC>
+__device__ __forceinline__ void activate_columns(const ConvArgs& args, int32_t* v, int kbase, int bias_off) {
+  if (args.bias != nullptr) {
+    const int32_t* b = args.bias + bias_off + kbase;
+    if (kbase + NC <= args.K && (bias_off & 3) == 0) {  // (kbase is a multiple of 16, the buffer 256-byte aligned)
+#pragma unroll
+      for (int j = 0; j < NC; j += 4) {
+        const int4 q = __ldg(reinterpret_cast<const int4*>(b + j));
+        v[j] += q.x;
+        v[j + 1] += q.y;
+        v[j + 2] += q.z;
+        v[j + 3] += q.w;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < NC; ++j)
+        if (kbase + j < args.K) v[j] += __ldg(b + j);
+    }
+  }
+  if (args.relu) {
+#pragma unroll
+    for (int j = 0; j < NC; ++j) v[j] = max(v[j], 0);
+  }
+}
+
 // Loads NC consecutive accumulator columns of this thread's TMEM lane.
 template <int NC>
 __device__ __forceinline__ void tmem_ld(uint32_t taddr, int32_t* v);
@@ -332,11 +361,7 @@ __device__ __forceinline__ void store_columns(const ConvArgs& args, int32_t* v, 
     }
     return;
   }
-  if (args.bias != nullptr || args.relu) {
-#pragma unroll
-    for (int j = 0; j < NC; ++j)
-      if (kbase + j < K) v[j] = activate(args, v[j], bias_off + kbase + j);
-  }
+  activate_columns<NC>(args, v, kbase, bias_off);
   if (!nhwc) {
     // NKPQ: for a fixed column the 32 lanes of a warp hold 32 consecutive pixels, so every
     // store instruction writes one contiguous run.
