@@ -22,6 +22,8 @@ struct b2c_plan {
   GatherEntry* table = nullptr;  // device, plan-owned (stencil lookup table)
   int32_t* table32 = nullptr;    // device, plan-owned (offsets into the staged window)
   WindowGeom win = {0, 0, 0, 0, 0};
+  PlaneArgs plane = {};          // plane kernel: geometry and device tables (plane.num_mma > 0: this plan runs it)
+  uint64_t* mma_table = nullptr; // device, plan-owned: A descriptors of the plane kernel
   TmaView view = {};             // geometry handed to the im2col-mode-TMA kernel (TMA-view variants)
   int32_t* wtable = nullptr;     // device, plan-owned: packed weight column -> index into one filter, -1 = zero
   int table_len = 0;
@@ -262,6 +264,14 @@ void fill_common_args(b2c_plan* p) {
       a.out_pad_h = d.pad_h;
       a.out_pad_w = d.pad_w;
     }
+  } else if (p->plane.num_mma > 0) {
+    p->amode = A_PLANE;
+    a.tile_n = p->plane.tile_n;
+    a.tmem_cols = p->plane.tmem_cols;
+    a.num_kb = p->plane.num_mma;
+    a.split_k = 1;
+    a.cluster_split = 0;
+    return;
   } else if (p->emb.variant == B2C_VARIANT_IM2COL_WINDOW) {
     WindowTile wt;
     window_tile_geom(p->g, &wt);  // legal: checked when the plan was created
@@ -405,7 +415,24 @@ void fill_common_args(b2c_plan* p) {
   a.stages = stages;
 }
 
-int create_plan_for(const Geom& g, const b2c_embedding& emb, b2c_plan** out, int group_count = 1) {
+// The embeddings of g, numbered; every variant but the channel pack goes through the stencil lookup table.
+void enumerate_legal(const Geom& g, std::vector<b2c_embedding>* all) {
+  enumerate_embeddings(g, all);
+  if (!table_variant_legal(g))
+    all->erase(std::remove_if(all->begin(), all->end(), [](const b2c_embedding& e) { return e.variant != B2C_VARIANT_CP_TMA; }),
+               all->end());
+  for (size_t i = 0; i < all->size(); ++i) (*all)[i].id = (int)i;
+}
+
+// Embeddings that differ only in the schedule of the plane kernel share all their fields: which of them entry idx of
+// an enumeration is.
+int schedule_of(const std::vector<b2c_embedding>& all, int idx) {
+  int nth = 0;
+  for (int i = 0; i < idx; ++i) nth += all[i].variant == all[idx].variant && all[i].tile_n == all[idx].tile_n ? 1 : 0;
+  return all[idx].variant == B2C_VARIANT_IM2COL_WINDOW ? nth : 0;
+}
+
+int create_plan_for(const Geom& g, const b2c_embedding& emb, int nth, b2c_plan** out, int group_count = 1) {
   b2c_plan* p = new (std::nothrow) b2c_plan();
   if (!p) return B2C_E_INVALID_ARG;
   p->g = g;
@@ -419,6 +446,10 @@ int create_plan_for(const Geom& g, const b2c_embedding& emb, b2c_plan** out, int
   };
   if (cudaMalloc(&p->status, kStatusWords * sizeof(int)) != cudaSuccess) return fail(B2C_E_CUDA);
   if (cudaMemset(p->status, 0, kStatusWords * sizeof(int)) != cudaSuccess) return fail(B2C_E_CUDA);
+  std::vector<uint64_t> mma;
+  std::vector<int32_t> wsrc;
+  const bool plane = emb.variant == B2C_VARIANT_IM2COL_WINDOW && plane_wanted(g) &&
+                     plane_plan(g, group_count, emb.tile_n, nth, &p->plane, &mma, &wsrc);
   if (is_tma_view_variant(emb.variant)) {
     if (!tma_view_for(g, emb.variant, &p->view)) return fail(B2C_E_UNSUPPORTED);
     const TmaView& v = p->view;
@@ -476,6 +507,14 @@ int create_plan_for(const Geom& g, const b2c_embedding& emb, b2c_plan** out, int
       if (cudaMemcpy(p->wtable, wt.data(), wt.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess)
         return fail(B2C_E_CUDA);
     }
+  } else if (plane) {
+    p->w_packed_bytes = (size_t)group_count * p->plane.cols * p->plane.w_bytes;
+    if (cudaMalloc(&p->mma_table, mma.size() * sizeof(uint64_t)) != cudaSuccess) return fail(B2C_E_CUDA);
+    if (cudaMemcpy(p->mma_table, mma.data(), mma.size() * sizeof(uint64_t), cudaMemcpyHostToDevice) != cudaSuccess)
+      return fail(B2C_E_CUDA);
+    if (cudaMalloc(&p->wtable, wsrc.size() * sizeof(int32_t)) != cudaSuccess) return fail(B2C_E_CUDA);
+    if (cudaMemcpy(p->wtable, wsrc.data(), wsrc.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess)
+      return fail(B2C_E_CUDA);
   } else {
     int K_pad = variant_k_pad(g, emb.variant);
     p->w_packed_bytes = (size_t)d.K * K_pad * group_count;  // grouped: the filters of all groups, one block of K rows each
@@ -543,6 +582,13 @@ int create_plan_for(const Geom& g, const b2c_embedding& emb, b2c_plan** out, int
   // Room for one extra box row block so that a TMA box never starts past the allocation.
   if (cudaMalloc(&p->w_packed, p->w_packed_bytes + 256) != cudaSuccess) return fail(B2C_E_CUDA);
   fill_common_args(p);
+  if (p->amode == A_PLANE) {
+    p->plane.w = reinterpret_cast<const uint8_t*>(p->w_packed);
+    p->plane.mma_table = p->mma_table;
+    p->ws_total = 0;
+    *out = p;  // (no tensor maps: raw rows and weights travel by plain bulk copies)
+    return B2C_OK;
+  }
   p->ws_total = workspace_bytes_for(g, emb.variant, emb.tile_n, emb.split_k, is_swapped(emb));
   if (p->fused_pack) {
     p->ws_ctl_offset = (p->ws_total + 255) / 256 * 256;
@@ -702,11 +748,7 @@ int b2c_enumerate(const b2c_conv_desc* desc, b2c_embedding* out, int32_t cap, in
   int rc = resolve_geom(desc, &g);
   if (rc != B2C_OK) return rc;
   std::vector<b2c_embedding> all;
-  enumerate_embeddings(g, &all);
-  if (!table_variant_legal(g))
-    all.erase(std::remove_if(all.begin(), all.end(), [](const b2c_embedding& e) { return e.variant != B2C_VARIANT_CP_TMA; }),
-              all.end());  // every other variant goes through the stencil lookup table
-  for (size_t i = 0; i < all.size(); ++i) all[i].id = (int)i;
+  enumerate_legal(g, &all);
   *count = (int32_t)all.size();
   for (int i = 0; i < cap && i < (int)all.size(); ++i) out[i] = all[i];
   return all.empty() ? B2C_E_UNSUPPORTED : B2C_OK;
@@ -718,18 +760,15 @@ int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_
   Geom g;
   int rc = resolve_geom(desc, &g);
   if (rc != B2C_OK) return rc;
-  int32_t count = 0;
-  rc = b2c_enumerate(desc, nullptr, 0, &count);
-  if (rc != B2C_OK) return rc;
-  std::vector<b2c_embedding> all(count);
-  rc = b2c_enumerate(desc, all.data(), count, &count);
-  if (rc != B2C_OK) return rc;
+  std::vector<b2c_embedding> all;
+  enumerate_legal(g, &all);
+  if (all.empty()) return B2C_E_UNSUPPORTED;
   if (policy_or_id < B2C_POLICY_AUTO_TIMED_CONCURRENT) return B2C_E_INVALID_ARG;
   const int lanes = policy_or_id == B2C_POLICY_AUTO_TIMED_CONCURRENT ? kMaxLanes : 1;
   if (policy_or_id != B2C_POLICY_AUTO_TIMED && policy_or_id != B2C_POLICY_AUTO_TIMED_CONCURRENT) {
     int idx = pick_by_policy(all, policy_or_id);
     if (idx < 0) return B2C_E_INVALID_ARG;
-    return create_plan_for(g, all[idx], out);
+    return create_plan_for(g, all[idx], schedule_of(all, idx), out);
   }
   // Timed selection (Section 6.1: the best candidates by the overhead metric are tuned and the
   // fastest is kept).  All schedules of the five lowest-overhead (axis map, layout variant)
@@ -774,7 +813,7 @@ int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_
     // A candidate that cannot be built or run (a tensor map the driver refuses, an allocation that
     // fails, a device wait that expires) is left out of the selection; the others are still timed.
     b2c_plan* p = nullptr;
-    rc = create_plan_for(g, all[i], &p);
+    rc = create_plan_for(g, all[i], schedule_of(all, (int)i), &p);
     if (rc == B2C_OK) rc = b2c_plan_set_weights(p, w, st);
     if (rc == B2C_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = B2C_E_CUDA;
     float us = -1;
@@ -793,7 +832,7 @@ int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_
   }
   cleanup();
   if (best < 0) return first_error != B2C_OK ? first_error : B2C_E_UNSUPPORTED;
-  return create_plan_for(g, all[best], out);
+  return create_plan_for(g, all[best], schedule_of(all, best), out);
 }
 
 int b2c_plan_create_grouped(const b2c_conv_desc* desc, int32_t groups, b2c_plan** out) {
@@ -858,7 +897,7 @@ int b2c_plan_create_grouped(const b2c_conv_desc* desc, int32_t groups, b2c_plan*
   }
   // one sub-plan runs all groups in one launch (the group is a grid axis of the kernel)
   b2c_plan* sub = nullptr;
-  rc = create_plan_for(sg, all[pick], &sub, run_groups);
+  rc = create_plan_for(sg, all[pick], 0, &sub, run_groups);
   if (rc != B2C_OK) {
     b2c_plan_destroy(p);
     return rc;
@@ -994,6 +1033,9 @@ static int set_weights_one(b2c_plan* p, const int8_t* w, cudaStream_t st) {
   if (p->emb.variant == B2C_VARIANT_CP_TMA || p->emb.variant == B2C_VARIANT_DILATION_PACK ||
       p->emb.variant == B2C_VARIANT_CP_SHIFT)
     CUDA_TRY(launch_pack_weights_cp(w, p->w_packed, d.K, d.C, d.R, d.S, p->C_pad, st));
+  else if (p->amode == A_PLANE)
+    CUDA_TRY(launch_pack_weights_plane(w, p->w_packed, p->group_count, d.K, p->g.Kg, p->plane.tile_n, p->plane.cols,
+                                       p->plane.num_mma, p->wtable, st));
   else if (is_tma_view_variant(p->emb.variant))
     CUDA_TRY(launch_pack_weights_table(w, p->w_packed, d.K, p->g.Kg, p->view.R * p->view.S * p->view.C, p->wtable, st));
   else
@@ -1135,6 +1177,10 @@ static int run_convolve(b2c_plan* p, const int8_t* x, int32_t* y32, int8_t* y8, 
       CUDA_TRY(cudaMemsetAsync(a.pk_ctl, 0, (size_t)(d.N + 1) * sizeof(int), st));
     }
     CUDA_TRY(launch_conv_mma_pair(p->amode, &tmap_a, &p->tmap_b, a, st));
+  } else if (p->amode == A_PLANE) {
+    PlaneArgs pl = p->plane;
+    pl.x_bytes = (long long)(d.N - 1) * a.x_stride_n + (long long)d.C * d.H * d.W * a.groups;
+    CUDA_TRY(launch_conv_mma_plane(a, pl, st));
   } else if (p->amode == A_WINDOW) {
     CUDA_TRY(launch_conv_mma_window(&tmap_a, &p->tmap_b, a, st));
   } else
@@ -1340,6 +1386,7 @@ void b2c_plan_destroy(b2c_plan* p) {
   cudaFree(p->w_expanded);
   cudaFree(p->table);
   cudaFree(p->table32);
+  cudaFree(p->mma_table);
   cudaFree(p->wtable);
   cudaFree(p->status);
   cudaFree(p->bias_buf);

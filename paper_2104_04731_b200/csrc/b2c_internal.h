@@ -78,7 +78,7 @@ struct Dbg {
   int* status = nullptr;         // [0] status word, [1] site, [2..3] byte offset of the first bad access from its range start
 };
 
-enum AMode { A_TILED = 0, A_IM2COL_TMA = 1, A_GATHER = 2, A_STAGED = 3, A_SHIFT = 4, A_WINDOW = 5 };
+enum AMode { A_TILED = 0, A_IM2COL_TMA = 1, A_GATHER = 2, A_STAGED = 3, A_SHIFT = 4, A_WINDOW = 5, A_PLANE = 6 };
 
 // Everything the MMA kernel needs besides its two tensor maps.
 struct ConvArgs {
@@ -170,6 +170,36 @@ struct ConvArgs {
   // then max(., 0) when relu != 0
   const int32_t* bias;
   int relu;
+};
+
+// Geometry of the window unroll over planes of units (A_PLANE, conv_mma_plane.cu); the kernel takes it beside ConvArgs.
+constexpr int kPlaneMinTiles = 2500;        // accumulator tiles of a problem from which the plane kernel runs it
+constexpr int kMaxStridePhases = 8;         // strides the window unroll handles
+constexpr int kPlaneMargin = 64;           // readable bytes on either side of the staged raw rows
+constexpr int kMaxAcc = 8;                  // accumulator ring
+constexpr int kPlaneSmemMax = 224 * 1024;  // dynamic shared memory of one block
+struct PlaneArgs {
+  int runw;      // 0: channel form (unit = 16 channels of a pixel), else words per run of the row form
+  int aligned;   // channel form: 2 = flat groups of four pixels, 1 = every row of every channel starts on a word
+  int sh, sw;    // strides
+  int ndh, ndw;  // row and column stride phases the taps use (row form: ndw = 1)
+  int max_dh;    // largest row phase
+  int8_t row_phase[kMaxStridePhases];  // phase index -> row phase
+  int8_t col_phase[kMaxStridePhases];  // column phase -> phase index, -1 if no tap uses it
+  int planes, pitch, rpi, total_rows;  // units per position; positions per grid row; grid rows per image and in all
+  int max_ri;                          // grid rows the taps reach below a window's output rows
+  int th, cr, tiles;                   // output grid rows of a window, grid rows of a raw chunk, accumulator tiles
+  int seg_rows, segs, blocks;          // output grid rows of a segment (walked by one block), segments, blocks
+  int plane_bytes, win_bytes, num_mma;
+  int whole_images, img_slot, c_pitch, raw_bytes;  // raw staging: whole images, or one slot per channel
+  int gpr, run_groups, zero_fill;                  // builder items per grid row (groups of columns)
+  int w_bytes;                                     // packed weights of one group and column tile
+  int nbuf, per_sm, win_stages, raw_stages, smem;
+  int tile_n, cols, tmem_cols;                     // column tile, column tiles, tensor-memory columns
+  FastDiv div_rpi, div_pitch, div_gpr, div_nu, div_sw, div_overlap, div_w, div_hw4;
+  const uint8_t* w;            // packed weights: [group][column tile][MMA][half][channel][16 bytes]
+  const uint64_t* mma_table;   // A descriptor of every MMA relative to the window: start (units) | distance of the halves << 16
+  long long x_bytes;           // bytes of the whole input tensor
 };
 
 // Programmatic dependent launch: a kernel launched through launch_pdl may start while the previous
@@ -363,6 +393,14 @@ struct WindowTile {
 };
 bool window_tile_geom(const Geom& g, WindowTile* wt);
 
+// The nth schedule of the plane kernel with column tile tile_n (0: any) for `groups` groups of the convolution g (1: g
+// itself), the lowest estimate first; false if there is none.  With table / wsrc: the MMA list (see
+// PlaneArgs::mma_table) and, per packed weight byte of one channel (32 per MMA), its index in a filter or -1.
+bool plane_plan(const Geom& g, int groups, int tile_n, int nth, PlaneArgs* pl, std::vector<uint64_t>* table = nullptr,
+                std::vector<int32_t>* wsrc = nullptr);
+// Which of the two kernels runs the window unroll of g: true for the plane kernel, where it applies.
+bool plane_wanted(const Geom& g);
+
 // --- tma.cpp -----------------------------------------------------------------------------------
 // Tensor-map encoders obtained through cudaGetDriverEntryPoint (no link-time libcuda dependency).
 int encode_tiled_2d(CUtensorMap* map, const void* base, uint64_t inner, uint64_t outer, uint64_t row_stride_bytes,
@@ -389,6 +427,10 @@ cudaError_t launch_pack_weights_table(const int8_t* w, int8_t* out, int K, int K
 cudaError_t launch_expand_group_weights(const int8_t* w, int8_t* out, int K, int cg, int kg, int m, int RS, cudaStream_t st);
 cudaError_t launch_pack_weights_rows(const int8_t* w, int8_t* out, int K, int Kg, int K_pad, int S, int S_run,
                                      cudaStream_t st);
+// Weights of the plane kernel: out[group][column tile][MMA][half][tile_n channels][16], byte b of half u of MMA m
+// = filter element wsrc[(2m + u) * 16 + b] (zero where that is -1 and for channels past K).
+cudaError_t launch_pack_weights_plane(const int8_t* w, int8_t* out, int groups, int K, int Kg, int tile_n, int cols, int num_mma,
+                                       const int32_t* wsrc, cudaStream_t st);
 cudaError_t launch_im2col(const int8_t* x, int8_t* a, const GatherEntry* table, long long Mg, int PQ, int Q, int H,
                           int W, int stride_h, int stride_w, int pad_h, int pad_w, long long x_stride_n,
                           int x_stride_h, int x_stride_w, int K_pad, cudaStream_t st, const Dbg& dbg = Dbg());
@@ -412,6 +454,7 @@ cudaError_t launch_conv_mma_pair(int amode, const CUtensorMap* tmap_a, const CUt
 size_t conv_mma_pair_smem_bytes(const ConvArgs& args);
 cudaError_t launch_conv_mma_window(const CUtensorMap* tmap_x, const CUtensorMap* tmap_b, const ConvArgs& args, cudaStream_t st);
 size_t conv_mma_window_smem_bytes(const ConvArgs& args);
+cudaError_t launch_conv_mma_plane(const ConvArgs& args, const PlaneArgs& pl, cudaStream_t st);
 // Geometry of the fused activation pack; false when the tensor has no bulk-copy form.
 bool fused_pack_geometry(int C, int H, int W, int C_pad, int* ct, int* pt, int* hw_tiles, int* ctiles, int* smem);
 cudaError_t launch_bounded_wait_selftest(int* status, cudaStream_t st);

@@ -380,6 +380,26 @@ __global__ void pack_weights_rows_kernel(const int8_t* __restrict__ w, int8_t* _
   }
 }
 
+// Weights of the plane kernel, in the order its MMAs read them: [group][column tile][MMA][half][channel][16].
+__global__ void pack_weights_plane_kernel(const int8_t* __restrict__ w, int8_t* __restrict__ out, int groups, int K, int Kg,
+                                           int tile_n, int cols, int num_mma, const int32_t* __restrict__ wsrc) {
+  const long long total = (long long)groups * cols * num_mma * 32 * tile_n;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int b = (int)(i & 15);
+    long long r = i >> 4;
+    const int kk = (int)(r % tile_n);
+    r /= tile_n;
+    const int unit = (int)(r % (num_mma * 2));
+    r /= num_mma * 2;
+    const int ct = (int)(r % cols);
+    const long long grp = r / cols;
+    const int k = ct * tile_n + kk;
+    const int src = wsrc[unit * 16 + b];
+    out[i] = (k < K && src >= 0) ? w[(grp * K + k) * Kg + src] : (int8_t)0;
+  }
+}
+
 // Explicit stencil unroll.  One thread produces 16 consecutive reduction entries of one output
 // pixel's row and stores them as one 16-byte vector; the window geometry comes from a lookup
 // table indexed by the reduction position, so no per-element division is needed.
@@ -786,6 +806,13 @@ cudaError_t launch_pack_weights_rows(const int8_t* w, int8_t* out, int K, int Kg
                                      cudaStream_t st) {
   const long long total = (long long)K * K_pad;
   pack_weights_rows_kernel<<<grid_for(total, 256), 256, 0, st>>>(w, out, K, Kg, K_pad, S, S_run);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pack_weights_plane(const int8_t* w, int8_t* out, int groups, int K, int Kg, int tile_n, int cols, int num_mma,
+                                       const int32_t* wsrc, cudaStream_t st) {
+  const long long total = (long long)groups * cols * num_mma * 32 * tile_n;
+  pack_weights_plane_kernel<<<grid_for(total, 256), 256, 0, st>>>(w, out, groups, K, Kg, tile_n, cols, num_mma, wsrc);
   return cudaGetLastError();
 }
 

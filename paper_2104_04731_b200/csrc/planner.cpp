@@ -9,7 +9,9 @@
 // directly, ranks it with the overhead terms of Section 4.4 and leaves the final choice to
 // measured device time, as Section 6.1 does with its five best candidates.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
+#include <utility>
 
 #include "b2c_internal.h"
 
@@ -373,8 +375,377 @@ bool window_tile_geom(const Geom& g, WindowTile* wt) {
   return wt->mtot <= 0x7FFFFF00LL && wt->smem <= 200 * 1024 && (long long)d.N * wt->tiles_h * wt->tiles_w < 0x7FFFFFFFLL;
 }
 
+// ---- window unroll over planes of units (B2C_VARIANT_IM2COL_WINDOW) ------------------------------------------------------------------
+namespace {
+
+// One form of the units (see conv_mma_plane.cu): which units a position has, and where the MMAs find them.
+struct PlaneForm {
+  int runw, ndh, ndw, planes, run_groups;
+  int qb;  // row form: columns of a builder item
+  int max_dh, max_ri, max_si;  // largest row phase, vertical and horizontal shift in grid positions
+  int8_t row_phase[kMaxStridePhases], col_phase[kMaxStridePhases];
+  int pitch, rpi;
+  struct Unit {
+    int plane, ri, si;
+    int src[16];  // filter element of every byte, -1 = zero
+  };
+  std::vector<Unit> units;
+};
+
+bool plane_form(const Geom& g, bool row_form, PlaneForm* f) {
+  const b2c_conv_desc& d = g.d;
+  const int sh = d.stride_h, sw = d.stride_w;
+  if (sh > kMaxStridePhases || sw > kMaxStridePhases) return false;
+  // (row form: from 8 channels on the 16-channel units are at least half full, and their builder moves more per load:
+  // 16 x 14 x 14, 15501 images, 97 us against 117)
+  if (row_form && (d.dil_w != 1 || d.S > 24 || d.C >= 8)) return false;
+  int rowidx[kMaxStridePhases];
+  std::fill(rowidx, rowidx + kMaxStridePhases, -1);
+  std::fill(f->row_phase, f->row_phase + kMaxStridePhases, (int8_t)0);
+  std::fill(f->col_phase, f->col_phase + kMaxStridePhases, (int8_t)-1);
+  f->max_dh = f->max_ri = f->max_si = 0;
+  for (int r = 0; r < d.R; ++r) {
+    rowidx[(long long)r * d.dil_h % sh] = 0;
+    f->max_ri = std::max<long long>(f->max_ri, (long long)r * d.dil_h / sh);
+  }
+  f->ndh = 0;
+  for (int p = 0; p < sh; ++p)
+    if (rowidx[p] == 0) {
+      f->row_phase[f->ndh] = (int8_t)p;
+      rowidx[p] = f->ndh++;
+      f->max_dh = p;
+    }
+  f->units.clear();
+  if (row_form) {
+    // Runs of RUNW words of one (channel, row phase); G of them make U units.
+    f->ndw = 1;
+    f->runw = d.S <= 4 ? 1 : (d.S <= 8 ? 2 : (d.S <= 16 ? 4 : 6));
+    const int G = f->runw == 1 ? 4 : (f->runw == 4 ? 1 : 2), U = G * f->runw / 4;
+    f->run_groups = (d.C * f->ndh + G - 1) / G;
+    f->qb = sw <= 2 ? 4 : 1;
+    f->planes = f->run_groups * U;
+    if (f->planes > 64) return false;
+    for (int plane = 0; plane < f->planes; ++plane)
+      for (int ri = 0; ri <= f->max_ri; ++ri) {
+        PlaneForm::Unit u;
+        u.plane = plane;
+        u.ri = ri;
+        u.si = 0;
+        bool any = false;
+        for (int b = 0; b < 16; ++b) {
+          const int word = (plane % U) * 4 + b / 4;
+          const int run = plane / U * G + word / f->runw;
+          const int s = word % f->runw * 4 + b % 4, c = run / f->ndh, dh = f->row_phase[run % f->ndh];
+          const long long off = (long long)ri * sh + dh;
+          const int r = (int)(off / d.dil_h);
+          u.src[b] = (c < d.C && s < d.S && off % d.dil_h == 0 && r < d.R) ? (c * d.R + r) * d.S + s : -1;
+          any |= u.src[b] >= 0;
+        }
+        if (any) f->units.push_back(u);
+      }
+  } else {
+    f->runw = 0;
+    f->run_groups = 0;
+    f->qb = 4;
+    int colidx[kMaxStridePhases];
+    std::fill(colidx, colidx + kMaxStridePhases, -1);
+    for (int s = 0; s < d.S; ++s) {
+      colidx[(long long)s * d.dil_w % sw] = 0;
+      f->max_si = std::max<long long>(f->max_si, (long long)s * d.dil_w / sw);
+    }
+    f->ndw = 0;
+    for (int p = 0; p < sw; ++p)
+      if (colidx[p] == 0) f->col_phase[p] = (int8_t)(colidx[p] = f->ndw++);
+    const int ncb = (d.C + 15) / 16;
+    if ((long long)ncb * f->ndh * f->ndw > 64 || (long long)ncb * d.R * d.S > 1024) return false;
+    f->planes = ncb * f->ndh * f->ndw;
+    for (int cb = 0; cb < ncb; ++cb)
+      for (int r = 0; r < d.R; ++r)
+        for (int s = 0; s < d.S; ++s) {
+          PlaneForm::Unit u;
+          u.plane = (cb * f->ndh + rowidx[r * d.dil_h % sh]) * f->ndw + colidx[s * d.dil_w % sw];
+          u.ri = r * d.dil_h / sh;
+          u.si = s * d.dil_w / sw;
+          for (int b = 0; b < 16; ++b) u.src[b] = cb * 16 + b < d.C ? ((cb * 16 + b) * d.R + r) * d.S + s : -1;
+          f->units.push_back(u);
+        }
+  }
+  // Grid of an image: P + max_ri rows of Q + max_si positions; with stride 1 the zero rows (columns) below
+  // (right of) an image are the ones above (left of) the next image (row).
+  const int cols = g.Q + f->max_si, rows = g.P + f->max_ri;
+  const int share_w = (row_form || sw != 1) ? 0 : std::max(0, std::min(std::min(d.pad_w, f->max_si), cols - (d.W + d.pad_w)));
+  const int share_h = sh != 1 ? 0 : std::max(0, std::min(std::min(d.pad_h, f->max_ri), rows - (d.H + d.pad_h)));
+  f->pitch = cols - share_w;
+  f->rpi = rows - share_h;
+  return true;
+}
+
+// Schedule of one form with per_sm blocks per SM, windows of min_tiles to max_tiles accumulator tiles, dealt one by one
+// (`dealt`) or in segments: window height,
+// column tile and stages with the lowest estimated time (returned; negative if nothing fits).  The estimate adds up,
+// in SM cycles, what a window costs each role (constants measured on the kernel: builder items, 39 cycles and up per
+// MMA, the store path) and takes the slowest role per window, the way of the first window to its MMAs and the stores
+// of the last one.
+double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm, bool dealt, int min_tiles, int max_tiles, PlaneArgs* pl) {
+  const b2c_conv_desc& d = g.d;
+  const int HW = d.H * d.W;
+  const long long total_rows = (long long)d.N * f.rpi;
+  if (total_rows > 0x3FFFFFFF || (total_rows + 64) * f.pitch > 0x3FFFFFFFLL) return -1;
+  const int num_mma = ((int)f.units.size() + 1) / 2;
+  const int n16 = round_up(d.K, 16);
+  const int nruns = d.C * f.ndh, ncb = (d.C + 15) / 16;
+  const double out_bytes = (d.out_mode & B2C_OUT_I32 ? 4.0 : 0.0) + (d.out_mode & B2C_OUT_I8 ? 1.0 : 0.0);
+  const double out_cost = (d.out_mode & B2C_OUT_I32 ? 5.0 : 0.0) + (d.out_mode & B2C_OUT_I8 ? 3.0 : 0.0);
+  const int kb = per_sm == 2 ? 4 : 8, sets = per_sm == 2 ? 1 : 2;  // builder warps; sets of four epilogue warps
+  const int smem_max = per_sm == 2 ? 110 * 1024 : kPlaneSmemMax;
+  double best = -1;
+  int tile_list[6], ntl = 0;
+  // column tiles: all channels if they fit; narrower ones repeat the building of the units, and are tried only while
+  // there are too few tiles for every SM
+  const bool few = total_rows * f.pitch * groups < 2LL * kNumSMs * kTileM;
+  for (int t = few ? 16 : 64; t < n16 && t <= 256; t <<= 1)
+    if (few || n16 > 128) tile_list[ntl++] = t;
+  if (n16 <= 256) tile_list[ntl++] = n16;
+  for (int ti = 0; ti < ntl; ++ti) {
+    const int tile_n = tile_list[ti];
+    const long long w_bytes = (long long)num_mma * 32 * tile_n;
+    if (w_bytes > 150 * 1024) continue;
+    const int cols = (d.K + tile_n - 1) / tile_n;
+    if ((long long)cols * groups > 65535) continue;
+    const int nbuf = std::min(kMaxAcc, 512 / per_sm / tile_n);
+    if (nbuf < (per_sm == 2 ? 2 : 1)) continue;
+    int tmem_cols = 32;
+    while (tmem_cols < nbuf * tile_n) tmem_cols <<= 1;
+    const int places = (int)std::max<long long>(1, (long long)kNumSMs * per_sm / ((long long)cols * groups));
+    for (int th = 1; th <= 128; th += 1 + th / 16) {
+      const int tiles = (th * f.pitch + kTileM - 1) / kTileM;
+      if (th > 1 && (tiles > max_tiles || th > total_rows)) break;
+      if (tiles < min_tiles) continue;
+      const int wr = th + f.max_ri;
+      const long long plane_units = (long long)wr * f.pitch;
+      const long long last_read = (long long)tiles * kTileM + (long long)f.max_ri * f.pitch + f.max_si + 1;
+      const long long win_bytes = ((f.planes - 1) * plane_units + std::max(plane_units, last_read)) * 16;
+      if (win_bytes > 200 * 1024) break;
+      // Segments: single windows; or a block's share of all rows, cut further when the outputs that are being written
+      // at the same time spread over more than about 100 MB; each segment builds its first max_ri rows anew.
+      const int blocks = (int)std::min<long long>(places, (total_rows + th - 1) / th);
+      long long share = (total_rows + blocks - 1) / blocks;
+      if (dealt) share = std::min<long long>(share, th);
+      const double active = (double)blocks * share * f.pitch * d.K * groups * out_bytes;
+      if (active > 100e6 && share > th) {
+        const int parts = (int)std::min<double>((double)((share + th - 1) / th), std::ceil(active / 100e6));
+        share = (total_rows + (long long)blocks * parts - 1) / ((long long)blocks * parts);
+      }
+      const long long segs = (total_rows + share - 1) / share, segs_per_block = (segs + blocks - 1) / blocks;
+      const long long per_block = (share + th - 1) / th * segs_per_block;
+      const double conc = (double)std::min<long long>(per_sm, std::max<long long>(1, ((long long)blocks * cols * groups + kNumSMs - 1) / kNumSMs));
+      const double mma = tiles * (num_mma * std::max(40.0, tile_n / 2.0) + 150.0);
+      const double valid = (double)g.P / f.rpi * g.Q / f.pitch;
+      const double tile_out = 4.0 * tile_n * out_cost * (0.4 + 0.6 * valid);  // store path of the SM
+      const double tile_lat = 600.0 + tile_n * 2.5 * out_cost;                // one set of warps, start to end
+      const double epi = std::max(conc * tiles * tile_out, (double)((tiles + sets - 1) / sets) * tile_lat);
+      // raw chunks of the window's new rows; also of the whole first window when a block has only that one
+      for (int cr = th; cr <= wr; cr += std::max(1, f.max_ri)) {
+        const bool whole_first = cr == wr && (dealt || per_block == 1);
+        if (dealt ? !whole_first : (cr != th && !whole_first)) continue;
+        // raw staging: rows of at most two images per channel, or whole images when a chunk spans more (or they
+        // are small enough not to matter: one copy per image instead of one per channel)
+        const int images = (int)std::min<long long>(d.N, cr <= 1 ? 1 : (cr - 2) / f.rpi + 2);
+        const int raw_rows = std::min(cr * d.stride_h, images * d.H);
+        const long long rows_bytes = (long long)d.C * (round_up(raw_rows * d.W, 16) + 64);
+        const int img_slot = round_up(d.C * HW + 15, 16) + 16;
+        const long long whole_bytes = (long long)images * img_slot;
+        const bool whole = images > 2 || whole_bytes <= rows_bytes + rows_bytes / 4 || whole_bytes <= 8192;
+        const long long raw_data = whole ? whole_bytes : rows_bytes;
+        const double copies = whole ? images : (double)d.C * (1.0 + (double)cr / f.rpi);
+        const long long raw_bytes = (raw_data + 2 * kPlaneMargin + 127) / 128 * 128;
+        const int first_chunks = (int)((std::min<long long>(share, th) + f.max_ri + cr - 1) / cr);
+        const long long row_items = f.runw ? (f.pitch + f.qb - 1) / f.qb : (long long)ncb * f.ndh * ((d.W + 3) / 4);
+        auto build_cycles = [&](long long rows, double* lat) {
+          // SM issue and shared-memory cycles of the items, and the way of one warp through its share of them
+          const double item = f.runw ? 15.0 + nruns * (4.0 + f.qb * 2.0 + 1.5 * f.runw) + f.planes * (6.0 + 6.0 * f.qb) : 150.0;
+          const double one = f.runw ? 250.0 + f.run_groups * (130.0 + 12.0 * f.qb * f.runw) : 900.0;
+          const long long items = rows * row_items;
+          *lat = (double)((items + kb * 32 - 1) / (kb * 32)) * one;
+          return (double)items / 32 * item;
+        };
+        double build_lat, first_lat;
+        const long long new_rows = dealt ? wr : th;
+        const double move = dealt || f.max_ri == 0 ? 0.0 : (double)f.planes * f.max_ri * f.pitch / 32 * 12.0 + 300.0;
+        const double build = build_cycles(new_rows, &build_lat) + move;
+        (void)build_cycles(std::min<long long>(share, th) + f.max_ri, &first_lat);
+        build_lat += move / kb + 300.0;
+        const double copy = 900.0 + (double)raw_data / 24.0 + copies * 60.0;
+        for (int st = 0; st < 3; ++st) {
+          const bool single = per_block == 1;
+          const int ws = st < 2 ? 2 : 1, rs = (single && whole_first) ? 1 : (st < 1 ? 2 : 1);
+          if (single && st < 2) continue;
+          if (ws == 1 && !dealt && !single && th < f.max_ri) continue;  // the overlap rows are moved inside the buffer
+          const long long smem = 128 + ws * win_bytes + rs * raw_bytes + w_bytes + 8LL * round_up(num_mma, 4);
+          if (smem > smem_max) continue;
+          // one buffer between two roles makes them take turns
+          double chain = rs == 1 ? copy + build_lat : std::max(copy, build_lat);
+          if (ws == 1) chain = build_lat + std::max(rs == 1 ? copy : 0.0, mma);
+          double steady = std::max(std::max(conc * build, conc * mma), std::max(epi, chain));
+          if (nbuf == 1) steady = std::max(steady, mma + epi);
+          // (a block's last window is as long as the others unless the rows run out)
+          const double windows = std::max(1.0, dealt ? std::ceil((double)segs / blocks) : (double)total_rows / blocks / th);
+          const double t = 3000 + copy * (rs == 1 ? first_chunks : 1) + first_lat + first_chunks * 150.0 + mma / tiles + epi + w_bytes / 40.0 * conc +
+                           (windows - 1) * steady + (dealt ? 0.0 : (double)(segs_per_block - 1) * f.max_ri / th * conc * build);
+          if (best >= 0 && t >= best * 0.999) continue;
+          best = t;
+          pl->tile_n = tile_n;
+          pl->cols = cols;
+          pl->tmem_cols = tmem_cols;
+          pl->nbuf = nbuf;
+          pl->per_sm = per_sm;
+          pl->th = th;
+          pl->cr = cr;
+          pl->tiles = tiles;
+          pl->seg_rows = (int)share;
+          pl->segs = (int)segs;
+          pl->blocks = std::min<int>(blocks, pl->segs);
+          pl->plane_bytes = (int)plane_units * 16;
+          pl->win_bytes = (int)win_bytes;
+          pl->whole_images = whole ? 1 : 0;
+          pl->img_slot = img_slot;
+          pl->c_pitch = round_up(raw_rows * d.W, 16) + 64;
+          pl->raw_bytes = (int)raw_bytes;
+          pl->win_stages = ws;
+          pl->raw_stages = rs;
+          pl->w_bytes = (int)w_bytes;
+          pl->smem = (int)smem;
+        }
+      }
+    }
+  }
+  return best;
+}
+
+// Form and schedules of the plane kernel, the lowest estimate first: the best one for each number of blocks per SM,
+// way of dealing windows and range of window heights (their order depends on how the store path, the builders and DRAM share the time, which
+// the estimate knows to 10 to 25 %; the timed selection tries them all).
+struct PlaneChoice {
+  double t;
+  PlaneArgs pl;
+};
+bool plane_choices(const Geom& g, int groups, PlaneForm* form, std::vector<PlaneChoice>* out) {
+  const b2c_conv_desc& d = g.d;
+  out->clear();
+  if (d.in_layout != B2C_LAYOUT_NCHW || d.pad_h > 32 || d.pad_w > 32 || d.K > 1024) return false;
+  // (above 96 channels the weights of a column tile and the units of a window no longer fit beside each other: 30
+  // images of 128 x 28 x 28 -> 128, 3x3, 19.7 us against 11.3 by the channel pack)
+  if (d.C > 96) return false;
+  // Images of a few pixels would fill a window with the overhang of many images; the channel-pack maps do those.
+  if ((d.W % 16) != 0 && g.PQ < 43) return false;
+  if ((long long)d.C * d.H * d.W > (1 << 26) || d.W > 8192) return false;
+  double best = -1;
+  for (int f = 0; f < 2; ++f) {
+    PlaneForm cand;
+    if (!plane_form(g, f == 1, &cand)) continue;
+    std::vector<PlaneChoice> list;
+    // blocks per SM, dealt, fewest and most tiles of a window (the last two: windows on the other side of what the
+    // estimate takes for the best height)
+    static const int kStyles[6][4] = {{1, 1, 1, 16}, {2, 1, 1, 16}, {1, 0, 1, 16}, {2, 0, 1, 16}, {1, 1, 1, 5}, {2, 1, 6, 16}};
+    for (const int* style : kStyles) {
+      PlaneChoice c;
+      std::memset(&c.pl, 0, sizeof(c.pl));
+      c.t = plane_schedule(g, groups, cand, style[0], style[1] != 0, style[2], style[3], &c.pl);
+      if (c.t < 0) continue;
+      bool same = false;
+      for (const PlaneChoice& o : list)
+        same |= o.pl.per_sm == c.pl.per_sm && o.pl.th == c.pl.th && o.pl.seg_rows == c.pl.seg_rows && o.pl.tile_n == c.pl.tile_n;
+      if (!same) list.push_back(c);
+    }
+    if (list.empty()) continue;
+    std::stable_sort(list.begin(), list.end(), [](const PlaneChoice& a, const PlaneChoice& b) { return a.t < b.t; });
+    if (best >= 0 && list[0].t >= best) continue;
+    best = list[0].t;
+    *form = cand;
+    *out = list;
+  }
+  return !out->empty();
+}
+
+}  // namespace
+
+bool plane_plan(const Geom& g, int groups, int tile_n, int nth, PlaneArgs* pl, std::vector<uint64_t>* table, std::vector<int32_t>* wsrc) {
+  const b2c_conv_desc& d = g.d;
+  std::memset(pl, 0, sizeof(*pl));
+  PlaneForm f;
+  std::vector<PlaneChoice> list;
+  if (!plane_choices(g, groups, &f, &list)) return false;
+  bool found = false;
+  for (const PlaneChoice& c : list)
+    if ((tile_n == 0 || c.pl.tile_n == tile_n) && nth-- == 0) {
+      *pl = c.pl;
+      found = true;
+      break;
+    }
+  if (!found) return false;
+  const int HW = d.H * d.W;
+  pl->runw = f.runw;
+  pl->sh = d.stride_h;
+  pl->sw = d.stride_w;
+  pl->ndh = f.ndh;
+  pl->ndw = f.ndw;
+  pl->max_dh = f.max_dh;
+  std::memcpy(pl->row_phase, f.row_phase, sizeof(pl->row_phase));
+  std::memcpy(pl->col_phase, f.col_phase, sizeof(pl->col_phase));
+  pl->planes = f.planes;
+  pl->pitch = f.pitch;
+  pl->rpi = f.rpi;
+  pl->total_rows = d.N * f.rpi;
+  pl->max_ri = f.max_ri;
+  pl->num_mma = ((int)f.units.size() + 1) / 2;
+  pl->gpr = f.runw ? (f.pitch + f.qb - 1) / f.qb : (d.W + 3) / 4;
+  pl->run_groups = f.run_groups;
+  pl->zero_fill = f.runw == 0 ? 1 : 0;
+  // words: rows start on one when W does and every channel starts on one (segments: 16 bytes, the alignment of
+  // all channels is then the same)
+  pl->aligned = (d.W % 4 == 0 && (pl->whole_images || HW % 16 == 0)) ? 1 : 0;
+  // flat groups: channels start on words (of memory, hence of the staged copy), and a group crosses one row end at most
+  if (f.runw == 0 && d.stride_h == 1 && d.stride_w == 1 && HW % 4 == 0 && d.W >= 4) pl->aligned = 2;
+  pl->div_rpi = make_fastdiv((uint32_t)f.rpi);
+  pl->div_pitch = make_fastdiv((uint32_t)f.pitch);
+  pl->div_gpr = make_fastdiv((uint32_t)pl->gpr);
+  pl->div_nu = make_fastdiv((uint32_t)std::max(1, f.planes / f.ndw));
+  pl->div_w = make_fastdiv((uint32_t)d.W);
+  pl->div_hw4 = make_fastdiv((uint32_t)std::max(1, HW / 4));
+  pl->div_overlap = make_fastdiv((uint32_t)std::max(1, f.max_ri * f.pitch));
+  pl->div_sw = make_fastdiv((uint32_t)d.stride_w);
+  if (table && wsrc) {
+    // units in address order, two per MMA; a last odd one is paired with its neighbour under zero weights
+    std::vector<std::pair<int, int>> order;
+    for (size_t i = 0; i < f.units.size(); ++i)
+      order.push_back({f.units[i].plane * (pl->plane_bytes / 16) + f.units[i].ri * f.pitch + f.units[i].si, (int)i});
+    std::sort(order.begin(), order.end());
+    table->clear();
+    wsrc->assign((size_t)pl->num_mma * 32, -1);
+    for (int m = 0; m < pl->num_mma; ++m) {
+      const bool two = 2 * m + 1 < (int)order.size();
+      const int a0 = order[2 * m].first, a1 = two ? order[2 * m + 1].first : a0 + 1;
+      table->push_back((uint64_t)a0 | ((uint64_t)(a1 - a0) << 16));
+      for (int u = 0; u < (two ? 2 : 1); ++u)
+        for (int b = 0; b < 16; ++b) (*wsrc)[(size_t)(2 * m + u) * 16 + b] = f.units[order[2 * m + u].second].src[b];
+    }
+    // (the issuing warp reads the table four entries at a time)
+    while (table->size() % 4 != 0) table->push_back(table->back());
+  }
+  return true;
+}
+
+// The plane kernel builds every input row once per window and needs windows of several tiles to pay for the rows the
+// taps reach below; the window kernel's tiles are independent of each other and spread a small problem over more
+// blocks.  7x7 stride 2 of 3 x 224 x 224, 98 tiles an image: 4 images 6.9 us (window) against 9.5, 16 images 14.3
+// against 15.3, 100 images 72 against 65.
+bool plane_wanted(const Geom& g) {
+  WindowTile wt;
+  return !(window_tile_geom(g, &wt) && wt.mtot <= (long long)kPlaneMinTiles * kTileM);
+}
+
 static void add(std::vector<b2c_embedding>* out, const Geom& g, int variant, int tile_n, int split_k,
-                bool swap = false, int tile_m = kTileM) {
+                bool swap = false, int tile_m = kTileM, long long plane_rows = 0, int plane_k = 0) {
   const b2c_conv_desc& d = g.d;
   b2c_embedding e;
   std::memset(&e, 0, sizeof(e));
@@ -410,7 +781,13 @@ static void add(std::vector<b2c_embedding>* out, const Geom& g, int variant, int
     int K_pad = variant_k_pad(g, variant);
     k_issued = K_pad;
     WindowTile wt;
-    if (variant == B2C_VARIANT_IM2COL_WINDOW && window_tile_geom(g, &wt)) M_pad = wt.mtot;  // whole two-dimensional tiles
+    if (plane_rows > 0) {
+      M_pad = (plane_rows + kTileM - 1) / kTileM * kTileM;  // plane kernel: grid positions, the taps' overhang among them
+      K_pad = plane_k;
+      k_issued = K_pad;
+    } else if (variant == B2C_VARIANT_IM2COL_WINDOW && window_tile_geom(g, &wt)) {
+      M_pad = wt.mtot;  // whole two-dimensional tiles
+    }
     if (variant == B2C_VARIANT_IM2COL_EXPLICIT)
       moved = g.x_elems + 2 * g.Mg * K_pad + (long long)d.K * K_pad + g.y_elems;
     else if (variant == B2C_VARIANT_IM2COL_STAGED)
@@ -446,9 +823,18 @@ void enumerate_embeddings(const Geom& g, std::vector<b2c_embedding>* out) {
     WindowGeom wg;
     if (variant == B2C_VARIANT_IM2COL_STAGED && !staged_window(g, &wg)) continue;
     if (variant == B2C_VARIANT_IM2COL_WINDOW) {
-      // one schedule: all output channels in one column tile (the weights are resident), no split
+      // window kernel: one schedule, all output channels in one column tile (the weights are resident), no split
       WindowTile wt;
-      if (window_tile_geom(g, &wt)) add(out, g, variant, wt.tile_n, 1);
+      PlaneForm form;
+      std::vector<PlaneChoice> plane;
+      if (plane_wanted(g) && plane_choices(g, 1, &form, &plane)) {
+        // one entry per schedule of the plane kernel
+        for (const PlaneChoice& c : plane)
+          add(out, g, variant, c.pl.tile_n, 1, false, kTileM, (long long)g.d.N * form.rpi * form.pitch,
+              ((int)form.units.size() + 1) / 2 * kMmaK);
+      } else if (window_tile_geom(g, &wt)) {
+        add(out, g, variant, wt.tile_n, 1);
+      }
       continue;
     }
     int num_kb;

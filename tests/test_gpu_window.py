@@ -34,3 +34,49 @@ def test_bias_vector_and_scalar_loads(lib, K, groups):
         assert plan.device_status() == b2c.OK
         assert np.array_equal(y32.cpu().numpy(), want[0]) and np.array_equal(y8.cpu().numpy(), want[1])
         plan.destroy()
+
+
+# ---- window unroll over planes of units: forms, staging and window dealing at the edges of their ranges -----------
+# (batches above the size from which this kernel runs, or shapes the window kernel does not take; every listed schedule)
+@pytest.mark.parametrize("case", [
+    # N, C, H, W, K, R, S, stride, pad, dil, shift
+    (3, 1, 40, 61, 32, 20, 5, 2, 0, 1, 9),             # one channel, odd width: runs of two words, 20 filter rows
+    (5, 3, 27, 35, 64, 7, 7, 2, 3, 1, 8),              # 7x7 stem on an odd image: six runs, columns outside on both sides
+    (2, 1, 12, 75, 17, 3, 21, 2, 4, 1, 7),             # runs of six words; 17 channels
+    (2, 2, 15, 33, 40, 2, 12, 1, 3, 1, 6),             # runs of four words, stride 1
+    (3, 5, 14, 22, 24, 3, 3, (1, 3), 1, (2, 1), 6),    # stride 3: one column per builder item; vertical dilation
+    (4, 17, 13, 15, 20, 3, 3, 1, 1, 1, 8),             # channel form, H * W odd: unaligned words
+    (2, 40, 18, 10, 96, 3, 3, 1, 1, 1, 9),             # channel form, flat groups across row ends, ragged channel block
+    (3, 24, 17, 12, 33, 3, 3, 2, 1, 1, 8),             # channel form, stride 2: four phase planes
+    (2, 12, 16, 20, 300, 1, 1, 1, 0, 1, 6),            # 1x1; three column tiles
+    (2, 9, 20, 18, 16, 3, 3, 1, (4, 0), 4, 7),         # dilation 4, padding on one axis
+    (1, 8, 9, 50, 16, 2, 2, 1, 32, 1, 5),              # padding as wide as the kernel takes
+    (60, 8, 7, 7, 8, 3, 3, 1, 1, 1, 7),                # small images: a window spans many (7 rows each)
+    (300, 18, 14, 14, 16, 3, 3, 1, 1, 1, 8),           # whole images staged (3528 bytes: two alignments in turn)
+    (30, 3, 225, 223, 16, 5, 5, 2, 2, 1, 7),           # enough rows for every block to walk windows in every schedule
+    (100, 48, 30, 30, 64, 3, 3, 1, 1, 1, 9),           # the same, channel form with moved overlap rows
+])
+@pytest.mark.parametrize("out_layout,out_mode", [(0, 3), (1, 2)])
+def test_plane_kernel(lib, case, out_layout, out_mode):
+    N, C, H, W, K, R, S, stride, pad, dil, shift = case
+    x = int8_uniform((N, C, H, W), 1021)
+    w = int8_uniform((K, C, R, S), 1022)
+    ref = oracle.conv2d_int8(x, w, stride, pad, dil, shift)
+    d = lib.make_desc(N, C, H, W, K, R, S, stride, pad, dil, shift, 0, out_layout, out_mode)
+    ids = [e.id for e in lib.enumerate_embeddings(d) if e.variant == b2c.VARIANT_IM2COL_WINDOW]
+    assert ids
+    for i in ids:
+        check_against_oracle(x, w, stride, pad, dil, shift, out_mode, i, ref=ref, out_layout=out_layout)
+
+
+def test_plane_kernel_reads_the_last_incomplete_16_bytes(lib):
+    """The tensor ends inside a 16-byte unit: its last bytes are copied one by one, nothing behind them is read."""
+    N, C, H, W, K = 3, 3, 29, 31, 16                     # 8091 bytes, 11 past the last whole unit
+    x = int8_uniform((N, C, H, W), 1031)
+    w = int8_uniform((K, C, 3, 3), 1032)
+    ref = oracle.conv2d_int8(x, w, 1, 1, 1, 5)
+    d = lib.make_desc(N, C, H, W, K, 3, 3, 1, 1, 1, 5, out_mode=3)
+    assert x.size % 16 == 11
+    for e in lib.enumerate_embeddings(d):
+        if e.variant == b2c.VARIANT_IM2COL_WINDOW:
+            check_against_oracle(x, w, 1, 1, 1, 5, 3, e.id, ref=ref)
