@@ -23,7 +23,8 @@ struct b2c_plan {
   int32_t* table32 = nullptr;    // device, plan-owned (offsets into the staged window)
   WindowGeom win = {0, 0, 0, 0, 0};
   PlaneArgs plane = {};          // plane kernel: geometry and device tables (plane.num_mma > 0: this plan runs it)
-  uint64_t* mma_table = nullptr; // device, plan-owned: A descriptors of the plane kernel
+  uint64_t* mma_table = nullptr; // device, plan-owned: A descriptors of the plane kernel, then its weight indices
+  const int32_t* plane_wsrc = nullptr;
   TmaView view = {};             // geometry handed to the im2col-mode-TMA kernel (TMA-view variants)
   int32_t* wtable = nullptr;     // device, plan-owned: packed weight column -> index into one filter, -1 = zero
   int table_len = 0;
@@ -448,8 +449,9 @@ int create_plan_for(const Geom& g, const b2c_embedding& emb, int nth, b2c_plan**
   if (cudaMemset(p->status, 0, kStatusWords * sizeof(int)) != cudaSuccess) return fail(B2C_E_CUDA);
   std::vector<uint64_t> mma;
   std::vector<int32_t> wsrc;
-  const bool plane = emb.variant == B2C_VARIANT_IM2COL_WINDOW && plane_wanted(g) &&
+  const bool plane = emb.variant == B2C_VARIANT_IM2COL_WINDOW && (group_count > 1 || plane_wanted(g)) &&
                      plane_plan(g, group_count, emb.tile_n, nth, &p->plane, &mma, &wsrc);
+  if (group_count > 1 && emb.variant == B2C_VARIANT_IM2COL_WINDOW && !plane) return fail(B2C_E_UNSUPPORTED);
   if (is_tma_view_variant(emb.variant)) {
     if (!tma_view_for(g, emb.variant, &p->view)) return fail(B2C_E_UNSUPPORTED);
     const TmaView& v = p->view;
@@ -509,12 +511,14 @@ int create_plan_for(const Geom& g, const b2c_embedding& emb, int nth, b2c_plan**
     }
   } else if (plane) {
     p->w_packed_bytes = (size_t)group_count * p->plane.cols * p->plane.w_bytes;
-    if (cudaMalloc(&p->mma_table, mma.size() * sizeof(uint64_t)) != cudaSuccess) return fail(B2C_E_CUDA);
-    if (cudaMemcpy(p->mma_table, mma.data(), mma.size() * sizeof(uint64_t), cudaMemcpyHostToDevice) != cudaSuccess)
+    // both tables in one buffer: the A descriptors, then the weight indices
+    std::vector<uint64_t> tables = mma;
+    tables.resize(mma.size() + (wsrc.size() + 1) / 2);
+    std::memcpy(tables.data() + mma.size(), wsrc.data(), wsrc.size() * sizeof(int32_t));
+    if (cudaMalloc(&p->mma_table, tables.size() * sizeof(uint64_t)) != cudaSuccess) return fail(B2C_E_CUDA);
+    if (cudaMemcpy(p->mma_table, tables.data(), tables.size() * sizeof(uint64_t), cudaMemcpyHostToDevice) != cudaSuccess)
       return fail(B2C_E_CUDA);
-    if (cudaMalloc(&p->wtable, wsrc.size() * sizeof(int32_t)) != cudaSuccess) return fail(B2C_E_CUDA);
-    if (cudaMemcpy(p->wtable, wsrc.data(), wsrc.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess)
-      return fail(B2C_E_CUDA);
+    p->plane_wsrc = reinterpret_cast<const int32_t*>(p->mma_table + mma.size());
   } else {
     int K_pad = variant_k_pad(g, emb.variant);
     p->w_packed_bytes = (size_t)d.K * K_pad * group_count;  // grouped: the filters of all groups, one block of K rows each
@@ -835,6 +839,45 @@ int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_
   return create_plan_for(g, all[best], schedule_of(all, best), out);
 }
 
+// Group plan that runs all groups in one launch, `merge` consecutive ones as one group sg with embedding emb.
+static int create_grouped_plan(const b2c_conv_desc* desc, int groups, int merge, const Geom& sg, const b2c_embedding& emb, int nth,
+                               b2c_plan** out) {
+  b2c_plan* p = new (std::nothrow) b2c_plan();
+  if (!p) return B2C_E_INVALID_ARG;
+  p->g = sg;
+  p->g.d.C = desc->C;  // the group plan describes the whole convolution
+  p->g.d.K = desc->K;
+  p->emb = emb;
+  p->groups = groups;
+  p->merge = merge;
+  cudaGetDevice(&p->device);
+  if (cudaMalloc(&p->status, kStatusWords * sizeof(int)) != cudaSuccess ||
+      cudaMemset(p->status, 0, kStatusWords * sizeof(int)) != cudaSuccess) {
+    set_last_cuda_error((int)cudaGetLastError());
+    b2c_plan_destroy(p);
+    return B2C_E_CUDA;
+  }
+  // one sub-plan runs all groups in one launch (the group is a grid axis of the kernel)
+  b2c_plan* sub = nullptr;
+  const int rc = create_plan_for(sg, emb, nth, &sub, groups / merge);
+  if (rc != B2C_OK) {
+    b2c_plan_destroy(p);
+    return rc;
+  }
+  if (merge > 1 &&
+      cudaMalloc(&p->w_expanded, (size_t)desc->K * sg.d.C * desc->R * desc->S + 256) != cudaSuccess) {
+    set_last_cuda_error((int)cudaGetLastError());
+    b2c_plan_destroy(sub);
+    b2c_plan_destroy(p);
+    return B2C_E_CUDA;
+  }
+  sub->x_stride_n_whole = (long long)desc->C * desc->H * desc->W;
+  sub->y_stride_n_whole = (long long)desc->K * sg.PQ;
+  p->subs.push_back(sub);
+  *out = p;
+  return B2C_OK;
+}
+
 int b2c_plan_create_grouped(const b2c_conv_desc* desc, int32_t groups, b2c_plan** out) {
   if (!desc || !out || groups < 1) return B2C_E_INVALID_ARG;
   *out = nullptr;
@@ -859,7 +902,6 @@ int b2c_plan_create_grouped(const b2c_conv_desc* desc, int32_t groups, b2c_plan*
   Geom sg;
   int rc = resolve_geom(&sd, &sg);
   if (rc != B2C_OK) return rc;
-  const int run_groups = groups / merge;
   // Embedding of every group: the lowest-overhead unsplit stencil unroll formed inside the kernel
   // (staged window where it fits, else the gather); both read their channel slice of x in place.
   std::vector<b2c_embedding> all;
@@ -880,40 +922,7 @@ int b2c_plan_create_grouped(const b2c_conv_desc* desc, int32_t groups, b2c_plan*
         (pick < 0 || better(all[i], all[pick])))
       pick = (int)i;
   if (pick < 0) return B2C_E_UNSUPPORTED;
-  b2c_plan* p = new (std::nothrow) b2c_plan();
-  if (!p) return B2C_E_INVALID_ARG;
-  p->g = sg;
-  p->g.d.C = desc->C;  // the group plan describes the whole convolution
-  p->g.d.K = desc->K;
-  p->emb = all[pick];
-  p->groups = groups;
-  p->merge = merge;
-  cudaGetDevice(&p->device);
-  if (cudaMalloc(&p->status, kStatusWords * sizeof(int)) != cudaSuccess ||
-      cudaMemset(p->status, 0, kStatusWords * sizeof(int)) != cudaSuccess) {
-    set_last_cuda_error((int)cudaGetLastError());
-    b2c_plan_destroy(p);
-    return B2C_E_CUDA;
-  }
-  // one sub-plan runs all groups in one launch (the group is a grid axis of the kernel)
-  b2c_plan* sub = nullptr;
-  rc = create_plan_for(sg, all[pick], 0, &sub, run_groups);
-  if (rc != B2C_OK) {
-    b2c_plan_destroy(p);
-    return rc;
-  }
-  if (merge > 1 &&
-      cudaMalloc(&p->w_expanded, (size_t)desc->K * sd.C * desc->R * desc->S + 256) != cudaSuccess) {
-    set_last_cuda_error((int)cudaGetLastError());
-    b2c_plan_destroy(sub);
-    b2c_plan_destroy(p);
-    return B2C_E_CUDA;
-  }
-  sub->x_stride_n_whole = (long long)desc->C * desc->H * desc->W;
-  sub->y_stride_n_whole = (long long)desc->K * sg.PQ;
-  p->subs.push_back(sub);
-  *out = p;
-  return B2C_OK;
+  return create_grouped_plan(desc, groups, merge, sg, all[pick], 0, out);
 }
 
 int b2c_plan_create_grouped_timed(const b2c_conv_desc* desc, int32_t groups, void* cuda_stream, b2c_plan** out) {
@@ -922,45 +931,96 @@ int b2c_plan_create_grouped_timed(const b2c_conv_desc* desc, int32_t groups, voi
   b2c_plan* inplace = nullptr;
   int rc = b2c_plan_create_grouped(desc, groups, &inplace);
   if (rc != B2C_OK) return rc;
-  // The other form: every group merged, i.e. the dense convolution with block-diagonal filters through the
-  // timed selection of dense plans.  It pays `groups` times the MACs and has the rewrite and the scratch
-  // of its embedding; on this device it still wins for a few hundred groups.
-  const long long dense_w = (long long)desc->K * desc->C * desc->R * desc->S;
-  if (groups < 2 || dense_w > (16ll << 20)) {
-    *out = inplace;
-    return B2C_OK;
-  }
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  b2c_plan* dense = nullptr;
-  if (b2c_plan_create(desc, B2C_POLICY_AUTO_TIMED, cuda_stream, &dense) != B2C_OK || dense->emb.device_us <= 0) {
-    b2c_plan_destroy(dense);
+  Geom g;
+  rc = resolve_geom(desc, &g);
+  if (rc != B2C_OK || groups < 2) {
     *out = inplace;
     return B2C_OK;
   }
-  // time the in-place form on scratch tensors, as the dense candidates were
-  const Geom& g = dense->g;
+  // scratch tensors for the timings (the grouped filter tensor is no larger than K x C / groups x R x S)
   int8_t *x = nullptr, *w = nullptr;
   LaneBuffers lane = {};
-  float us = -1;
-  bool ok = cudaMalloc(&x, g.x_elems + 256) == cudaSuccess && cudaMalloc(&w, g.w_elems + 256) == cudaSuccess &&
+  const size_t w_bytes = (size_t)desc->K * (desc->C / groups) * desc->R * desc->S;
+  bool ok = cudaMalloc(&x, g.x_elems + 256) == cudaSuccess && cudaMalloc(&w, w_bytes + 256) == cudaSuccess &&
             cudaMalloc(&lane.y8, g.y_elems + 256) == cudaSuccess && cudaMalloc(&lane.y32, g.y_elems * 4 + 256) == cudaSuccess &&
             cudaMalloc(&lane.ws, 1024) == cudaSuccess;
+  float us = -1;
+  auto timed = [&](b2c_plan* q, float* t) {
+    const bool good = b2c_plan_set_weights(q, w, st) == B2C_OK && cudaStreamSynchronize(st) == cudaSuccess &&
+                      time_plan(q, x, &lane, 1, t) == B2C_OK;
+    q->weights_set = false;  // the caller's filters are still to come
+    if (!good) (void)cudaGetLastError();
+    return good;
+  };
   if (ok) {
     cudaMemsetAsync(x, 1, g.x_elems, st);
-    cudaMemsetAsync(w, 1, g.w_elems, st);  // (the grouped filter tensor is smaller than the dense one)
-    ok = b2c_plan_set_weights(inplace, w, st) == B2C_OK && cudaStreamSynchronize(st) == cudaSuccess &&
-         time_plan(inplace, x, &lane, 1, &us) == B2C_OK;
-    inplace->weights_set = false;  // the caller's filters are still to come
+    cudaMemsetAsync(w, 1, w_bytes, st);
+    if (!timed(inplace, &us)) us = -1;
+    inplace->emb.device_us = us;
+    // The plane kernel on merged groups of 16 to 64 channels: its schedules for each such merge factor.  (Depth-wise,
+    // 128 x 256 x 28 x 28, 3x3: 33 us by 32 channels; the staged window on merged groups takes 165, the dense form 61.)
+    const int cg = desc->C / groups, kg = desc->K / groups;
+    // (m == groups is the dense form below; fewer than 16 channels leave the 16-byte units part empty)
+    for (int m = 1; m < groups && us > 0; ++m) {
+      if (groups % m != 0 || m * cg < 16 || m * cg > 64 || m * kg > 128) continue;
+      b2c_conv_desc sd = *desc;
+      sd.C = m * cg;
+      sd.K = m * kg;
+      Geom sg;
+      if (resolve_geom(&sd, &sg) != B2C_OK) continue;
+      for (int nth = 0; nth < 6; ++nth) {
+        PlaneArgs pl;
+        if (!plane_plan(sg, groups / m, 0, nth, &pl)) break;
+        b2c_embedding e;
+        std::memset(&e, 0, sizeof(e));
+        e.map_m = B2C_AXIS_NPQ;
+        e.map_n = B2C_AXIS_K;
+        e.map_k = B2C_AXIS_CRS;
+        e.variant = B2C_VARIANT_IM2COL_WINDOW;
+        e.tile_m = kTileM;
+        e.tile_n = pl.tile_n;
+        e.split_k = 1;
+        e.o_mac = (int64_t)pl.total_rows * pl.pitch * pl.cols * pl.tile_n * pl.num_mma * kMmaK * (groups / m) - g.Mg * desc->K * cg * desc->R * desc->S;
+        e.o_data = (int64_t)(groups / m) * pl.cols * pl.w_bytes - (int64_t)w_bytes;
+        e.device_us = -1.0f;
+        int same = 0;  // schedules with this column tile before this one
+        for (int i = 0; i < nth; ++i) {
+          PlaneArgs before;
+          same += plane_plan(sg, groups / m, 0, i, &before) && before.tile_n == pl.tile_n ? 1 : 0;
+        }
+        b2c_plan* q = nullptr;
+        float t = -1;
+        if (create_grouped_plan(desc, groups, m, sg, e, same, &q) == B2C_OK && timed(q, &t) && t < us) {
+          b2c_plan_destroy(inplace);
+          inplace = q;
+          us = t;
+          inplace->emb.device_us = t;
+        } else {
+          b2c_plan_destroy(q);
+          (void)cudaGetLastError();
+        }
+      }
+    }
+  } else {
+    (void)cudaGetLastError();
   }
   cudaFree(x);
   cudaFree(w);
   cudaFree(lane.y8);
   cudaFree(lane.y32);
   cudaFree(lane.ws);
-  if (!ok) (void)cudaGetLastError();
-  if (!ok || us <= dense->emb.device_us) {  // (an in-place form that could not be timed is still the safe choice)
+  // The other form: every group merged, i.e. the dense convolution with block-diagonal filters through the
+  // timed selection of dense plans.  It pays `groups` times the MACs and has the rewrite and the scratch
+  // of its embedding; it is built while those MACs, at 0.62 of the intrinsic's issue rate (the most a path from
+  // NCHW input reaches), would not take longer than the best form in place.
+  const long long dense_w = (long long)desc->K * desc->C * desc->R * desc->S;
+  const double dense_us = 2.0 * (double)g.Mg * (double)dense_w / (0.62 * 4.5e9);  // 4.5 POPS
+  b2c_plan* dense = nullptr;
+  if (us <= 0 || dense_w > (16ll << 20) || dense_us >= us ||  // (a form in place that could not be timed is still the safe choice)
+      b2c_plan_create(desc, B2C_POLICY_AUTO_TIMED, cuda_stream, &dense) != B2C_OK || dense->emb.device_us <= 0 ||
+      us <= dense->emb.device_us) {
     b2c_plan_destroy(dense);
-    inplace->emb.device_us = us;
     *out = inplace;
     return B2C_OK;
   }
@@ -1035,7 +1095,7 @@ static int set_weights_one(b2c_plan* p, const int8_t* w, cudaStream_t st) {
     CUDA_TRY(launch_pack_weights_cp(w, p->w_packed, d.K, d.C, d.R, d.S, p->C_pad, st));
   else if (p->amode == A_PLANE)
     CUDA_TRY(launch_pack_weights_plane(w, p->w_packed, p->group_count, d.K, p->g.Kg, p->plane.tile_n, p->plane.cols,
-                                       p->plane.num_mma, p->wtable, st));
+                                       p->plane.num_mma, p->plane_wsrc, st));
   else if (is_tma_view_variant(p->emb.variant))
     CUDA_TRY(launch_pack_weights_table(w, p->w_packed, d.K, p->g.Kg, p->view.R * p->view.S * p->view.C, p->wtable, st));
   else

@@ -631,6 +631,20 @@ struct PlaneChoice {
 };
 bool plane_choices(const Geom& g, int groups, PlaneForm* form, std::vector<PlaneChoice>* out) {
   const b2c_conv_desc& d = g.d;
+  // (enumerating a problem and creating a plan for one of its embeddings search the same descriptor one after the
+  // other: the last search of this thread is kept, by the descriptor's values)
+  struct Last {
+    b2c_conv_desc d;
+    int groups = 0;
+    PlaneForm form;
+    std::vector<PlaneChoice> list;
+  };
+  static thread_local Last last;
+  if (last.groups == groups && std::memcmp(&last.d, &d, sizeof(d)) == 0) {
+    *form = last.form;
+    *out = last.list;
+    return !out->empty();
+  }
   out->clear();
   if (d.in_layout != B2C_LAYOUT_NCHW || d.pad_h > 32 || d.pad_w > 32 || d.K > 1024) return false;
   // (above 96 channels the weights of a column tile and the units of a window no longer fit beside each other: 30
@@ -664,6 +678,10 @@ bool plane_choices(const Geom& g, int groups, PlaneForm* form, std::vector<Plane
     *form = cand;
     *out = list;
   }
+  last.d = d;
+  last.groups = groups;
+  last.form = *form;
+  last.list = *out;
   return !out->empty();
 }
 

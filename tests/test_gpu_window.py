@@ -80,3 +80,31 @@ def test_plane_kernel_reads_the_last_incomplete_16_bytes(lib):
     for e in lib.enumerate_embeddings(d):
         if e.variant == b2c.VARIANT_IM2COL_WINDOW:
             check_against_oracle(x, w, 1, 1, 1, 5, 3, e.id, ref=ref)
+
+
+@pytest.mark.parametrize("case", [
+    # N, C, H, W, K, groups, R, shift, out_mode
+    (40, 64, 28, 28, 64, 64, 3, 5, 3),       # depth-wise: groups merged 16 at a time and more
+    (30, 96, 17, 23, 96, 96, 3, 5, 1),       # odd image: every group's channel slice at another alignment
+    (16, 128, 20, 20, 256, 8, 3, 7, 2),      # 16 -> 32 channels a group, nothing to merge
+])
+def test_grouped_plane_kernel(lib, case):
+    N, C, H, W, K, groups, R, shift, out_mode = case
+    x = int8_uniform((N, C, H, W), 1041)
+    w = int8_uniform((K, C // groups, R, R), 1042)
+    bias = int8_uniform((K,), 1043).astype(np.int32) * 97
+    want = oracle.conv2d_int8(x, w, 1, 1, 1, shift, bias=bias, relu=True, groups=groups)
+    d = lib.make_desc(N, C, H, W, K, R, R, 1, 1, 1, shift, out_mode=out_mode)
+    plan = lib.Plan(d, b2c.POLICY_AUTO_TIMED, groups=groups)
+    assert plan.info().device_us > 0
+    plan.set_weights(to_dev(w))
+    plan.set_activation(to_dev(bias), True)
+    y32 = torch.full((N, K, H, W), -7777777, dtype=torch.int32, device="cuda") if out_mode & 1 else None
+    y8 = torch.full((N, K, H, W), 77, dtype=torch.int8, device="cuda") if out_mode & 2 else None
+    ws = torch.zeros(max(16, plan.workspace_bytes()), dtype=torch.uint8, device="cuda")
+    plan.run(to_dev(x), y32, y8, ws)
+    torch.cuda.synchronize()
+    assert plan.device_status() == b2c.OK
+    assert y32 is None or np.array_equal(y32.cpu().numpy(), want[0])
+    assert y8 is None or np.array_equal(y8.cpu().numpy(), want[1])
+    plan.destroy()
