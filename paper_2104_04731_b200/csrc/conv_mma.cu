@@ -42,6 +42,13 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
   // (PERSIST is a template parameter so that the one-tile-per-block instantiation carries none of
   // the loop, buffer-index and hand-back overhead.)
   constexpr bool persistent = PERSIST != 0;
+  // Which of the kernel's cases an instantiation can meet.  What it cannot meet is not compiled into it: the swapped
+  // map's stores alone, unused in the shift execution, took its 64-column NHWC tiles from 10.4 to 12.5 us.
+  constexpr bool kTmaFed = AMODE == A_TILED || AMODE == A_IM2COL_TMA;
+  const bool swap_map = kTmaFed && !persistent && args.swap != 0;
+  const bool cluster_split = !persistent && AMODE != A_SHIFT && args.cluster_split != 0;
+  constexpr bool kSplit = !persistent && AMODE != A_SHIFT;
+  const int remap = AMODE == A_SHIFT ? 2 + (args.remap == 3 ? 1 : 0) : (AMODE == A_IM2COL_TMA && args.remap == 1 ? 1 : 0);
   const int tile_first = persistent ? (int)blockIdx.x : 0;
   const int tile_step = persistent ? (int)gridDim.x : 1;
   const int tile_end = persistent ? args.num_tiles : 1;
@@ -53,7 +60,7 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
     const int mt_ = (int)args.div_tiles_n.div((uint32_t)(t));                       \
     m0 = mt_ * kTileM;                                                              \
     n0 = ((t) - mt_ * args.tiles_n) * args.tile_n;                                  \
-  } else if (args.swap) {                                                           \
+  } else if (swap_map) {                                                            \
     m0 = (int)blockIdx.y * kTileM;     /* accumulator rows: output channels */      \
     n0 = (int)blockIdx.x * args.tile_n; /* accumulator columns: fused pixels */     \
   } else {                                                                          \
@@ -172,7 +179,7 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
         const uint32_t full = smem_u32(&ctl.full[s]);
         mbar_arrive_expect_tx(full, win_tx, leader);
         uint32_t dst = a_base + s * a_stage_bytes;
-        if (args.remap == 3) {
+        if (remap == 3) {
           // two-dimensional tile (image, tile row, tile column): the window is one box of sh_rows rows
           // of sh_wps pixels per channel block, from the tile's first window origin on
           const int img = (int)args.div_tiles_hw.div((uint32_t)t);
@@ -205,7 +212,7 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
       int n_img = 0, h_org = 0, w_org = 0, cb = 0, sx = 0, r = 0;
       // Swapped axis map: the activations are the N operand (tile_n pixels from n0 on, into the B
       // region) and the packed weights the 128-row operand (rows m0 .., into the A region).
-      const bool swap = args.swap != 0;
+      const bool swap = swap_map;
       const int pix0 = swap ? n0 : m0;
       const int wrow0 = swap ? m0 : n0;
       if (AMODE == A_IM2COL_TMA) {
@@ -402,23 +409,23 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
     uint32_t ph = 0;
     // two-dimensional tiles: the pixel of this row inside a tile does not change from tile to tile
     // (the tile width is a power of two)
-    const int tile_w_log2 = args.remap == 3 ? 31 - __clz(args.sh_wps) : 0;
+    const int tile_w_log2 = remap == 3 ? 31 - __clz(args.sh_wps) : 0;
     const int tile_h3 = kTileM >> tile_w_log2;
     const int row_in_tile = row >> tile_w_log2, col_in_tile = row & ((1 << tile_w_log2) - 1);
     for (int t = tile_first; t < tile_end && ok; t += tile_step, ++ti) {
     if (alternate && (ti & 1) != half) continue;
     B2C_TILE_ORIGIN(t)
     const unsigned m = (unsigned)m0 + (unsigned)row;
-    bool row_valid = m < (unsigned)(args.swap ? args.K : args.Mg);
+    bool row_valid = m < (unsigned)(swap_map ? args.K : args.Mg);
     int n_img = 0, pq = 0;
-    if (row_valid && !args.swap && args.remap < 2) {
+    if (row_valid && !swap_map && remap < 2) {
       n_img = (int)args.div_pq.div(m);
       pq = (int)(m - (unsigned)n_img * (unsigned)args.PQ);
     }
     // Where this row's results go: (out_img, out_pq) in the convolution's own output.  The phase
     // pack interleaves the sub-image results back and drops rows that fall outside the output.
     int out_img = n_img, out_pq = pq;
-    if (args.remap == 3 && row_valid) {
+    if (remap == 3 && row_valid) {
       // two-dimensional tiles: tile (image, tile row, tile column), row = pixel (row / 16, row % 16) of it
       const uint32_t tile = (uint32_t)m0 / kTileM;
       out_img = (int)args.div_tiles_hw.div(tile);
@@ -427,7 +434,7 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
       const int po = th * tile_h3 + row_in_tile, qo = tw * args.sh_valid_w + col_in_tile;
       row_valid = col_in_tile < args.sh_valid_w && po < args.out_P && qo < args.out_Q;
       out_pq = po * args.out_Q + qo;
-    } else if (args.remap == 2 && row_valid) {
+    } else if (remap == 2 && row_valid) {
       // shift execution: row m is window origin (n, hp, wp) on the padded grid of sh_hp x sh_wps positions
       const uint32_t rowi = args.div_wps.div(m);
       const int wp = (int)(m - rowi * (uint32_t)args.sh_wps);
@@ -435,7 +442,7 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
       const int hp = (int)rowi - out_img * args.sh_hp;
       row_valid = hp < args.out_P && wp < args.out_Q;
       out_pq = hp * args.out_Q + wp;
-    } else if (args.remap && row_valid) {
+    } else if (remap == 1 && row_valid) {
       const int ps = (int)args.div_q.div((uint32_t)pq), qs = pq - ps * args.Q;
       const int phases = args.ph_dh * args.ph_dw;
       out_img = n_img / phases;
@@ -629,15 +636,15 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
     if (ok) {
       // Output index of (m, k): NKPQ -> (n*K + k)*PQ + pq ; NPQK -> m*K + k.
       const long long base_nkpq = (long long)out_img * args.y_stride_n + out_pq + (long long)grp * args.K * args.out_PQ;
-      const long long base_npqk = args.remap ? ((long long)out_img * args.out_PQ + out_pq) * args.K : (long long)m * args.K;
+      const long long base_npqk = remap ? ((long long)out_img * args.out_PQ + out_pq) * args.K : (long long)m * args.K;
       const int cols = alternate ? args.tile_n : (args.tile_n >= 32 ? (args.tile_n >> 1) : 16);  // columns handled by this warp
       const int c_begin = alternate ? 0 : half * cols;
       if (c_begin < args.tile_n) {
         const uint32_t taddr =
             tmem_acc + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * args.tmem_cols) + (uint32_t)c_begin;
         // cluster reduction: the stage buffers are free once the accumulator is complete
-        const uint32_t xch = args.cluster_split ? a_base + (uint32_t)row * 4u + (uint32_t)c_begin * (kTileM * 4) : 0u;
-        if (args.swap) {
+        const uint32_t xch = cluster_split ? a_base + (uint32_t)row * 4u + (uint32_t)c_begin * (kTileM * 4) : 0u;
+        if (swap_map) {
           // accumulator row = output channel m, columns = pixels n0 + c_begin ..
           for (int c = 0; c < cols; c += 16) {
             int32_t v[16];
@@ -647,11 +654,11 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
           }
         } else if ((cols & 31) == 0) {
           for (int c = 0; c < cols; c += 32)
-            epilogue_columns<32>(args, taddr + (uint32_t)c, n0 + c_begin + c, row_valid, base_nkpq, base_npqk,
+            epilogue_columns<32, kSplit>(args, taddr + (uint32_t)c, n0 + c_begin + c, row_valid, base_nkpq, base_npqk,
                                  xch ? xch + (uint32_t)c * (kTileM * 4) : 0u, grp * args.K);
         } else {
           for (int c = 0; c < cols; c += 16)
-            epilogue_columns<16>(args, taddr + (uint32_t)c, n0 + c_begin + c, row_valid, base_nkpq, base_npqk,
+            epilogue_columns<16, kSplit>(args, taddr + (uint32_t)c, n0 + c_begin + c, row_valid, base_nkpq, base_npqk,
                                  xch ? xch + (uint32_t)c * (kTileM * 4) : 0u, grp * args.K);
         }
       }
@@ -665,7 +672,7 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
     }  // tile loop
   }
 
-  if (args.cluster_split) {
+  if (cluster_split) {
     B2C_TILE_ORIGIN(0)
     // ---------------------------------------------------------------- cluster reduction
     // Barrier 1: every slice's partial tile is in its block's shared memory.  Then block `rank`
@@ -756,10 +763,7 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
             }
             if (args.out_mode & B2C_OUT_I8) {
               int8_t* dst = args.y8 + o;
-              const uint32_t q4 = (uint32_t)(uint8_t)requant(acc[b][0], args.shift) |
-                                  ((uint32_t)(uint8_t)requant(acc[b][1], args.shift) << 8) |
-                                  ((uint32_t)(uint8_t)requant(acc[b][2], args.shift) << 16) |
-                                  ((uint32_t)(uint8_t)requant(acc[b][3], args.shift) << 24);
+              const uint32_t q4 = requant4(acc[b][0], acc[b][1], acc[b][2], acc[b][3], args.shift);
               if ((reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
                 *reinterpret_cast<uint32_t*>(dst) = q4;
               } else {
