@@ -969,7 +969,7 @@ int b2c_plan_create_grouped_timed(const b2c_conv_desc* desc, int32_t groups, voi
       sd.K = m * kg;
       Geom sg;
       if (resolve_geom(&sd, &sg) != B2C_OK) continue;
-      for (int nth = 0; nth < 6; ++nth) {
+      for (int nth = 0; nth < 10; ++nth) {
         PlaneArgs pl;
         if (!plane_plan(sg, groups / m, 0, nth, &pl)) break;
         b2c_embedding e;
@@ -1203,6 +1203,11 @@ static int run_convolve(b2c_plan* p, const int8_t* x, int32_t* y32, int8_t* y8, 
   } else if (p->emb.variant == B2C_VARIANT_IM2COL_EXPLICIT) {
     rc = encode_tiled_2d(&tmap_a, wsb, p->K_pad, (uint64_t)g.Mg, p->K_pad, 128, a.swap ? a.tile_n : kTileM, 128);
     if (rc != B2C_OK) return rc;
+  } else if (p->amode == A_PLANE) {
+    if (p->plane.box_bytes > 0) {
+      rc = encode_tiled_channels(&tmap_a, x, (long long)d.N * p->plane.img_channels, d.H * d.W, d.C, p->plane.box_bytes);
+      if (rc != B2C_OK) return rc;
+    }
   } else if (p->amode == A_WINDOW) {
     if (a.wn_linear) {
       tmap_a = p->tmap_b;  // the images arrive by plain bulk copies; any valid map
@@ -1240,7 +1245,7 @@ static int run_convolve(b2c_plan* p, const int8_t* x, int32_t* y32, int8_t* y8, 
   } else if (p->amode == A_PLANE) {
     PlaneArgs pl = p->plane;
     pl.x_bytes = (long long)(d.N - 1) * a.x_stride_n + (long long)d.C * d.H * d.W * a.groups;
-    CUDA_TRY(launch_conv_mma_plane(a, pl, st));
+    CUDA_TRY(launch_conv_mma_plane(tmap_a, a, pl, st));
   } else if (p->amode == A_WINDOW) {
     CUDA_TRY(launch_conv_mma_window(&tmap_a, &p->tmap_b, a, st));
   } else

@@ -175,7 +175,7 @@ struct ConvArgs {
 // Geometry of the window unroll over planes of units (A_PLANE, conv_mma_plane.cu); the kernel takes it beside ConvArgs.
 constexpr int kPlaneMinTiles = 2500;        // accumulator tiles of a problem from which the plane kernel runs it
 constexpr int kMaxStridePhases = 8;         // strides the window unroll handles
-constexpr int kPlaneMargin = 64;           // readable bytes on either side of the staged raw rows
+constexpr int kPlaneMargin = 128;          // readable bytes on either side of the staged raw rows
 constexpr int kMaxAcc = 8;                  // accumulator ring
 constexpr int kPlaneSmemMax = 224 * 1024;  // dynamic shared memory of one block
 struct PlaneArgs {
@@ -190,13 +190,15 @@ struct PlaneArgs {
   int max_ri;                          // grid rows the taps reach below a window's output rows
   int th, cr, tiles;                   // output grid rows of a window, grid rows of a raw chunk, accumulator tiles
   int seg_rows, segs, blocks;          // output grid rows of a segment (walked by one block), segments, blocks
+  int spi;                             // segments per image, or 0: segments of the batch's rows
   int plane_bytes, win_bytes, num_mma;
   int whole_images, img_slot, c_pitch, raw_bytes;  // raw staging: whole images, or one slot per channel
+  int box_bytes, img_channels;                     // tiled copies: bytes per channel (0: bulk copies); channels of an image
   int gpr, run_groups, zero_fill;                  // builder items per grid row (groups of columns)
   int w_bytes;                                     // packed weights of one group and column tile
   int nbuf, per_sm, win_stages, raw_stages, smem;
   int tile_n, cols, tmem_cols;                     // column tile, column tiles, tensor-memory columns
-  FastDiv div_rpi, div_pitch, div_gpr, div_nu, div_sw, div_overlap, div_w, div_hw4;
+  FastDiv div_rpi, div_pitch, div_gpr, div_nu, div_sw, div_overlap, div_w, div_hw4, div_spi;
   const uint8_t* w;            // packed weights: [group][column tile][MMA][half][channel][16 bytes]
   const uint64_t* mma_table;   // A descriptor of every MMA relative to the window: start (units) | distance of the halves << 16
   long long x_bytes;           // bytes of the whole input tensor
@@ -410,6 +412,8 @@ int encode_tiled_nhwc_rows(CUtensorMap* map, const void* base, int C_pad, int W,
 int encode_im2col_nhwc(CUtensorMap* map, const void* base, int C_pad, int W, int H, int N, int pad_w, int pad_h,
                        int S, int R, int dil_w, int dil_h, int stride_w, int stride_h, int channels_per_pixel,
                        int pixels_per_column, int swizzle_bytes);
+// NCHW int8 tensor as rows of hw / 4 words, one per (image, channel); a box is box_bytes of box_rows channels.
+int encode_tiled_channels(CUtensorMap* map, const void* base, long long rows, int hw, int box_rows, int box_bytes);
 int encode_tiled_nchw_window(CUtensorMap* map, const void* base, int W, int H, int C, int N, int box_w, int box_h);
 void set_last_cuda_error(int e);
 int get_last_cuda_error();
@@ -454,7 +458,7 @@ cudaError_t launch_conv_mma_pair(int amode, const CUtensorMap* tmap_a, const CUt
 size_t conv_mma_pair_smem_bytes(const ConvArgs& args);
 cudaError_t launch_conv_mma_window(const CUtensorMap* tmap_x, const CUtensorMap* tmap_b, const ConvArgs& args, cudaStream_t st);
 size_t conv_mma_window_smem_bytes(const ConvArgs& args);
-cudaError_t launch_conv_mma_plane(const ConvArgs& args, const PlaneArgs& pl, cudaStream_t st);
+cudaError_t launch_conv_mma_plane(const CUtensorMap& tmap, const ConvArgs& args, const PlaneArgs& pl, cudaStream_t st);
 // Geometry of the fused activation pack; false when the tensor has no bulk-copy form.
 bool fused_pack_geometry(int C, int H, int W, int C_pad, int* ct, int* pt, int* hw_tiles, int* ctiles, int* smem);
 cudaError_t launch_bounded_wait_selftest(int* status, cudaStream_t st);

@@ -20,15 +20,17 @@
 // walks consecutive windows, so the last max_ri rows of one are the first of the next: they are moved as units,
 // and every input row is fetched and turned into units once per block.
 //
-// Roles: warp 0 fetches the raw NCHW rows of a window by bulk copies (whole images, or one row segment per
-// channel; any width, the 16-byte boundaries around a segment are fetched with it) in chunks of at most `cr` grid rows, warp 1 issues the MMAs,
+// Roles: warp 0 fetches the raw NCHW rows of a window in chunks of at most `cr` grid rows: whole images or one row
+// segment per channel by bulk copies (any width, the 16-byte boundaries around a segment are fetched with it), or all
+// channels by one tiled copy where every channel starts on 16 bytes (bulk copies cost about 60 cycles each to issue,
+// 7600 a window of 64 channels; 315 images of 64 x 56 x 56, 3x3, 84 us with them, 70 without); warp 1 issues the MMAs,
 // the builder warps turn raw rows into units (byte transposes or unaligned words, zeros outside the image), the
 // epilogue warps drain the accumulators (activation step, shift / clip, NKPQ or NPQK stores).  The weights stay
 // resident.
 // What bounds it now: the stores of the results (about 5 cycles of the SM's store path per 128 bytes, 32 lanes from any
 // start) beside the builders' shared-memory traffic.  Before (operand rows written out by builder warps, or a rewrite
-// through memory) and after: 64 images of 3 x 227 x 227, 7x7 stride 2, 64 channels 97 -> 53 us; 32 of 1 x 700 x 161,
-// 20x5 stride 2, 76 -> 35; 15501 of 16 x 14 x 14, 3x3, 124 -> 104; 315 of 64 x 56 x 56, 3x3, 100 -> 91.
+// through memory) and after: 64 images of 3 x 227 x 227, 7x7 stride 2, 64 channels 97 -> 51 us; 32 of 1 x 700 x 161,
+// 20x5 stride 2, 76 -> 33; 15501 of 16 x 14 x 14, 3x3, 124 -> 94; 315 of 64 x 56 x 56, 3x3, 99 -> 81.
 // Copies of window w + 2, units of w + 1, MMAs of w and stores of w - 1 overlap.  Every wait is
 // bounded as in the other kernels.
 #include <algorithm>
@@ -123,14 +125,22 @@ __device__ __forceinline__ ChunkRows chunk_rows(const ConvArgs& args, const Plan
   return r;
 }
 // The grid rows are cut into segments, dealt to the blocks in turn; a segment is walked in windows of th output
-// rows.  Segment seg, and its window w: output rows [gr0, gr0 + rows), new unit rows [new0, new1).
+// rows.  Segment seg, and its window w: output rows [gr0, gr0 + rows), new unit rows [new0, new1).  With spi > 0 the
+// segments are those of one image each (spi per image, its P output rows only), else seg_rows rows of the batch.
 struct SegRows {
   int begin, end, windows;
 };
-__device__ __forceinline__ SegRows seg_rows(const PlaneArgs& pl, int seg) {
+__device__ __forceinline__ SegRows seg_rows(const ConvArgs& args, const PlaneArgs& pl, int seg) {
   SegRows b;
-  b.begin = seg * pl.seg_rows;
-  b.end = min(b.begin + pl.seg_rows, pl.total_rows);
+  if (pl.spi > 0) {
+    const int n = (int)pl.div_spi.div((uint32_t)seg);
+    const int r0 = (seg - n * pl.spi) * pl.seg_rows;
+    b.begin = n * pl.rpi + r0;
+    b.end = n * pl.rpi + min(r0 + pl.seg_rows, args.out_P);
+  } else {
+    b.begin = seg * pl.seg_rows;
+    b.end = min(b.begin + pl.seg_rows, pl.total_rows);
+  }
   b.windows = (b.end - b.begin + pl.th - 1) / pl.th;
   return b;
 }
@@ -154,7 +164,7 @@ __device__ __forceinline__ int segment_bytes(int rows, int W) { return (rows * W
 // stride (one column).  KB builder warps, KE epilogue warps, MINB blocks per SM.
 template <int RUNW, int VAR, int KB, int KE, int MINB>
 __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
-    conv_mma_plane_kernel(const ConvArgs args, const PlaneArgs pl) {
+    conv_mma_plane_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvArgs args, const PlaneArgs pl) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ PlaneCtl pc;
   SharedCtl* ctl = &pc.base;
@@ -237,7 +247,7 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
     uint32_t ph = 0;
     bool alive = true;
     for (int seg = seg_first; seg < seg_end && alive; seg += seg_step) {
-    const SegRows blk = seg_rows(pl, seg);
+    const SegRows blk = seg_rows(args, pl, seg);
     for (int win = 0; win < blk.windows && alive; ++win) {
       const WindowSpan sp = window_span(pl, blk, win);
       for (int c0 = sp.new0; c0 < sp.new1; c0 += pl.cr) {
@@ -246,6 +256,20 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
       if (!alive) break;
       const uint32_t full = smem_u32(&pc.raw_full[s]);
       const uint32_t raw = raw_off + (uint32_t)(s * pl.raw_bytes) + kPlaneMargin;
+      if (pl.box_bytes > 0) {
+        // one tiled copy: box_bytes of every channel of the image from the 16-byte boundary before row lo_a on
+        if (r.rows_a > 0) {
+          mbar_arrive_expect_tx(full, (uint32_t)(args.C * pl.box_bytes), leader);
+          tma_load_2d(smem_base + raw, &tmap_x, ((r.lo_a * args.W) & ~15) >> 2, r.n_a * pl.img_channels + grp * args.C, full, leader);
+        } else {
+          mbar_arrive_expect_tx(full, 0u, leader);
+        }
+        if (++s == pl.raw_stages) {
+          s = 0;
+          ph ^= 1u;
+        }
+        continue;
+      }
       // Copies of this chunk, dealt to the lanes twice: first the byte count, then the copies.  Each fetches
       // the 16-byte units its bytes lie in; bytes in the tensor's last, incomplete unit are copied by hand.
       const int copies = pl.whole_images ? r.images : args.C * r.images;
@@ -309,7 +333,7 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
     int s = 0, buf = 0;
     uint32_t ph = 0, aph = 0;
     for (int seg = seg_first; seg < seg_end && alive; seg += seg_step) {
-    const SegRows blk = seg_rows(pl, seg);
+    const SegRows blk = seg_rows(args, pl, seg);
     for (int win = 0; win < blk.windows && alive; ++win) {
       alive = __all_sync(0xffffffffu, mbar_wait(smem_u32(&pc.win_full[s]), ph, ctl, args.status));
       if (!alive) break;
@@ -362,7 +386,7 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
       return met;
     };
     for (int seg = seg_first; seg < seg_end && ok; seg += seg_step) {
-    const SegRows blk = seg_rows(pl, seg);
+    const SegRows blk = seg_rows(args, pl, seg);
     for (int win = 0; win < blk.windows && ok; ++win) {
       const WindowSpan sp = window_span(pl, blk, win);
       ok = mbar_wait_sleep(smem_u32(&pc.win_empty[ws]), wph ^ 1u, ctl, args.status, kSleepWindow);
@@ -685,7 +709,7 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
     int buf = 0, ti = 0;
     uint32_t aph = 0;
     for (int seg = seg_first; seg < seg_end && ok; seg += seg_step) {
-    const SegRows blk = seg_rows(pl, seg);
+    const SegRows blk = seg_rows(args, pl, seg);
     for (int win = 0; win < blk.windows && ok; ++win) {
       const WindowSpan sp = window_span(pl, blk, win);
       const int positions = sp.rows * pitch;
@@ -744,41 +768,41 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
 }
 
 template <int RUNW, int VAR, int KB, int KE, int MINB>
-cudaError_t launch_one(const ConvArgs& args, const PlaneArgs& pl, dim3 grid, cudaStream_t st) {
+cudaError_t launch_one(const CUtensorMap& tmap, const ConvArgs& args, const PlaneArgs& pl, dim3 grid, cudaStream_t st) {
   static std::atomic<unsigned long long> configured{0};
   cudaError_t e =
       set_max_dynamic_smem_once(configured, (const void*)conv_mma_plane_kernel<RUNW, VAR, KB, KE, MINB>, kPlaneSmemMax);
   if (e != cudaSuccess) return e;
-  return launch_pdl(conv_mma_plane_kernel<RUNW, VAR, KB, KE, MINB>, grid, dim3(64 + 32 * (KB + KE)), (size_t)pl.smem, st, args, pl);
+  return launch_pdl(conv_mma_plane_kernel<RUNW, VAR, KB, KE, MINB>, grid, dim3(64 + 32 * (KB + KE)), (size_t)pl.smem, st, tmap, args, pl);
 }
 
 template <int RUNW, int VAR>
-cudaError_t launch_form(const ConvArgs& args, const PlaneArgs& pl, dim3 grid, cudaStream_t st) {
+cudaError_t launch_form(const CUtensorMap& tmap, const ConvArgs& args, const PlaneArgs& pl, dim3 grid, cudaStream_t st) {
   // One block per SM: eight builder and eight epilogue warps; two blocks: four of each.
-  if (pl.per_sm == 1) return launch_one<RUNW, VAR, 8, 8, 1>(args, pl, grid, st);
-  return launch_one<RUNW, VAR, 4, 4, 2>(args, pl, grid, st);
+  if (pl.per_sm == 1) return launch_one<RUNW, VAR, 8, 8, 1>(tmap, args, pl, grid, st);
+  return launch_one<RUNW, VAR, 4, 4, 2>(tmap, args, pl, grid, st);
 }
 template <int RUNW>
-cudaError_t launch_row_form(const ConvArgs& args, const PlaneArgs& pl, dim3 grid, cudaStream_t st) {
-  if (pl.sw == 1) return launch_form<RUNW, 1>(args, pl, grid, st);
-  if (pl.sw == 2) return launch_form<RUNW, 2>(args, pl, grid, st);
-  return launch_form<RUNW, 0>(args, pl, grid, st);
+cudaError_t launch_row_form(const CUtensorMap& tmap, const ConvArgs& args, const PlaneArgs& pl, dim3 grid, cudaStream_t st) {
+  if (pl.sw == 1) return launch_form<RUNW, 1>(tmap, args, pl, grid, st);
+  if (pl.sw == 2) return launch_form<RUNW, 2>(tmap, args, pl, grid, st);
+  return launch_form<RUNW, 0>(tmap, args, pl, grid, st);
 }
 
 }  // namespace
 
-cudaError_t launch_conv_mma_plane(const ConvArgs& args, const PlaneArgs& pl, cudaStream_t st) {
+cudaError_t launch_conv_mma_plane(const CUtensorMap& tmap, const ConvArgs& args, const PlaneArgs& pl, cudaStream_t st) {
   const dim3 grid((unsigned)pl.blocks, (unsigned)pl.cols, (unsigned)std::max(1, args.groups));
   cudaError_t e;
   switch (pl.runw) {
     case 0:
-      e = pl.aligned == 2 ? launch_form<0, 2>(args, pl, grid, st)
-                          : (pl.aligned == 1 ? launch_form<0, 1>(args, pl, grid, st) : launch_form<0, 0>(args, pl, grid, st));
+      e = pl.aligned == 2 ? launch_form<0, 2>(tmap, args, pl, grid, st)
+                          : (pl.aligned == 1 ? launch_form<0, 1>(tmap, args, pl, grid, st) : launch_form<0, 0>(tmap, args, pl, grid, st));
       break;
-    case 1: e = launch_row_form<1>(args, pl, grid, st); break;
-    case 2: e = launch_row_form<2>(args, pl, grid, st); break;
-    case 4: e = launch_row_form<4>(args, pl, grid, st); break;
-    default: e = launch_row_form<6>(args, pl, grid, st); break;
+    case 1: e = launch_row_form<1>(tmap, args, pl, grid, st); break;
+    case 2: e = launch_row_form<2>(tmap, args, pl, grid, st); break;
+    case 4: e = launch_row_form<4>(tmap, args, pl, grid, st); break;
+    default: e = launch_row_form<6>(tmap, args, pl, grid, st); break;
   }
   return e != cudaSuccess ? e : cudaGetLastError();
 }

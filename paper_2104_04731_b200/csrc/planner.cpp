@@ -481,12 +481,13 @@ bool plane_form(const Geom& g, bool row_form, PlaneForm* f) {
 }
 
 // Schedule of one form with per_sm blocks per SM, windows of min_tiles to max_tiles accumulator tiles, dealt one by one
-// (`dealt`) or in segments: window height,
+// (`dealt`) or in segments, at most `stages` (see plane_choices): window height,
 // column tile and stages with the lowest estimated time (returned; negative if nothing fits).  The estimate adds up,
 // in SM cycles, what a window costs each role (constants measured on the kernel: builder items, 39 cycles and up per
 // MMA, the store path) and takes the slowest role per window, the way of the first window to its MMAs and the stores
 // of the last one.
-double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm, bool dealt, int min_tiles, int max_tiles, PlaneArgs* pl) {
+double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm, bool dealt, int min_tiles, int max_tiles, int stages,
+                      PlaneArgs* pl) {
   const b2c_conv_desc& d = g.d;
   const int HW = d.H * d.W;
   const long long total_rows = (long long)d.N * f.rpi;
@@ -524,26 +525,37 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
       const int wr = th + f.max_ri;
       const long long plane_units = (long long)wr * f.pitch;
       const long long last_read = (long long)tiles * kTileM + (long long)f.max_ri * f.pitch + f.max_si + 1;
-      const long long win_bytes = ((f.planes - 1) * plane_units + std::max(plane_units, last_read)) * 16;
+      const long long win_bytes = (((f.planes - 1) * plane_units + std::max(plane_units, last_read)) * 16 + 127) / 128 * 128;
       if (win_bytes > 200 * 1024) break;
       // Segments: single windows; or a block's share of all rows, cut further when the outputs that are being written
       // at the same time spread over more than about 100 MB; each segment builds its first max_ri rows anew.
-      const int blocks = (int)std::min<long long>(places, (total_rows + th - 1) / th);
+      int blocks = (int)std::min<long long>(places, (total_rows + th - 1) / th);
       long long share = (total_rows + blocks - 1) / blocks;
       if (dealt) share = std::min<long long>(share, th);
+      // Images of several windows: windows and segments end with the image (its overhang rows are no output rows, and
+      // no window needs rows of two images); equal parts of it.
+      int spi = 0;
+      if (f.rpi >= 2 * th) {
+        const long long want = std::max<long long>(th, std::min<long long>(share, g.P));  // rows of a segment
+        spi = (int)((g.P + want - 1) / want);
+        share = (g.P + spi - 1) / spi;
+        if (share > th && !dealt) share = (share + th - 1) / th * th;
+        spi = (int)((g.P + share - 1) / share);
+        blocks = (int)std::min<long long>(places, (long long)d.N * spi);
+      }
       const double active = (double)blocks * share * f.pitch * d.K * groups * out_bytes;
-      if (active > 100e6 && share > th) {
+      if (spi == 0 && active > 100e6 && share > th) {
         const int parts = (int)std::min<double>((double)((share + th - 1) / th), std::ceil(active / 100e6));
         share = (total_rows + (long long)blocks * parts - 1) / ((long long)blocks * parts);
       }
-      const long long segs = (total_rows + share - 1) / share, segs_per_block = (segs + blocks - 1) / blocks;
+      const long long segs = spi ? (long long)d.N * spi : (total_rows + share - 1) / share, segs_per_block = (segs + blocks - 1) / blocks;
       const long long per_block = (share + th - 1) / th * segs_per_block;
       const double conc = (double)std::min<long long>(per_sm, std::max<long long>(1, ((long long)blocks * cols * groups + kNumSMs - 1) / kNumSMs));
       const double mma = tiles * (num_mma * std::max(40.0, tile_n / 2.0) + 150.0);
       const double valid = (double)g.P / f.rpi * g.Q / f.pitch;
       const double tile_out = 4.0 * tile_n * out_cost * (0.4 + 0.6 * valid);  // store path of the SM
       const double tile_lat = 600.0 + tile_n * 2.5 * out_cost;                // one set of warps, start to end
-      const double epi = std::max(conc * tiles * tile_out, (double)((tiles + sets - 1) / sets) * tile_lat);
+      const double epi = std::max(conc * th * f.pitch / kTileM * tile_out, (double)((tiles + sets - 1) / sets) * tile_lat);
       // raw chunks of the window's new rows; also of the whole first window when a block has only that one
       for (int cr = th; cr <= wr; cr += std::max(1, f.max_ri)) {
         const bool whole_first = cr == wr && (dealt || per_block == 1);
@@ -556,8 +568,11 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
         const int img_slot = round_up(d.C * HW + 15, 16) + 16;
         const long long whole_bytes = (long long)images * img_slot;
         const bool whole = images > 2 || whole_bytes <= rows_bytes + rows_bytes / 4 || whole_bytes <= 8192;
-        const long long raw_data = whole ? whole_bytes : rows_bytes;
-        const double copies = whole ? images : (double)d.C * (1.0 + (double)cr / f.rpi);
+        // one tiled copy for all channels: they start on 16 bytes, the segment fits a box, and no chunk has two images
+        const int box = round_up(raw_rows * d.W + 15, 16);
+        const bool tiled = !whole && spi > 0 && HW % 16 == 0 && d.C >= 4 && d.C <= 256 && box <= 1024;
+        const long long raw_data = whole ? whole_bytes : (tiled ? (long long)d.C * box : rows_bytes);
+        const double copies = whole ? images : (tiled ? 1.0 : (double)d.C * (spi ? 1.0 : 1.0 + (double)cr / f.rpi));
         const long long raw_bytes = (raw_data + 2 * kPlaneMargin + 127) / 128 * 128;
         const int first_chunks = (int)((std::min<long long>(share, th) + f.max_ri + cr - 1) / cr);
         const long long row_items = f.runw ? (f.pitch + f.qb - 1) / f.qb : (long long)ncb * f.ndh * ((d.W + 3) / 4);
@@ -576,7 +591,7 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
         (void)build_cycles(std::min<long long>(share, th) + f.max_ri, &first_lat);
         build_lat += move / kb + 300.0;
         const double copy = 900.0 + (double)raw_data / 24.0 + copies * 60.0;
-        for (int st = 0; st < 3; ++st) {
+        for (int st = 2 - stages; st < 3; ++st) {
           const bool single = per_block == 1;
           const int ws = st < 2 ? 2 : 1, rs = (single && whole_first) ? 1 : (st < 1 ? 2 : 1);
           if (single && st < 2) continue;
@@ -588,8 +603,8 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
           if (ws == 1) chain = build_lat + std::max(rs == 1 ? copy : 0.0, mma);
           double steady = std::max(std::max(conc * build, conc * mma), std::max(epi, chain));
           if (nbuf == 1) steady = std::max(steady, mma + epi);
-          // (a block's last window is as long as the others unless the rows run out)
-          const double windows = std::max(1.0, dealt ? std::ceil((double)segs / blocks) : (double)total_rows / blocks / th);
+          // (a last, partly filled round of segments: the stores of the others' get its share of the memory)
+          const double windows = std::max(1.0, (dealt || spi) ? (double)((share + th - 1) / th) * 0.5 * (std::ceil((double)segs / blocks) + (double)segs / blocks) : (double)total_rows / blocks / th);
           const double t = 3000 + copy * (rs == 1 ? first_chunks : 1) + first_lat + first_chunks * 150.0 + mma / tiles + epi + w_bytes / 40.0 * conc +
                            (windows - 1) * steady + (dealt ? 0.0 : (double)(segs_per_block - 1) * f.max_ri / th * conc * build);
           if (best >= 0 && t >= best * 0.999) continue;
@@ -609,7 +624,9 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
           pl->win_bytes = (int)win_bytes;
           pl->whole_images = whole ? 1 : 0;
           pl->img_slot = img_slot;
-          pl->c_pitch = round_up(raw_rows * d.W, 16) + 64;
+          pl->c_pitch = tiled ? box : round_up(raw_rows * d.W, 16) + 64;
+          pl->box_bytes = tiled ? box : 0;
+          pl->spi = spi;
           pl->raw_bytes = (int)raw_bytes;
           pl->win_stages = ws;
           pl->raw_stages = rs;
@@ -623,7 +640,7 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
 }
 
 // Form and schedules of the plane kernel, the lowest estimate first: the best one for each number of blocks per SM,
-// way of dealing windows and range of window heights (their order depends on how the store path, the builders and DRAM share the time, which
+// way of dealing windows, range of window heights and number of buffers (their order depends on how the store path, the builders and DRAM share the time, which
 // the estimate knows to 10 to 25 %; the timed selection tries them all).
 struct PlaneChoice {
   double t;
@@ -658,17 +675,19 @@ bool plane_choices(const Geom& g, int groups, PlaneForm* form, std::vector<Plane
     PlaneForm cand;
     if (!plane_form(g, f == 1, &cand)) continue;
     std::vector<PlaneChoice> list;
-    // blocks per SM, dealt, fewest and most tiles of a window (the last two: windows on the other side of what the
-    // estimate takes for the best height)
-    static const int kStyles[6][4] = {{1, 1, 1, 16}, {2, 1, 1, 16}, {1, 0, 1, 16}, {2, 0, 1, 16}, {1, 1, 1, 5}, {2, 1, 6, 16}};
+    // blocks per SM, dealt, fewest and most tiles of a window, buffers (2: two windows and two raw chunks, 1: two and
+    // one, 0: one of each; fewer are often better although no role waits less: they leave the L1 more room)
+    static const int kStyles[10][5] = {{1, 1, 4, 5, 0}, {1, 1, 5, 8, 1}, {1, 1, 4, 8, 2},  {1, 1, 9, 16, 2}, {2, 1, 1, 4, 2},
+                                       {2, 1, 5, 16, 0}, {2, 1, 5, 8, 1}, {2, 1, 9, 16, 1}, {2, 0, 5, 16, 2}, {1, 0, 1, 16, 2}};
     for (const int* style : kStyles) {
       PlaneChoice c;
       std::memset(&c.pl, 0, sizeof(c.pl));
-      c.t = plane_schedule(g, groups, cand, style[0], style[1] != 0, style[2], style[3], &c.pl);
+      c.t = plane_schedule(g, groups, cand, style[0], style[1] != 0, style[2], style[3], style[4], &c.pl);
       if (c.t < 0) continue;
       bool same = false;
       for (const PlaneChoice& o : list)
-        same |= o.pl.per_sm == c.pl.per_sm && o.pl.th == c.pl.th && o.pl.seg_rows == c.pl.seg_rows && o.pl.tile_n == c.pl.tile_n;
+        same |= o.pl.per_sm == c.pl.per_sm && o.pl.th == c.pl.th && o.pl.seg_rows == c.pl.seg_rows && o.pl.tile_n == c.pl.tile_n &&
+                o.pl.win_stages == c.pl.win_stages && o.pl.raw_stages == c.pl.raw_stages;
       if (!same) list.push_back(c);
     }
     if (list.empty()) continue;
@@ -729,6 +748,8 @@ bool plane_plan(const Geom& g, int groups, int tile_n, int nth, PlaneArgs* pl, s
   pl->div_gpr = make_fastdiv((uint32_t)pl->gpr);
   pl->div_nu = make_fastdiv((uint32_t)std::max(1, f.planes / f.ndw));
   pl->div_w = make_fastdiv((uint32_t)d.W);
+  pl->div_spi = make_fastdiv((uint32_t)std::max(1, pl->spi));
+  pl->img_channels = d.C * groups;
   pl->div_hw4 = make_fastdiv((uint32_t)std::max(1, HW / 4));
   pl->div_overlap = make_fastdiv((uint32_t)std::max(1, f.max_ri * f.pitch));
   pl->div_sw = make_fastdiv((uint32_t)d.stride_w);

@@ -161,6 +161,28 @@ int encode_tiled_nchw_window(CUtensorMap* map, const void* base, int W, int H, i
   return B2C_OK;
 }
 
+int encode_tiled_channels(CUtensorMap* map, const void* base, long long rows, int hw, int box_rows, int box_bytes) {
+  std::call_once(g_once, resolve);
+  if (injected_failure()) return B2C_E_CUDA;
+  if (!g_tiled) {
+    set_last_cuda_error((int)CUDA_ERROR_NOT_FOUND);
+    return B2C_E_CUDA;
+  }
+  // (words, because a box is at most 256 elements wide)
+  cuuint64_t dims[2] = {(cuuint64_t)hw / 4, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)hw};
+  cuuint32_t box[2] = {(cuuint32_t)box_bytes / 4, (cuuint32_t)box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  CUresult r = g_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<void*>(base), dims, strides, box, estr,
+                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    set_last_cuda_error((int)r);
+    return B2C_E_CUDA;
+  }
+  return B2C_OK;
+}
+
 }  // namespace b2c
 
 extern "C" int b2c_last_cuda_error(void) { return b2c::get_last_cuda_error(); }

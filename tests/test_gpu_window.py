@@ -55,6 +55,8 @@ def test_bias_vector_and_scalar_loads(lib, K, groups):
     (300, 18, 14, 14, 16, 3, 3, 1, 1, 1, 8),           # whole images staged (3528 bytes: two alignments in turn)
     (30, 3, 225, 223, 16, 5, 5, 2, 2, 1, 7),           # enough rows for every block to walk windows in every schedule
     (100, 48, 30, 30, 64, 3, 3, 1, 1, 1, 9),           # the same, channel form with moved overlap rows
+    (20, 64, 56, 24, 40, 3, 3, 1, 1, 1, 9),            # one tiled copy for all channels: segments of single images
+    (12, 20, 96, 44, 32, 3, 5, 2, (1, 2), 1, 8),       # the same with stride 2; ragged last segment of an image
 ])
 @pytest.mark.parametrize("out_layout,out_mode", [(0, 3), (1, 2)])
 def test_plane_kernel(lib, case, out_layout, out_mode):
