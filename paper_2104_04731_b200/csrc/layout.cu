@@ -16,6 +16,31 @@ constexpr int kPackMaxC = 128;  // channels per tile (64 when the padded channel
 constexpr int kPackMaxP = 256;  // pixels per tile
 constexpr int kPackSmem = kPackMaxC * (kPackMaxP + 4) + (kPackMaxC / 16) * 16;
 
+// Channel-pack weights: out[k][(r*S + s)][c_pad] = w[k][c][r][s], zeros for c >= C.  A thread forms four consecutive
+// channels of one tap.
+__device__ __forceinline__ void pack_weights_cp_words(const WeightPack& p, unsigned first, unsigned step) {
+  const unsigned words = (unsigned)p.C_pad >> 2, total = (unsigned)p.K * (unsigned)p.RS * words;  // (fewer than 2^31: checked by the host)
+  for (unsigned i = first; i < total; i += step) {
+    const unsigned kt = i / words, c = (i - kt * words) * 4u;
+    const unsigned k = kt / (unsigned)p.RS, tap = kt - k * (unsigned)p.RS;
+    const int8_t* src = p.w + ((size_t)k * p.C + c) * p.RS + tap;
+    uint32_t v = 0;
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      if ((int)c + b < p.C) v |= (uint32_t)(uint8_t)src[(size_t)b * p.RS] << (8 * b);
+    reinterpret_cast<uint32_t*>(p.out)[i] = v;
+  }
+}
+// The activation-pack kernels take the weight pack along: the last p.blocks blocks of the x axis do it.
+__device__ __forceinline__ bool weight_pack_block(const WeightPack& p) {
+  const int extra = (int)blockIdx.x - ((int)gridDim.x - p.blocks);
+  if (p.blocks == 0 || extra < 0) return false;
+  pdl_wait();
+  if (blockIdx.y == 0) pack_weights_cp_words(p, (unsigned)extra * blockDim.x + threadIdx.x, (unsigned)p.blocks * blockDim.x);
+  pdl_launch_dependents();
+  return true;
+}
+
 // One block moves a [CT channels] x [PT pixels] tile of one image through shared memory.
 // Reads run along the pixel axis of NCHW in VEC-byte vectors (VEC = 16 or 4 when H*W allows the
 // alignment, else 1) with many loads in flight per thread; the tile is kept as rows of `pitch`
@@ -27,8 +52,10 @@ constexpr int kPackSmem = kPackMaxC * (kPackMaxP + 4) + (kPackMaxC / 16) * 16;
 template <int VEC>
 __global__ void __launch_bounds__(kPackThreads) pack_activations_kernel(const int8_t* __restrict__ x,
                                                                         int8_t* __restrict__ out, int C, int HW,
-                                                                        int C_pad, int hw_tiles, int CT, int PT, Dbg dbg) {
+                                                                        int C_pad, int hw_tiles, int CT, int PT, WeightPack wp,
+                                                                        Dbg dbg) {
   __shared__ __align__(16) uint8_t tile[kPackSmem];
+  if (weight_pack_block(wp)) return;
   const int n = blockIdx.x / hw_tiles;
   const int c0 = blockIdx.y * CT;
   const int hw0 = (blockIdx.x - n * hw_tiles) * PT;
@@ -178,9 +205,10 @@ template <bool kRowMode>
 __global__ void __launch_bounds__(kPackThreads) pack_activations_bulk_kernel(const int8_t* __restrict__ x,
                                                                              int8_t* __restrict__ out, int C, int HW,
                                                                              int C_pad, int hw_tiles, int CT, int PT,
-                                                                             int* status, Dbg dbg) {
+                                                                             WeightPack wp, int* status, Dbg dbg) {
   extern __shared__ __align__(128) uint8_t btile[];
   __shared__ __align__(8) unsigned long long bar;
+  if (weight_pack_block(wp)) return;
   const int n = blockIdx.x / hw_tiles;
   const int c0 = blockIdx.y * CT;
   const int hw0 = (blockIdx.x - n * hw_tiles) * PT;
@@ -338,23 +366,16 @@ __global__ void __launch_bounds__(kPackThreads) pack_small_images_kernel(const i
   }
 }
 
-// Channel-pack weights: out[k][(r*S + s)][c_pad] = w[k][c][r][s], zeros for c >= C.
-__global__ void pack_weights_cp_kernel(const int8_t* __restrict__ w, int8_t* __restrict__ out, int K, int C, int RS,
-                                       int C_pad) {
-  const long long total = (long long)K * RS * C_pad;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C_pad);
-    const long long kt = i / C_pad;
-    const int tap = (int)(kt % RS);
-    const long long k = kt / RS;
-    out[i] = c < C ? w[(k * C + c) * RS + tap] : (int8_t)0;
-  }
+__global__ void __launch_bounds__(256) pack_weights_cp_kernel(WeightPack p) {
+  pdl_wait();
+  pack_weights_cp_words(p, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  pdl_launch_dependents();
 }
 
 // Table-driven weight pack for the rewritten maps: out[k][j] = w[k][table[j]], zero where table[j] < 0.
 __global__ void pack_weights_table_kernel(const int8_t* __restrict__ w, int8_t* __restrict__ out, int K, int Kg, int cols,
                                           const int32_t* __restrict__ table) {
+  pdl_wait();
   const long long total = (long long)K * cols;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
@@ -363,12 +384,14 @@ __global__ void pack_weights_table_kernel(const int8_t* __restrict__ w, int8_t* 
     const int src = table[j];
     out[i] = src >= 0 ? w[k * Kg + src] : (int8_t)0;
   }
+  pdl_launch_dependents();
 }
 
 // Stencil-unroll weights: rows of w[k][(c,r,s)] with every (c, r) run of S taps padded with zeros
 // to S_run entries (S_run = S for the plain unroll), then the row zero-padded to K_pad.
 __global__ void pack_weights_rows_kernel(const int8_t* __restrict__ w, int8_t* __restrict__ out, int K, int Kg,
                                          int K_pad, int S, int S_run) {
+  pdl_wait();
   const long long total = (long long)K * K_pad;
   const int runs = Kg / S;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
@@ -378,11 +401,13 @@ __global__ void pack_weights_rows_kernel(const int8_t* __restrict__ w, int8_t* _
     const int run = j / S_run, s = j - run * S_run;
     out[i] = (run < runs && s < S) ? w[k * Kg + run * S + s] : (int8_t)0;
   }
+  pdl_launch_dependents();
 }
 
 // Weights of the plane kernel, in the order its MMAs read them: [group][column tile][MMA][half][channel][16].
 __global__ void pack_weights_plane_kernel(const int8_t* __restrict__ w, int8_t* __restrict__ out, int groups, int K, int Kg,
                                            int tile_n, int cols, int num_mma, const int32_t* __restrict__ wsrc) {
+  pdl_wait();
   const long long total = (long long)groups * cols * num_mma * 32 * tile_n;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
@@ -398,6 +423,7 @@ __global__ void pack_weights_plane_kernel(const int8_t* __restrict__ w, int8_t* 
     const int src = wsrc[unit * 16 + b];
     out[i] = (k < K && src >= 0) ? w[(grp * K + k) * Kg + src] : (int8_t)0;
   }
+  pdl_launch_dependents();
 }
 
 // Explicit stencil unroll.  One thread produces 16 consecutive reduction entries of one output
@@ -720,9 +746,22 @@ int grid_for(long long total, int block) {
 
 }  // namespace
 
-cudaError_t launch_pack_activations(const int8_t* x, int8_t* out, int N, int C, int H, int W, int C_pad,
-                                    cudaStream_t st, int* status, const Dbg& dbg) {
+WeightPack make_weight_pack(const int8_t* w, int8_t* out, int K, int C, int RS, int C_pad) {
+  WeightPack p = {w, out, K, C, RS, C_pad, 0};
+  p.blocks = (int)std::min<long long>(4 * kNumSMs, ((long long)K * RS * (C_pad / 4) + kPackThreads - 1) / kPackThreads);
+  return p;
+}
+bool weight_pack_rides(const int8_t* x, int N, int C, int H, int W) {
   const int HW = H * W;
+  const bool small_images = (reinterpret_cast<uintptr_t>(x) & 15) == 0 && (C % 16) == 0 && C <= 64 && (HW % 4) == 0 && HW <= 256 &&
+                            C * HW <= 12 * 1024 && N >= 8 * kNumSMs;
+  return !small_images;  // (that kernel moves enough that a launch more does not show)
+}
+
+cudaError_t launch_pack_activations(const int8_t* x, int8_t* out, int N, int C, int H, int W, int C_pad,
+                                    cudaStream_t st, int* status, const Dbg& dbg, const WeightPack* ride) {
+  const int HW = H * W;
+  const WeightPack wp = ride ? *ride : WeightPack{nullptr, nullptr, 0, 0, 0, 0, 0};
   int CT = C_pad >= 128 ? 128 : 64;
   const bool a16 = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
   // large batches of small images with few channels: several whole images per block
@@ -741,23 +780,23 @@ cudaError_t launch_pack_activations(const int8_t* x, int8_t* out, int N, int C, 
     // small tensors: narrower channel tiles so that the grid still covers the machine
     while (CT > 32 && (long long)hw_tiles * N * ((C_pad + CT - 1) / CT) < 2 * kNumSMs) CT >>= 1;
     const size_t smem = (size_t)(CT / 16) * (16 * PT + 16);
-    dim3 grid((unsigned)hw_tiles * (unsigned)N, (C_pad + CT - 1) / CT, 1);
+    dim3 grid((unsigned)hw_tiles * (unsigned)N + (unsigned)wp.blocks, (C_pad + CT - 1) / CT, 1);
     if (row_mode)
       return launch_pdl(pack_activations_bulk_kernel<true>, grid, dim3(kPackThreads), smem, st, x, out, C, HW, C_pad,
-                        hw_tiles, CT, PT, status, dbg);
+                        hw_tiles, CT, PT, wp, status, dbg);
     return launch_pdl(pack_activations_bulk_kernel<false>, grid, dim3(kPackThreads), smem, st, x, out, C, HW, C_pad,
-                      hw_tiles, CT, PT, status, dbg);
+                      hw_tiles, CT, PT, wp, status, dbg);
   }
   const int PT = HW > 128 ? 256 : (HW > 64 ? 128 : 64);
   const int hw_tiles = (HW + PT - 1) / PT;
-  dim3 grid((unsigned)hw_tiles * (unsigned)N, (C_pad + CT - 1) / CT, 1);
+  dim3 grid((unsigned)hw_tiles * (unsigned)N + (unsigned)wp.blocks, (C_pad + CT - 1) / CT, 1);
   if ((HW % 16) == 0 && a16)
     return launch_pdl(pack_activations_kernel<16>, grid, dim3(kPackThreads), 0, st, x, out, C, HW, C_pad, hw_tiles, CT,
-                      PT, dbg);
+                      PT, wp, dbg);
   if ((HW % 4) == 0 && a16)
     return launch_pdl(pack_activations_kernel<4>, grid, dim3(kPackThreads), 0, st, x, out, C, HW, C_pad, hw_tiles, CT,
-                      PT, dbg);
-  return launch_pdl(pack_activations_kernel<1>, grid, dim3(kPackThreads), 0, st, x, out, C, HW, C_pad, hw_tiles, CT, PT, dbg);
+                      PT, wp, dbg);
+  return launch_pdl(pack_activations_kernel<1>, grid, dim3(kPackThreads), 0, st, x, out, C, HW, C_pad, hw_tiles, CT, PT, wp, dbg);
 }
 
 cudaError_t launch_pack_wait_selftest(int* status, cudaStream_t st) {
@@ -767,16 +806,14 @@ cudaError_t launch_pack_wait_selftest(int* status, cudaStream_t st) {
 
 cudaError_t launch_pack_weights_cp(const int8_t* w, int8_t* out, int K, int C, int R, int S, int C_pad,
                                    cudaStream_t st) {
-  const long long total = (long long)K * R * S * C_pad;
-  pack_weights_cp_kernel<<<grid_for(total, 256), 256, 0, st>>>(w, out, K, C, R * S, C_pad);
-  return cudaGetLastError();
+  const WeightPack p = make_weight_pack(w, out, K, C, R * S, C_pad);
+  return launch_pdl(pack_weights_cp_kernel, dim3((unsigned)p.blocks), dim3(kPackThreads), 0, st, p);
 }
 
 cudaError_t launch_pack_weights_table(const int8_t* w, int8_t* out, int K, int Kg, int cols, const int32_t* table,
                                       cudaStream_t st) {
   const long long total = (long long)K * cols;
-  pack_weights_table_kernel<<<grid_for(total, 256), 256, 0, st>>>(w, out, K, Kg, cols, table);
-  return cudaGetLastError();
+  return launch_pdl(pack_weights_table_kernel, dim3(grid_for(total, 256)), dim3(256), 0, st, w, out, K, Kg, cols, table);
 }
 
 namespace {
@@ -805,15 +842,14 @@ cudaError_t launch_expand_group_weights(const int8_t* w, int8_t* out, int K, int
 cudaError_t launch_pack_weights_rows(const int8_t* w, int8_t* out, int K, int Kg, int K_pad, int S, int S_run,
                                      cudaStream_t st) {
   const long long total = (long long)K * K_pad;
-  pack_weights_rows_kernel<<<grid_for(total, 256), 256, 0, st>>>(w, out, K, Kg, K_pad, S, S_run);
-  return cudaGetLastError();
+  return launch_pdl(pack_weights_rows_kernel, dim3(grid_for(total, 256)), dim3(256), 0, st, w, out, K, Kg, K_pad, S, S_run);
 }
 
 cudaError_t launch_pack_weights_plane(const int8_t* w, int8_t* out, int groups, int K, int Kg, int tile_n, int cols, int num_mma,
                                        const int32_t* wsrc, cudaStream_t st) {
   const long long total = (long long)groups * cols * num_mma * 32 * tile_n;
-  pack_weights_plane_kernel<<<grid_for(total, 256), 256, 0, st>>>(w, out, groups, K, Kg, tile_n, cols, num_mma, wsrc);
-  return cudaGetLastError();
+  return launch_pdl(pack_weights_plane_kernel, dim3(grid_for(total, 256)), dim3(256), 0, st, w, out, groups, K, Kg, tile_n, cols, num_mma,
+                    wsrc);
 }
 
 cudaError_t launch_im2col(const int8_t* x, int8_t* a, const GatherEntry* table, long long Mg, int PQ, int Q, int H,

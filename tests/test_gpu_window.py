@@ -110,3 +110,27 @@ def test_grouped_plane_kernel(lib, case):
     assert y32 is None or np.array_equal(y32.cpu().numpy(), want[0])
     assert y8 is None or np.array_equal(y8.cpu().numpy(), want[1])
     plan.destroy()
+
+
+# ---- one-shot call: weights packed by the launch that packs the activations -----------------------------------------
+@pytest.mark.parametrize("case", [
+    # N, C, H, W, K, R, stride, pad, dil
+    (1, 64, 56, 56, 64, 3, 1, 1, 1),     # rows by bulk copies
+    (2, 48, 14, 14, 72, 3, 1, 1, 1),     # whole images by bulk copies; 48 channels padded to 64
+    (3, 33, 9, 11, 40, 3, 2, 1, 1),      # odd image: the loads of the plain pack kernel; 33 channels
+    (2, 70, 12, 10, 129, 1, 1, 0, 1),    # 1x1
+])
+def test_one_shot_packs_weights_with_the_activations(lib, case):
+    N, C, H, W, K, R, stride, pad, dil = case
+    xs = [int8_uniform((N, C, H, W), 1051 + i) for i in range(2)]
+    ws = [int8_uniform((K, C, R, R), 1061 + i) for i in range(2)]
+    lib.oneshot_cache_clear()
+    for x, w in zip(xs + xs[::-1], ws + ws):   # weights and activations change from call to call
+        want = oracle.conv2d_int8(x, w, stride, pad, dil, 9)
+        y32 = torch.full(want[0].shape, -7777777, dtype=torch.int32, device="cuda")
+        y8 = torch.full(want[1].shape, 77, dtype=torch.int8, device="cuda")
+        lib.conv2d_int8(to_dev(x), to_dev(w), stride, pad, dil, 9, y32, y8)
+        torch.cuda.synchronize()
+        assert np.array_equal(y32.cpu().numpy(), want[0]) and np.array_equal(y8.cpu().numpy(), want[1])
+    assert lib.oneshot_status() == b2c.OK
+    lib.oneshot_cache_clear()
