@@ -417,6 +417,12 @@ __device__ __forceinline__ void store_columns(const ConvArgs& args, int32_t* v, 
       if (full && (K & 3) == 0) {
 #pragma unroll
         for (int j = 0; j < NC; j += 4) *reinterpret_cast<int4*>(dst + j) = make_int4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+      } else if ((K & 3) == 0) {
+        // (a last, shorter run of channels in 16-byte pieces too, as in the int8 rows below: 32 images of 32 x 112 x 112 ->
+        // 48, 3x3, value by value 60 us, so 35; int8 55, so 18; both 84, so 41)
+#pragma unroll
+        for (int j = 0; j < NC; j += 4)
+          if (kbase + j < K) *reinterpret_cast<int4*>(dst + j) = make_int4(v[j], v[j + 1], v[j + 2], v[j + 3]);
       } else {
 #pragma unroll
         for (int j = 0; j < NC; ++j)
@@ -425,9 +431,10 @@ __device__ __forceinline__ void store_columns(const ConvArgs& args, int32_t* v, 
     }
     if (args.out_mode & B2C_OUT_I8) {
       int8_t* dst = args.y8 + base_npqk + kbase;
-      if (full && (K & 15) == 0) {
+      if ((K & 15) == 0) {
 #pragma unroll
         for (int g = 0; g < NC; g += 16) {
+          if (kbase + g >= K) break;
           uint32_t w[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) w[j] = requant4(v[g + j * 4], v[g + j * 4 + 1], v[g + j * 4 + 2], v[g + j * 4 + 3], args.shift);
@@ -580,6 +587,68 @@ __device__ __forceinline__ void epilogue_columns(const ConvArgs& args, uint32_t 
     return;
   }
   store_columns<NC, SPLIT>(args, v, kbase, row_valid, base_nkpq, base_npqk, bias_off);
+}
+
+// NPQK int32 results whose rows (a pixel's channels) are multiples of 16 bytes, in the int8 tensor too if there is one.
+__device__ __forceinline__ bool rows_of_pieces(const ConvArgs& args) {
+  return args.out_layout == B2C_LAYOUT_NHWC && (args.out_mode & B2C_OUT_I32) &&
+         (args.K & ((args.out_mode & B2C_OUT_I8) ? 15 : 3)) == 0;
+}
+
+// Epilogue of `cols` (a multiple of 16) accumulator columns into such rows.  A lane holds the channels of its own pixel;
+// stored as they are, every 16-byte store of a warp touches 32 rows and half a sector of each.  Instead four lanes
+// exchange 16-byte pieces of their sums (a 4 x 4 transpose by shuffles), so that a store covers 64 consecutive bytes of
+// each of 8 pixels.  16 columns at a time: these kernels have 64 registers, and 32 columns with the exchange spill.
+// (int8 alone stays with store_columns: 16 bytes of 32 rows a store, and the exchange costs more than it saves, 128
+// images of 64 x 28 x 28 -> 128, 3x3: 11.2 us, exchanged 14.2.)  base: this lane's pixel in the tensor, -1 = not stored;
+// executed by all lanes.  Measured with the channel pack, int32 alone: 128 images of 64 x 28 x 28 -> 128, 3x3, 26.6 -> 19.5
+// us; 64 of 64 x 56 x 56 -> 64, 1x1, 24.6 -> 13.7; 256 of 128 x 14 x 14 -> 256, 1x1, 19.6 -> 12.2.
+__device__ __forceinline__ void epilogue_rows(const ConvArgs& args, uint32_t taddr, int cols, int kbase, long long base,
+                                              int bias_off = 0) {
+  const int lane = threadIdx.x & 31;
+  const bool b0 = lane & 1, b1 = lane & 2;
+#ifdef B2C_DEBUG_BOUNDS
+  if (base >= 0 && kbase < args.K) {
+    const long long first = base + kbase, last = base + min(kbase + cols, args.K) - 1;
+    bool ok = B2C_O32_OK(args.dbg, 21, args.y32 + first, 4) && B2C_O32_OK(args.dbg, 21, args.y32 + last, 4);
+    if (ok && (args.out_mode & B2C_OUT_I8)) ok = B2C_O8_OK(args.dbg, 22, args.y8 + first, 1) && B2C_O8_OK(args.dbg, 22, args.y8 + last, 1);
+    if (!ok) base = -1;
+  }
+#endif
+#pragma unroll 1
+  for (int c = 0; c < cols && kbase + c < args.K; c += 16) {
+    int32_t x[16];
+    __syncwarp();
+    tmem_ld<16>(taddr + (uint32_t)c, x);
+    activate_columns<16>(args, x, kbase + c, bias_off);
+    if ((args.out_mode & B2C_OUT_I8) && base >= 0) {
+      uint32_t w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) w[j] = requant4(x[j * 4], x[j * 4 + 1], x[j * 4 + 2], x[j * 4 + 3], args.shift);
+      *reinterpret_cast<uint4*>(args.y8 + base + kbase + c) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    // piece p of this lane's pixel becomes piece (lane & 3) of pixel p of the four lanes
+#pragma unroll
+    for (int p = 0; p < 16; p += 8)
+#pragma unroll
+      for (int k = p; k < p + 4; ++k) {
+        const int32_t got = __shfl_xor_sync(0xffffffffu, b0 ? x[k] : x[k + 4], 1);
+        x[k] = b0 ? got : x[k];
+        x[k + 4] = b0 ? x[k + 4] : got;
+      }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int32_t got = __shfl_xor_sync(0xffffffffu, b1 ? x[k] : x[k + 8], 2);
+      x[k] = b1 ? got : x[k];
+      x[k + 8] = b1 ? x[k + 8] : got;
+    }
+    const int k = kbase + c + (lane & 3) * 4;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const long long at = __shfl_sync(0xffffffffu, base, (lane & ~3) + j);
+      if (at >= 0 && k < args.K) *reinterpret_cast<int4*>(args.y32 + at + k) = make_int4(x[j * 4], x[j * 4 + 1], x[j * 4 + 2], x[j * 4 + 3]);
+    }
+  }
 }
 
 }  // namespace

@@ -134,3 +134,36 @@ def test_one_shot_packs_weights_with_the_activations(lib, case):
         assert np.array_equal(y32.cpu().numpy(), want[0]) and np.array_equal(y8.cpu().numpy(), want[1])
     assert lib.oneshot_status() == b2c.OK
     lib.oneshot_cache_clear()
+
+
+# ---- NPQK results in 16-byte pieces: exchanged between four lanes (int32 sums), a last run of channels shorter than a tile ----
+@pytest.mark.parametrize("K", [4, 12, 16, 36, 48, 80, 272])
+@pytest.mark.parametrize("in_layout,case", [
+    # N, C, H, W, R, S, stride, pad, dil, shift: pixel counts that are no multiple of 4, 32 or 128
+    (1, (3, 32, 7, 9, 3, 3, 1, 1, 1, 8)),
+    (0, (1, 3, 21, 17, 3, 3, 2, 1, 1, 6)),
+    (1, (2, 16, 13, 11, 2, 2, 1, 0, 3, 7)),     # dilation: rows that fall outside the output
+])
+def test_npqk_results_in_pieces(lib, K, in_layout, case):
+    N, C, H, W, R, S, st, pad, dil, shift = case
+    x = int8_uniform((N, C, H, W), 1021)
+    w = int8_uniform((K, C, R, S), 1022)
+    bias = int8_uniform((K,), 1023).astype(np.int32) * 311
+    want = [np.ascontiguousarray(v.transpose(0, 2, 3, 1))
+            for v in oracle.conv2d_int8(x, w, st, pad, dil, shift, bias=bias, relu=True)[:2]]
+    xd = to_dev(np.ascontiguousarray(x.transpose(0, 2, 3, 1)) if in_layout else x)
+    for mode in (1, 2, 3):
+        d = lib.make_desc(N, C, H, W, K, R, S, st, pad, dil, shift, in_layout, 1, mode)
+        for e in lib.enumerate_embeddings(d):
+            plan = lib.Plan(d, e.id)
+            plan.set_weights(to_dev(w))
+            plan.set_activation(to_dev(bias), True)
+            y32 = torch.full(want[0].shape, -7777777, dtype=torch.int32, device="cuda") if mode & 1 else None
+            y8 = torch.full(want[0].shape, 77, dtype=torch.int8, device="cuda") if mode & 2 else None
+            ws = torch.zeros(max(16, plan.workspace_bytes()), dtype=torch.uint8, device="cuda")
+            plan.run(xd, y32, y8, ws)
+            torch.cuda.synchronize()
+            assert plan.device_status() == b2c.OK
+            assert y32 is None or np.array_equal(y32.cpu().numpy(), want[0]), (mode, e.id)
+            assert y8 is None or np.array_equal(y8.cpu().numpy(), want[1]), (mode, e.id)
+            plan.destroy()
