@@ -103,6 +103,13 @@ __device__ __forceinline__ bool mbar_wait_sleep(uint32_t bar, uint32_t parity, S
   }
 }
 
+// Debug build: is the unit at this offset in shared memory inside the window of `bytes` bytes at `lo`?
+#ifdef B2C_DEBUG_BOUNDS
+#define B2C_WINDOW_OK(d, site, lo, bytes, at) b2c_dbg_in_range((d).status, site, smem + (lo), bytes, smem + (at), 16)
+#else
+#define B2C_WINDOW_OK(d, site, lo, bytes, at) true
+#endif
+
 // Which raw rows a chunk of grid rows [gr0, gr0 + cnt) needs: those of images n_a .. n_b (none if the chunk lies
 // past the batch: images == 0).
 struct ChunkRows {
@@ -491,7 +498,7 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
               }
               const int f = (g0 + g) * 4;
               if (f + 4 <= f0 || f >= f1) continue;
-              const uint32_t pos0 = (uint32_t)((j0 - first) * pl.pitch + args.pad_w);  // position of raw row 0, column 0
+              const int pos0 = (j0 - first) * pl.pitch + args.pad_w;  // position of raw row 0, column 0: negative if it lies above the window
               const uint32_t a = a_row + (uint32_t)(g * 4) + (uint32_t)(u * 16) * c_step;
               const int left = args.C - u * 16;
               uint32_t px[4][4];
@@ -513,13 +520,17 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
               rotate(px);
               const int h = (int)pl.div_w.div((uint32_t)f);
               const int wcol = f - h * args.W;
-              uint8_t* dst = smem + win_s + (uint32_t)(u * pl.plane_bytes) + (pos0 + (uint32_t)(h * pl.pitch + wcol)) * 16u;
-              const int wrap = (pl.pitch - args.W) * 16;  // W >= 4: at most one row end inside a group
+              // Offset of the group's first pixel in shared memory, in 32 bits that may wrap: where a window starts inside an
+              // image, the group of its first pixel can begin in the row above (30 x 30, segments of 6 rows: pixel 150 is in
+              // the group of 148), before the window.  Only the whole sum, of a pixel that is stored, becomes a pointer.
+              const uint32_t dst = win_s + (uint32_t)(u * pl.plane_bytes) + (uint32_t)(pos0 + h * pl.pitch + wcol) * 16u;
+              const uint32_t wrap = (uint32_t)(pl.pitch - args.W) * 16u;  // W >= 4: at most one row end inside a group
 #pragma unroll
               for (int p = 0; p < 4; ++p) {
                 const int q = p ^ y;
-                if (f + q >= f0 && f + q < f1)
-                  *reinterpret_cast<uint4*>(dst + q * 16 + (wcol + q >= args.W ? wrap : 0)) = make_uint4(px[p][0], px[p][1], px[p][2], px[p][3]);
+                const uint32_t at = dst + (uint32_t)q * 16u + (wcol + q >= args.W ? wrap : 0u);
+                if (f + q >= f0 && f + q < f1 && B2C_WINDOW_OK(args.dbg, 52, win_s, pl.win_bytes, at))
+                  *reinterpret_cast<uint4*>(smem + at) = make_uint4(px[p][0], px[p][1], px[p][2], px[p][3]);
               }
             }
           }

@@ -5,7 +5,8 @@ tensor's range, and the workspace sits between two guard bands.  The GPU test ru
 shapes through every layout variant in that build (a child process, because the binding picks its
 library when it is first loaded): no report, guard bands intact, outputs equal to the oracle's.  It
 then declares every range 64 bytes too short: the accesses to the last elements, which are in range,
-must be reported with their site and skipped, and nothing else may change.
+must be reported with their site and skipped, and nothing else may change.  A second child process runs
+every schedule of the plane kernel at shapes of its own, with the units its builders store checked too.
 """
 import ctypes
 import os
@@ -83,6 +84,46 @@ for e in b2c.enumerate_embeddings(d):
 print("debug build ok: %d runs, shrink reported for variants %s" % (runs, sorted(sites)))
 '''
 
+# Every schedule of the plane kernel, at shapes of each of its forms and ways of staging.
+CHILD_PLANE = r'''
+import numpy as np
+import torch
+import oracle
+import paper_2104_04731_b200 as b2c
+from paper_2104_04731_b200.synth import int8_uniform
+
+assert b2c.debug_build()
+runs = 0
+for N, C, H, W, K, R, S, st, pad, dil in [
+    (100, 48, 30, 30, 64, 3, 3, 1, 1, 1),    # flat groups; segments that start inside an image, where a row does not start on a group
+    (40, 40, 18, 10, 32, 3, 3, 1, 1, 1),     # the same with short rows
+    (300, 18, 14, 14, 16, 3, 3, 1, 1, 1),    # flat groups over whole images
+    (20, 64, 56, 24, 40, 3, 3, 1, 1, 1),     # one tiled copy for all channels
+    (4, 17, 13, 15, 20, 3, 3, 1, 1, 1),      # unaligned words
+    (3, 24, 17, 12, 33, 3, 3, 2, 1, 1),      # stride phases
+    (30, 3, 225, 223, 16, 5, 5, 2, 2, 1),    # row form, stride 2
+    (3, 5, 14, 22, 24, 3, 3, (1, 3), 1, (2, 1)),   # row form, one column per item
+]:
+    x, w = int8_uniform((N, C, H, W), 2011), int8_uniform((K, C, R, S), 2012)
+    ref32, ref8 = oracle.conv2d_int8(x, w, st, pad, dil, 8)
+    d = b2c.make_desc(N, C, H, W, K, R, S, st, pad, dil, 8, out_mode=3)
+    xd, wd = torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda()
+    ids = [e.id for e in b2c.enumerate_embeddings(d) if e.variant == b2c.VARIANT_IM2COL_WINDOW]
+    assert ids, (N, C, H, W, K)
+    for i in ids:
+        plan = b2c.Plan(d, i)
+        y32 = torch.full(ref32.shape, -7777777, dtype=torch.int32, device="cuda")
+        y8 = torch.full(ref8.shape, 77, dtype=torch.int8, device="cuda")
+        plan.set_weights(wd)
+        plan.run(xd, y32, y8, torch.zeros(16, dtype=torch.uint8, device="cuda"))
+        status = plan.device_status()
+        assert status == b2c.OK, (N, C, H, W, K, i, status, plan.debug_info())
+        assert np.array_equal(y32.cpu().numpy(), ref32) and np.array_equal(y8.cpu().numpy(), ref8), (N, C, H, W, K, i)
+        plan.destroy()
+        runs += 1
+print("debug build ok: %d runs" % runs)
+'''
+
 
 def test_debug_library_exports_the_same_interface():
     from paper_2104_04731_b200 import build
@@ -99,5 +140,13 @@ def test_debug_library_exports_the_same_interface():
 def test_five_shapes_through_the_bounds_checked_build():
     env = dict(os.environ, B2C_DEBUG_LIB="1", PYTHONPATH=ROOT + os.pathsep + os.environ.get("PYTHONPATH", ""))
     r = subprocess.run([sys.executable, "-c", CHILD], env=env, cwd=ROOT, capture_output=True, text=True, timeout=900)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
+    assert "debug build ok" in r.stdout
+
+
+@pytest.mark.gpu
+def test_plane_schedules_through_the_bounds_checked_build():
+    env = dict(os.environ, B2C_DEBUG_LIB="1", PYTHONPATH=ROOT + os.pathsep + os.environ.get("PYTHONPATH", ""))
+    r = subprocess.run([sys.executable, "-c", CHILD_PLANE], env=env, cwd=ROOT, capture_output=True, text=True, timeout=900)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
     assert "debug build ok" in r.stdout
