@@ -17,12 +17,15 @@ constexpr int kPackMaxP = 256;  // pixels per tile
 constexpr int kPackSmem = kPackMaxC * (kPackMaxP + 4) + (kPackMaxC / 16) * 16;
 
 // Channel-pack weights: out[k][(r*S + s)][c_pad] = w[k][c][r][s], zeros for c >= C.  A thread forms four consecutive
-// channels of one tap.
-__device__ __forceinline__ void pack_weights_cp_words(const WeightPack& p, unsigned first, unsigned step) {
-  const unsigned words = (unsigned)p.C_pad >> 2, total = (unsigned)p.K * (unsigned)p.RS * words;  // (fewer than 2^31: checked by the host)
-  for (unsigned i = first; i < total; i += step) {
-    const unsigned kt = i / words, c = (i - kt * words) * 4u;
-    const unsigned k = kt / (unsigned)p.RS, tap = kt - k * (unsigned)p.RS;
+// channels of one tap.  Idx: unsigned up to kPackWords32 words (the last index plus a step of the grid then fits), else 64 bits.
+constexpr long long kPackWords32 = 0x7FFFFFFF;
+template <typename Idx>
+__device__ __forceinline__ void pack_weights_cp_words(const WeightPack& p, Idx first, Idx step) {
+  const Idx words = (Idx)p.C_pad >> 2, total = (Idx)p.K * (Idx)p.RS * words;
+  for (Idx i = first; i < total; i += step) {
+    const Idx kt = i / words;
+    const unsigned c = (unsigned)(i - kt * words) * 4u;
+    const Idx k = kt / (Idx)p.RS, tap = kt - k * (Idx)p.RS;
     const int8_t* src = p.w + ((size_t)k * p.C + c) * p.RS + tap;
     uint32_t v = 0;
 #pragma unroll
@@ -36,7 +39,7 @@ __device__ __forceinline__ bool weight_pack_block(const WeightPack& p) {
   const int extra = (int)blockIdx.x - ((int)gridDim.x - p.blocks);
   if (p.blocks == 0 || extra < 0) return false;
   pdl_wait();
-  if (blockIdx.y == 0) pack_weights_cp_words(p, (unsigned)extra * blockDim.x + threadIdx.x, (unsigned)p.blocks * blockDim.x);
+  if (blockIdx.y == 0) pack_weights_cp_words<unsigned>(p, (unsigned)extra * blockDim.x + threadIdx.x, (unsigned)p.blocks * blockDim.x);
   pdl_launch_dependents();
   return true;
 }
@@ -366,9 +369,10 @@ __global__ void __launch_bounds__(kPackThreads) pack_small_images_kernel(const i
   }
 }
 
+template <typename Idx>
 __global__ void __launch_bounds__(256) pack_weights_cp_kernel(WeightPack p) {
   pdl_wait();
-  pack_weights_cp_words(p, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  pack_weights_cp_words<Idx>(p, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
   pdl_launch_dependents();
 }
 
@@ -807,7 +811,9 @@ cudaError_t launch_pack_wait_selftest(int* status, cudaStream_t st) {
 cudaError_t launch_pack_weights_cp(const int8_t* w, int8_t* out, int K, int C, int R, int S, int C_pad,
                                    cudaStream_t st) {
   const WeightPack p = make_weight_pack(w, out, K, C, R * S, C_pad);
-  return launch_pdl(pack_weights_cp_kernel, dim3((unsigned)p.blocks), dim3(kPackThreads), 0, st, p);
+  const bool small = (long long)K * R * S * (C_pad / 4) <= kPackWords32;
+  return launch_pdl(small ? pack_weights_cp_kernel<unsigned> : pack_weights_cp_kernel<unsigned long long>, dim3((unsigned)p.blocks),
+                    dim3(kPackThreads), 0, st, p);
 }
 
 cudaError_t launch_pack_weights_table(const int8_t* w, int8_t* out, int K, int Kg, int cols, const int32_t* table,

@@ -136,6 +136,33 @@ def test_one_shot_packs_weights_with_the_activations(lib, case):
     lib.oneshot_cache_clear()
 
 
+# ---- channel-pack weights of more than 2^32 words: the filter index needs 64 bits -----------------------------------------
+def test_channel_pack_of_weights_beyond_32_bit_indices(lib):
+    """One channel is packed as 32, so 32769 filters of 128 x 128 taps are 2^32 + 131072 words (17 GB) from 0.5 GB."""
+    K, R = 32769, 128
+    assert K * R * R * 8 == 2**32 + 131072
+    if torch.cuda.mem_get_info()[0] < 30 << 30:
+        pytest.skip("needs 30 GB of free device memory")
+    gen = torch.Generator(device="cuda").manual_seed(1071)
+    w = torch.randint(-128, 128, (K, 1, R, R), dtype=torch.int8, device="cuda", generator=gen)
+    x = torch.randint(-128, 128, (1, 1, R, R), dtype=torch.int8, device="cuda", generator=gen)
+    want = torch.mv(w.view(K, R * R).double(), x.view(R * R).double()).to(torch.int32)   # (exact: sums below 2^28)
+    d = lib.make_desc(1, 1, R, R, K, R, R)
+    e = max((e for e in lib.enumerate_embeddings(d) if e.variant == b2c.VARIANT_CP_TMA and e.split_k == 1
+             and e.map_m == b2c.AXIS_NPQ), key=lambda e: e.tile_n)
+    plan = lib.Plan(d, e.id)
+    try:
+        plan.set_weights(w)
+        y32 = torch.full((1, K, 1, 1), -7777777, dtype=torch.int32, device="cuda")
+        ws = torch.zeros(max(16, plan.workspace_bytes()), dtype=torch.uint8, device="cuda")
+        plan.run(x, y32, None, ws)
+        torch.cuda.synchronize()
+        assert plan.device_status() == b2c.OK
+        assert torch.equal(y32.view(K), want)
+    finally:
+        plan.destroy()
+
+
 # ---- NPQK results in 16-byte pieces: exchanged between four lanes (int32 sums), a last run of channels shorter than a tile ----
 @pytest.mark.parametrize("K", [4, 12, 16, 36, 48, 80, 272])
 @pytest.mark.parametrize("in_layout,case", [
