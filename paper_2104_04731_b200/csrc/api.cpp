@@ -1497,15 +1497,14 @@ int b2c_conv2d_int8(int N, int C, int H, int W, int K, int R, int S, int stride,
   // Channel-pack maps: the launch that packs the activations packs the weights as well (a launch costs this call 2.8 us
   // of host time; 64 x 56 x 56, one image: 11.2 -> 8.8 us).
   const bool packs_input = shift_base_variant(p->emb.variant) == B2C_VARIANT_CP_TMA && p->ws_layout_bytes > 0 && p->subs.empty();
-  if (packs_input && !p->fused_pack && aligned16(x) && aligned16(w) && weight_pack_rides(x, N, C, H, W) &&
-      (long long)K * R * S * p->C_pad < 0x7FFFFFFFLL) {
+  const WeightPack ride = make_weight_pack(w, p->w_packed, K, C, R * S, p->C_pad);
+  if (packs_input && !p->fused_pack && aligned16(x) && aligned16(w) && weight_pack_rides(ride, x, N, C, H * W)) {
     cudaStream_t st = (cudaStream_t)cuda_stream;
     p->weights_set = true;
     int rc = check_run_args(p, x, true, y32, y8, true, p->own_ws);
     if (rc != B2C_OK) return rc;
     void* ws = guard_workspace(p, p->own_ws, st, &rc);
     if (rc != B2C_OK) return rc;
-    const WeightPack ride = make_weight_pack(w, p->w_packed, K, C, R * S, p->C_pad);
     rc = run_rewrite(p, x, ws, st, &ride);
     if (rc != B2C_OK) return rc;
     return run_convolve(p, x, y32, y8, ws, st);

@@ -427,10 +427,10 @@ struct WeightPack {
   int K, C, RS, C_pad, blocks;
 };
 WeightPack make_weight_pack(const int8_t* w, int8_t* out, int K, int C, int RS, int C_pad);
-// ride: a weight pack to be done by the same launch (only where weight_pack_rides says so)
+// ride: a weight pack to be done by the same launch (an error where weight_pack_rides says no)
 cudaError_t launch_pack_activations(const int8_t* x, int8_t* out, int N, int C, int H, int W, int C_pad,
                                     cudaStream_t st, int* status, const Dbg& dbg = Dbg(), const WeightPack* ride = nullptr);
-bool weight_pack_rides(const int8_t* x, int N, int C, int H, int W);
+bool weight_pack_rides(const WeightPack& p, const int8_t* x, int N, int C, int HW);
 cudaError_t launch_pack_weights_cp(const int8_t* w, int8_t* out, int K, int C, int R, int S, int C_pad,
                                    cudaStream_t st);
 cudaError_t launch_pack_weights_table(const int8_t* w, int8_t* out, int K, int Kg, int cols, const int32_t* table,

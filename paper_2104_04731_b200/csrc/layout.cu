@@ -755,11 +755,15 @@ WeightPack make_weight_pack(const int8_t* w, int8_t* out, int K, int C, int RS, 
   p.blocks = (int)std::min<long long>(4 * kNumSMs, ((long long)K * RS * (C_pad / 4) + kPackThreads - 1) / kPackThreads);
   return p;
 }
-bool weight_pack_rides(const int8_t* x, int N, int C, int H, int W) {
-  const int HW = H * W;
-  const bool small_images = (reinterpret_cast<uintptr_t>(x) & 15) == 0 && (C % 16) == 0 && C <= 64 && (HW % 4) == 0 && HW <= 256 &&
-                            C * HW <= 12 * 1024 && N >= 8 * kNumSMs;
-  return !small_images;  // (that kernel moves enough that a launch more does not show)
+// Large batches of small images with few channels: several whole images per block (pack_small_images_kernel).
+static bool packs_small_images(const int8_t* x, int N, int C, int HW) {
+  return (reinterpret_cast<uintptr_t>(x) & 15) == 0 && (C % 16) == 0 && C <= 64 && (HW % 4) == 0 && HW <= 256 && C * HW <= 12 * 1024 &&
+         N >= 8 * kNumSMs;
+}
+// Every activation pack takes weights along but the one of small images (it moves enough that a launch more does not
+// show); their words are counted in 32 bits there.
+bool weight_pack_rides(const WeightPack& p, const int8_t* x, int N, int C, int HW) {
+  return !packs_small_images(x, N, C, HW) && (long long)p.K * p.RS * (p.C_pad / 4) <= kPackWords32;
 }
 
 cudaError_t launch_pack_activations(const int8_t* x, int8_t* out, int N, int C, int H, int W, int C_pad,
@@ -768,8 +772,8 @@ cudaError_t launch_pack_activations(const int8_t* x, int8_t* out, int N, int C, 
   const WeightPack wp = ride ? *ride : WeightPack{nullptr, nullptr, 0, 0, 0, 0, 0};
   int CT = C_pad >= 128 ? 128 : 64;
   const bool a16 = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
-  // large batches of small images with few channels: several whole images per block
-  if (a16 && (C % 16) == 0 && C <= 64 && (HW % 4) == 0 && HW <= 256 && C * HW <= 12 * 1024 && N >= 8 * kNumSMs) {
+  if (ride && !weight_pack_rides(*ride, x, N, C, HW)) return cudaErrorInvalidValue;  // (never the previous call's weights)
+  if (packs_small_images(x, N, C, HW)) {
     const int ipb = std::max(1, std::min(16, (24 * 1024) / (C * HW)));
     const size_t smem = (size_t)ipb * C * HW;
     return launch_pdl(pack_small_images_kernel, dim3((unsigned)((N + ipb - 1) / ipb)), dim3(kPackThreads), smem, st, x, out, N, C,
