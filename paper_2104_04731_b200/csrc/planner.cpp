@@ -513,8 +513,10 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
     if (w_bytes > 150 * 1024) continue;
     const int cols = (d.K + tile_n - 1) / tile_n;
     if ((long long)cols * groups > 65535) continue;
+    // (two accumulators at least: with one, a set of epilogue warps that takes every other tile would find its wait
+    // already satisfied by the phase of two tiles before)
     const int nbuf = std::min(kMaxAcc, 512 / per_sm / tile_n);
-    if (nbuf < (per_sm == 2 ? 2 : 1)) continue;
+    if (nbuf < 2) continue;
     int tmem_cols = 32;
     while (tmem_cols < nbuf * tile_n) tmem_cols <<= 1;
     const int places = (int)std::max<long long>(1, (long long)kNumSMs * per_sm / ((long long)cols * groups));
@@ -601,8 +603,7 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
           // one buffer between two roles makes them take turns
           double chain = rs == 1 ? copy + build_lat : std::max(copy, build_lat);
           if (ws == 1) chain = build_lat + std::max(rs == 1 ? copy : 0.0, mma);
-          double steady = std::max(std::max(conc * build, conc * mma), std::max(epi, chain));
-          if (nbuf == 1) steady = std::max(steady, mma + epi);
+          const double steady = std::max(std::max(conc * build, conc * mma), std::max(epi, chain));
           // (a last, partly filled round of segments: the stores of the others' get its share of the memory)
           const double windows = std::max(1.0, (dealt || spi) ? (double)((share + th - 1) / th) * 0.5 * (std::ceil((double)segs / blocks) + (double)segs / blocks) : (double)total_rows / blocks / th);
           const double t = 3000 + copy * (rs == 1 ? first_chunks : 1) + first_lat + first_chunks * 150.0 + mma / tiles + epi + w_bytes / 40.0 * conc +
