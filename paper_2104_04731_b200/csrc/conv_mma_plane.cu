@@ -400,7 +400,12 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
       if (!__all_sync(0xffffffffu, ok)) break;
       const uint32_t win_s = win_off + (uint32_t)(ws * pl.win_bytes);
       if (win > 0 && pl.max_ri > 0) {
-        // the overlap rows: the last max_ri rows of the previous window become the first of this one
+        // The overlap rows: the last max_ri rows of the previous window become the first of this one.
+        // With two buffers a builder that is done with the last window of a segment goes on to the next segment, whose
+        // first window has no rendezvous and is built where a slower builder may still be reading rows to move.  These
+        // are rows th and up, and they arrive there in a second raw chunk, because segments of several windows have
+        // cr == th (the planner lists no others): it lands in the raw stage of the slower builder's window, which
+        // that builder releases after its move.
         const uint32_t prev = win_off + (uint32_t)((pl.win_stages == 1 ? 0 : ws ^ 1) * pl.win_bytes) + (uint32_t)(pl.th * pl.pitch) * 16u;
         ok = rendezvous();  // every builder has finished the previous window
         if (!ok) break;

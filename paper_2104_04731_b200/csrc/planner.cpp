@@ -562,6 +562,7 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
       for (int cr = th; cr <= wr; cr += std::max(1, f.max_ri)) {
         const bool whole_first = cr == wr && (dealt || per_block == 1);
         if (dealt ? !whole_first : (cr != th && !whole_first)) continue;
+        if (share > th && cr != th) continue;  // segments of several windows: the kernel's overlap move relies on it
         // raw staging: rows of at most two images per channel, or whole images when a chunk spans more (or they
         // are small enough not to matter: one copy per image instead of one per channel)
         const int images = (int)std::min<long long>(d.N, cr <= 1 ? 1 : (cr - 2) / f.rpi + 2);
