@@ -89,12 +89,13 @@ typedef struct {
                                       * is an R' x 1 stride-1 convolution, executed as operand shifts over 8 x 16-pixel tiles */
 
 #define B2C_VARIANT_IM2COL_WINDOW 10  /* stencil unroll formed in shared memory, nothing written to HBM between input and result.
-                                      * Small problems (C*R*S bytes a row, NCHW, unit horizontal dilation, rows that are multiples
-                                      * of 16 bytes or whole small images): one tiled TMA copy stages a tile's input patch, builder
-                                      * warps write the swizzled A rows.  Large ones (C <= 96, NCHW, rows of any width, any stride
-                                      * and dilation): the input becomes planes of 16-byte units in shared memory and a tap is a
-                                      * start address into them.  Such a problem is listed once per schedule worth timing (entries
-                                      * that differ in no field but the id).  Weights stay resident in shared memory */
+                                      * C*R*S bytes a row, NCHW, unit horizontal dilation, rows that are multiples of 16 bytes or
+                                      * whole small images: one tiled TMA copy stages a tile's input patch, builder warps write
+                                      * the swizzled A rows.  Large problems (C <= 96, NCHW, rows of any width, any stride and
+                                      * dilation): the input becomes planes of 16-byte units in shared memory and a tap is a
+                                      * start address into them; listed once per schedule worth timing (entries that may differ in
+                                      * no field but the id), beside the first form where both apply.
+                                      * Weights stay resident in shared memory */
 
 typedef struct {
   int32_t id;       /* index in the enumeration for this descriptor; pass to b2c_plan_create      */

@@ -417,23 +417,16 @@ void fill_common_args(b2c_plan* p) {
 }
 
 // The embeddings of g, numbered; every variant but the channel pack goes through the stencil lookup table.
-void enumerate_legal(const Geom& g, std::vector<b2c_embedding>* all) {
+void enumerate_legal(const Geom& g, std::vector<Candidate>* all) {
   enumerate_embeddings(g, all);
   if (!table_variant_legal(g))
-    all->erase(std::remove_if(all->begin(), all->end(), [](const b2c_embedding& e) { return e.variant != B2C_VARIANT_CP_TMA; }),
+    all->erase(std::remove_if(all->begin(), all->end(), [](const Candidate& e) { return e.variant != B2C_VARIANT_CP_TMA; }),
                all->end());
   for (size_t i = 0; i < all->size(); ++i) (*all)[i].id = (int)i;
 }
 
-// Embeddings that differ only in the schedule of the plane kernel share all their fields: which of them entry idx of
-// an enumeration is.
-int schedule_of(const std::vector<b2c_embedding>& all, int idx) {
-  int nth = 0;
-  for (int i = 0; i < idx; ++i) nth += all[i].variant == all[idx].variant && all[i].tile_n == all[idx].tile_n ? 1 : 0;
-  return all[idx].variant == B2C_VARIANT_IM2COL_WINDOW ? nth : 0;
-}
-
-int create_plan_for(const Geom& g, const b2c_embedding& emb, int nth, b2c_plan** out, int group_count = 1) {
+// schedule: that of the plane kernel if it is the one to run the embedding, else -1.
+int create_plan_for(const Geom& g, const b2c_embedding& emb, int schedule, b2c_plan** out, int group_count = 1) {
   b2c_plan* p = new (std::nothrow) b2c_plan();
   if (!p) return B2C_E_INVALID_ARG;
   p->g = g;
@@ -449,9 +442,8 @@ int create_plan_for(const Geom& g, const b2c_embedding& emb, int nth, b2c_plan**
   if (cudaMemset(p->status, 0, kStatusWords * sizeof(int)) != cudaSuccess) return fail(B2C_E_CUDA);
   std::vector<uint64_t> mma;
   std::vector<int32_t> wsrc;
-  const bool plane = emb.variant == B2C_VARIANT_IM2COL_WINDOW && (group_count > 1 || plane_wanted(g)) &&
-                     plane_plan(g, group_count, emb.tile_n, nth, &p->plane, &mma, &wsrc);
-  if (group_count > 1 && emb.variant == B2C_VARIANT_IM2COL_WINDOW && !plane) return fail(B2C_E_UNSUPPORTED);
+  const bool plane = schedule >= 0;
+  if (plane && !plane_plan(g, group_count, schedule, &p->plane, &mma, &wsrc)) return fail(B2C_E_UNSUPPORTED);
   if (is_tma_view_variant(emb.variant)) {
     if (!tma_view_for(g, emb.variant, &p->view)) return fail(B2C_E_UNSUPPORTED);
     const TmaView& v = p->view;
@@ -751,7 +743,7 @@ int b2c_enumerate(const b2c_conv_desc* desc, b2c_embedding* out, int32_t cap, in
   Geom g;
   int rc = resolve_geom(desc, &g);
   if (rc != B2C_OK) return rc;
-  std::vector<b2c_embedding> all;
+  std::vector<Candidate> all;
   enumerate_legal(g, &all);
   *count = (int32_t)all.size();
   for (int i = 0; i < cap && i < (int)all.size(); ++i) out[i] = all[i];
@@ -764,7 +756,7 @@ int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_
   Geom g;
   int rc = resolve_geom(desc, &g);
   if (rc != B2C_OK) return rc;
-  std::vector<b2c_embedding> all;
+  std::vector<Candidate> all;
   enumerate_legal(g, &all);
   if (all.empty()) return B2C_E_UNSUPPORTED;
   if (policy_or_id < B2C_POLICY_AUTO_TIMED_CONCURRENT) return B2C_E_INVALID_ARG;
@@ -772,7 +764,7 @@ int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_
   if (policy_or_id != B2C_POLICY_AUTO_TIMED && policy_or_id != B2C_POLICY_AUTO_TIMED_CONCURRENT) {
     int idx = pick_by_policy(all, policy_or_id);
     if (idx < 0) return B2C_E_INVALID_ARG;
-    return create_plan_for(g, all[idx], schedule_of(all, idx), out);
+    return create_plan_for(g, all[idx], all[idx].schedule, out);
   }
   // Timed selection (Section 6.1: the best candidates by the overhead metric are tuned and the
   // fastest is kept).  All schedules of the five lowest-overhead (axis map, layout variant)
@@ -780,11 +772,11 @@ int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_
   cudaStream_t st = (cudaStream_t)cuda_stream;
   // (Variants of one family count as one candidate: a view and its shift execution, the row unrolls.)
   std::vector<int> groups;
-  for (const b2c_embedding& e : all)
+  for (const Candidate& e : all)
     if (std::find(groups.begin(), groups.end(), variant_family(e.variant)) == groups.end() && groups.size() < 5)
       groups.push_back(variant_family(e.variant));
   size_t ws_max = 0;
-  for (const b2c_embedding& e : all) ws_max = std::max(ws_max, (size_t)e.workspace_bytes);
+  for (const Candidate& e : all) ws_max = std::max(ws_max, (size_t)e.workspace_bytes);
   int8_t *x = nullptr, *w = nullptr;
   LaneBuffers lane[kMaxLanes] = {};
   auto cleanup = [&]() {
@@ -817,7 +809,7 @@ int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_
     // A candidate that cannot be built or run (a tensor map the driver refuses, an allocation that
     // fails, a device wait that expires) is left out of the selection; the others are still timed.
     b2c_plan* p = nullptr;
-    rc = create_plan_for(g, all[i], schedule_of(all, (int)i), &p);
+    rc = create_plan_for(g, all[i], all[i].schedule, &p);
     if (rc == B2C_OK) rc = b2c_plan_set_weights(p, w, st);
     if (rc == B2C_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = B2C_E_CUDA;
     float us = -1;
@@ -836,11 +828,11 @@ int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_
   }
   cleanup();
   if (best < 0) return first_error != B2C_OK ? first_error : B2C_E_UNSUPPORTED;
-  return create_plan_for(g, all[best], schedule_of(all, best), out);
+  return create_plan_for(g, all[best], all[best].schedule, out);
 }
 
 // Group plan that runs all groups in one launch, `merge` consecutive ones as one group sg with embedding emb.
-static int create_grouped_plan(const b2c_conv_desc* desc, int groups, int merge, const Geom& sg, const b2c_embedding& emb, int nth,
+static int create_grouped_plan(const b2c_conv_desc* desc, int groups, int merge, const Geom& sg, const b2c_embedding& emb, int schedule,
                                b2c_plan** out) {
   b2c_plan* p = new (std::nothrow) b2c_plan();
   if (!p) return B2C_E_INVALID_ARG;
@@ -859,7 +851,7 @@ static int create_grouped_plan(const b2c_conv_desc* desc, int groups, int merge,
   }
   // one sub-plan runs all groups in one launch (the group is a grid axis of the kernel)
   b2c_plan* sub = nullptr;
-  const int rc = create_plan_for(sg, emb, nth, &sub, groups / merge);
+  const int rc = create_plan_for(sg, emb, schedule, &sub, groups / merge);
   if (rc != B2C_OK) {
     b2c_plan_destroy(p);
     return rc;
@@ -904,7 +896,7 @@ int b2c_plan_create_grouped(const b2c_conv_desc* desc, int32_t groups, b2c_plan*
   if (rc != B2C_OK) return rc;
   // Embedding of every group: the lowest-overhead unsplit stencil unroll formed inside the kernel
   // (staged window where it fits, else the gather); both read their channel slice of x in place.
-  std::vector<b2c_embedding> all;
+  std::vector<Candidate> all;
   enumerate_embeddings(sg, &all);
   // (the staged window before the gather: it builds the operand from shared memory with word loads; of
   // one variant's schedules the one whose column tile holds a whole group, else the widest)
@@ -922,7 +914,7 @@ int b2c_plan_create_grouped(const b2c_conv_desc* desc, int32_t groups, b2c_plan*
         (pick < 0 || better(all[i], all[pick])))
       pick = (int)i;
   if (pick < 0) return B2C_E_UNSUPPORTED;
-  return create_grouped_plan(desc, groups, merge, sg, all[pick], 0, out);
+  return create_grouped_plan(desc, groups, merge, sg, all[pick], -1, out);
 }
 
 int b2c_plan_create_grouped_timed(const b2c_conv_desc* desc, int32_t groups, void* cuda_stream, b2c_plan** out) {
@@ -971,7 +963,7 @@ int b2c_plan_create_grouped_timed(const b2c_conv_desc* desc, int32_t groups, voi
       if (resolve_geom(&sd, &sg) != B2C_OK) continue;
       for (int nth = 0; nth < 10; ++nth) {
         PlaneArgs pl;
-        if (!plane_plan(sg, groups / m, 0, nth, &pl)) break;
+        if (!plane_plan(sg, groups / m, nth, &pl)) break;
         b2c_embedding e;
         std::memset(&e, 0, sizeof(e));
         e.map_m = B2C_AXIS_NPQ;
@@ -984,14 +976,9 @@ int b2c_plan_create_grouped_timed(const b2c_conv_desc* desc, int32_t groups, voi
         e.o_mac = (int64_t)pl.total_rows * pl.pitch * pl.cols * pl.tile_n * pl.num_mma * kMmaK * (groups / m) - g.Mg * desc->K * cg * desc->R * desc->S;
         e.o_data = (int64_t)(groups / m) * pl.cols * pl.w_bytes - (int64_t)w_bytes;
         e.device_us = -1.0f;
-        int same = 0;  // schedules with this column tile before this one
-        for (int i = 0; i < nth; ++i) {
-          PlaneArgs before;
-          same += plane_plan(sg, groups / m, 0, i, &before) && before.tile_n == pl.tile_n ? 1 : 0;
-        }
         b2c_plan* q = nullptr;
         float t = -1;
-        if (create_grouped_plan(desc, groups, m, sg, e, same, &q) == B2C_OK && timed(q, &t) && t < us) {
+        if (create_grouped_plan(desc, groups, m, sg, e, nth, &q) == B2C_OK && timed(q, &t) && t < us) {
           b2c_plan_destroy(inplace);
           inplace = q;
           us = t;

@@ -344,8 +344,12 @@ int round_up(int v, int m);
 int cp_channel_pad(int C);           // channels after Pad for the channel-pack map
 int cp_block_bytes(int C_pad);       // reduction bytes per block for the channel-pack map
 int im2col_k_pad(int Kg);            // padded reduction length for the stencil-unroll maps
-void enumerate_embeddings(const Geom& g, std::vector<b2c_embedding>* out);
-int pick_by_policy(const std::vector<b2c_embedding>& all, int policy);  // index or -1
+// An embedding and, for the window unroll, which kernel runs it.
+struct Candidate : b2c_embedding {
+  int schedule;  // plane kernel: index of its schedule (plane_plan); -1: any other kernel, the window kernel among them
+};
+void enumerate_embeddings(const Geom& g, std::vector<Candidate>* out);
+int pick_by_policy(const std::vector<Candidate>& all, int policy);  // index or -1
 size_t workspace_bytes_for(const Geom& g, int variant, int tile_n, int split_k, bool swap = false);
 inline bool is_swapped(const b2c_embedding& e) { return e.map_m == B2C_AXIS_K; }
 // A split reduction of 2, 4 or 8 slices whose tile is wide enough runs as a thread-block cluster:
@@ -395,13 +399,11 @@ struct WindowTile {
 };
 bool window_tile_geom(const Geom& g, WindowTile* wt);
 
-// The nth schedule of the plane kernel with column tile tile_n (0: any) for `groups` groups of the convolution g (1: g
-// itself), the lowest estimate first; false if there is none.  With table / wsrc: the MMA list (see
-// PlaneArgs::mma_table) and, per packed weight byte of one channel (32 per MMA), its index in a filter or -1.
-bool plane_plan(const Geom& g, int groups, int tile_n, int nth, PlaneArgs* pl, std::vector<uint64_t>* table = nullptr,
+// The nth schedule of the plane kernel for `groups` groups of the convolution g (1: g itself), the lowest estimate
+// first; false if there is none.  With table / wsrc: the MMA list (see PlaneArgs::mma_table) and, per packed weight byte
+// of one channel (32 per MMA), its index in a filter or -1.
+bool plane_plan(const Geom& g, int groups, int nth, PlaneArgs* pl, std::vector<uint64_t>* table = nullptr,
                 std::vector<int32_t>* wsrc = nullptr);
-// Which of the two kernels runs the window unroll of g: true for the plane kernel, where it applies.
-bool plane_wanted(const Geom& g);
 
 // --- tma.cpp -----------------------------------------------------------------------------------
 // Tensor-map encoders obtained through cudaGetDriverEntryPoint (no link-time libcuda dependency).

@@ -708,20 +708,14 @@ bool plane_choices(const Geom& g, int groups, PlaneForm* form, std::vector<Plane
 
 }  // namespace
 
-bool plane_plan(const Geom& g, int groups, int tile_n, int nth, PlaneArgs* pl, std::vector<uint64_t>* table, std::vector<int32_t>* wsrc) {
+bool plane_plan(const Geom& g, int groups, int nth, PlaneArgs* pl, std::vector<uint64_t>* table, std::vector<int32_t>* wsrc) {
   const b2c_conv_desc& d = g.d;
   std::memset(pl, 0, sizeof(*pl));
   PlaneForm f;
   std::vector<PlaneChoice> list;
   if (!plane_choices(g, groups, &f, &list)) return false;
-  bool found = false;
-  for (const PlaneChoice& c : list)
-    if ((tile_n == 0 || c.pl.tile_n == tile_n) && nth-- == 0) {
-      *pl = c.pl;
-      found = true;
-      break;
-    }
-  if (!found) return false;
+  if (nth < 0 || nth >= (int)list.size()) return false;
+  *pl = list[nth].pl;
   const int HW = d.H * d.W;
   pl->runw = f.runw;
   pl->sh = d.stride_h;
@@ -778,18 +772,18 @@ bool plane_plan(const Geom& g, int groups, int tile_n, int nth, PlaneArgs* pl, s
 
 // The plane kernel builds every input row once per window and needs windows of several tiles to pay for the rows the
 // taps reach below; the window kernel's tiles are independent of each other and spread a small problem over more
-// blocks.  7x7 stride 2 of 3 x 224 x 224, 98 tiles an image: 4 images 6.9 us (window) against 9.5, 16 images 14.3
-// against 15.3, 100 images 72 against 65.
-bool plane_wanted(const Geom& g) {
-  WindowTile wt;
-  return !(window_tile_geom(g, &wt) && wt.mtot <= (long long)kPlaneMinTiles * kTileM);
-}
+// blocks.  Up to kPlaneMinTiles accumulator tiles a problem that the window kernel takes is listed for it alone; above,
+// both are listed and the timed selection decides: which is faster depends on more than the number of tiles (7x7
+// stride 2 of 3 x 224 x 224, 98 tiles an image: 16 images 14.3 us by the window kernel, 15.3 by this one, 100 images 72
+// and 65; but 3x3 stride 2 of 12 x 36 x 256, 159 images, 64 channels, 2862 tiles, 31.5 and 42.2, and 3x3 of
+// 8 x 154 x 48, 158 images, 24 channels, 9480 tiles, 96 and 119).
+static bool plane_wanted(const WindowTile* wt) { return wt == nullptr || wt->mtot > (long long)kPlaneMinTiles * kTileM; }
 
-static void add(std::vector<b2c_embedding>* out, const Geom& g, int variant, int tile_n, int split_k,
-                bool swap = false, int tile_m = kTileM, long long plane_rows = 0, int plane_k = 0) {
+static void add(std::vector<Candidate>* out, const Geom& g, int variant, int tile_n, int split_k,
+                bool swap = false, int tile_m = kTileM, int schedule = -1, long long plane_rows = 0, int plane_k = 0) {
   const b2c_conv_desc& d = g.d;
-  b2c_embedding e;
-  std::memset(&e, 0, sizeof(e));
+  Candidate e = {};
+  e.schedule = schedule;
   e.map_m = swap ? B2C_AXIS_K : B2C_AXIS_NPQ;
   e.map_n = swap ? B2C_AXIS_NPQ : B2C_AXIS_K;
   e.variant = variant;
@@ -822,7 +816,7 @@ static void add(std::vector<b2c_embedding>* out, const Geom& g, int variant, int
     int K_pad = variant_k_pad(g, variant);
     k_issued = K_pad;
     WindowTile wt;
-    if (plane_rows > 0) {
+    if (schedule >= 0) {
       M_pad = (plane_rows + kTileM - 1) / kTileM * kTileM;  // plane kernel: grid positions, the taps' overhang among them
       K_pad = plane_k;
       k_issued = K_pad;
@@ -847,7 +841,7 @@ static void add(std::vector<b2c_embedding>* out, const Geom& g, int variant, int
   out->push_back(e);
 }
 
-void enumerate_embeddings(const Geom& g, std::vector<b2c_embedding>* out) {
+void enumerate_embeddings(const Geom& g, std::vector<Candidate>* out) {
   out->clear();
   const b2c_conv_desc& d = g.d;
   // Tile widths: every MMA N extent up to the first one that covers K.
@@ -866,16 +860,15 @@ void enumerate_embeddings(const Geom& g, std::vector<b2c_embedding>* out) {
     if (variant == B2C_VARIANT_IM2COL_WINDOW) {
       // window kernel: one schedule, all output channels in one column tile (the weights are resident), no split
       WindowTile wt;
+      const bool window = window_tile_geom(g, &wt);
+      if (window) add(out, g, variant, wt.tile_n, 1);
+      // plane kernel: one entry per schedule
       PlaneForm form;
       std::vector<PlaneChoice> plane;
-      if (plane_wanted(g) && plane_choices(g, 1, &form, &plane)) {
-        // one entry per schedule of the plane kernel
-        for (const PlaneChoice& c : plane)
-          add(out, g, variant, c.pl.tile_n, 1, false, kTileM, (long long)g.d.N * form.rpi * form.pitch,
+      if (plane_wanted(window ? &wt : nullptr) && plane_choices(g, 1, &form, &plane))
+        for (int i = 0; i < (int)plane.size(); ++i)
+          add(out, g, variant, plane[i].pl.tile_n, 1, false, kTileM, i, (long long)g.d.N * form.rpi * form.pitch,
               ((int)form.units.size() + 1) / 2 * kMmaK);
-      } else if (window_tile_geom(g, &wt)) {
-        add(out, g, variant, wt.tile_n, 1);
-      }
       continue;
     }
     int num_kb;
@@ -927,13 +920,13 @@ void enumerate_embeddings(const Geom& g, std::vector<b2c_embedding>* out) {
       }
     }
   }
-  std::stable_sort(out->begin(), out->end(), [](const b2c_embedding& a, const b2c_embedding& b) {
+  std::stable_sort(out->begin(), out->end(), [](const Candidate& a, const Candidate& b) {
     return a.o_mac + a.o_data < b.o_mac + b.o_data;
   });
   for (size_t i = 0; i < out->size(); ++i) (*out)[i].id = (int)i;
 }
 
-int pick_by_policy(const std::vector<b2c_embedding>& all, int policy) {
+int pick_by_policy(const std::vector<Candidate>& all, int policy) {
   if (all.empty()) return -1;
   if (policy >= 0) return policy < (int)all.size() ? policy : -1;
   if (policy == B2C_POLICY_MIN_WORKSPACE) {

@@ -196,3 +196,21 @@ def test_fault_injection_hook_arms_and_disarms(lib):
     assert b2c.load().b2c_test_fail_nth_encode(-1) == b2c.E_INVALID_ARG
     b2c.test_fail_nth_encode(3)
     b2c.test_fail_nth_encode(0)
+
+
+@pytest.mark.parametrize("shape", [
+    # N, C, H, W, K, R, S, stride, pad: more than 2500 accumulator tiles, input the window kernel takes
+    (636, 2, 24, 69, 28, 3, 3, 1, 1),
+    (2637, 1, 16, 84, 21, 3, 3, 1, 1),
+    (1527, 4, 48, 35, 13, 1, 1, 2, 0),
+    (1391, 2, 44, 12, 14, 3, 3, 1, 1),
+])
+def test_window_kernel_is_listed_beside_the_plane_kernel(lib, shape):
+    """The plane kernel's schedules do not replace the window kernel: it has the lowest overhead here."""
+    N, C, H, W, K, R, S, stride, pad = shape
+    es = b2c.enumerate_embeddings(b2c.make_desc(N, C, H, W, K, R, S, stride, pad))
+    tile_n = max(16, 1 << (K - 1).bit_length())
+    assert (es[0].variant, es[0].tile_n) == (b2c.VARIANT_IM2COL_WINDOW, tile_n)
+    issued = es[0].o_mac + N * K * C * R * S * int.__mul__(*b2c.out_shape(b2c.make_desc(N, C, H, W, K, R, S, stride, pad)))
+    assert issued % (tile_n * ((C * R * ((S + 3) // 4 * 4) + 31) // 32 * 32)) == 0   # whole words of every filter row
+    assert sum(e.variant == b2c.VARIANT_IM2COL_WINDOW for e in es) > 1
