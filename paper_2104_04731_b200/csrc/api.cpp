@@ -973,7 +973,7 @@ int b2c_plan_create_grouped_timed(const b2c_conv_desc* desc, int32_t groups, voi
         e.tile_m = kTileM;
         e.tile_n = pl.tile_n;
         e.split_k = 1;
-        e.o_mac = (int64_t)pl.total_rows * pl.pitch * pl.cols * pl.tile_n * pl.num_mma * kMmaK * (groups / m) - g.Mg * desc->K * cg * desc->R * desc->S;
+        e.o_mac = plane_rows_issued(sg, pl) * pl.cols * pl.tile_n * pl.num_mma * kMmaK * (groups / m) - g.Mg * desc->K * cg * desc->R * desc->S;
         e.o_data = (int64_t)(groups / m) * pl.cols * pl.w_bytes - (int64_t)w_bytes;
         e.device_us = -1.0f;
         b2c_plan* q = nullptr;

@@ -404,6 +404,7 @@ bool window_tile_geom(const Geom& g, WindowTile* wt);
 // of one channel (32 per MMA), its index in a filter or -1.
 bool plane_plan(const Geom& g, int groups, int nth, PlaneArgs* pl, std::vector<uint64_t>* table = nullptr,
                 std::vector<int32_t>* wsrc = nullptr);
+long long plane_rows_issued(const Geom& g, const PlaneArgs& pl);
 
 // --- tma.cpp -----------------------------------------------------------------------------------
 // Tensor-map encoders obtained through cudaGetDriverEntryPoint (no link-time libcuda dependency).

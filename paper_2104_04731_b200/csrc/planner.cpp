@@ -611,6 +611,8 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
                            (windows - 1) * steady + (dealt ? 0.0 : (double)(segs_per_block - 1) * f.max_ri / th * conc * build);
           if (best >= 0 && t >= best * 0.999) continue;
           best = t;
+          pl->pitch = f.pitch;
+          pl->total_rows = (int)total_rows;
           pl->tile_n = tile_n;
           pl->cols = cols;
           pl->tmem_cols = tmem_cols;
@@ -726,9 +728,7 @@ bool plane_plan(const Geom& g, int groups, int nth, PlaneArgs* pl, std::vector<u
   std::memcpy(pl->row_phase, f.row_phase, sizeof(pl->row_phase));
   std::memcpy(pl->col_phase, f.col_phase, sizeof(pl->col_phase));
   pl->planes = f.planes;
-  pl->pitch = f.pitch;
   pl->rpi = f.rpi;
-  pl->total_rows = d.N * f.rpi;
   pl->max_ri = f.max_ri;
   pl->num_mma = ((int)f.units.size() + 1) / 2;
   pl->gpr = f.runw ? (f.pitch + f.qb - 1) / f.qb : (d.W + 3) / 4;
@@ -779,6 +779,17 @@ bool plane_plan(const Geom& g, int groups, int nth, PlaneArgs* pl, std::vector<u
 // 8 x 154 x 48, 158 images, 24 channels, 9480 tiles, 96 and 119).
 static bool plane_wanted(const WindowTile* wt) { return wt == nullptr || wt->mtot > (long long)kPlaneMinTiles * kTileM; }
 
+// Accumulator rows that a schedule of the plane kernel issues: whole tiles of every window, the taps' overhang among
+// them (see seg_rows and window_span in conv_mma_plane.cu).
+long long plane_rows_issued(const Geom& g, const PlaneArgs& pl) {
+  auto tiles = [&](long long rows) {  // of a segment
+    const long long full = ((long long)pl.th * pl.pitch + kTileM - 1) / kTileM;
+    return rows / pl.th * full + (rows % pl.th * pl.pitch + kTileM - 1) / kTileM;
+  };
+  const long long all = pl.spi > 0 ? g.P : pl.total_rows;  // rows that are cut into segments: an image's, or the batch's
+  return ((all / pl.seg_rows) * tiles(pl.seg_rows) + tiles(all % pl.seg_rows)) * (pl.spi > 0 ? g.d.N : 1) * kTileM;
+}
+
 static void add(std::vector<Candidate>* out, const Geom& g, int variant, int tile_n, int split_k,
                 bool swap = false, int tile_m = kTileM, int schedule = -1, long long plane_rows = 0, int plane_k = 0) {
   const b2c_conv_desc& d = g.d;
@@ -817,7 +828,7 @@ static void add(std::vector<Candidate>* out, const Geom& g, int variant, int til
     k_issued = K_pad;
     WindowTile wt;
     if (schedule >= 0) {
-      M_pad = (plane_rows + kTileM - 1) / kTileM * kTileM;  // plane kernel: grid positions, the taps' overhang among them
+      M_pad = plane_rows;
       K_pad = plane_k;
       k_issued = K_pad;
     } else if (variant == B2C_VARIANT_IM2COL_WINDOW && window_tile_geom(g, &wt)) {
@@ -867,7 +878,7 @@ void enumerate_embeddings(const Geom& g, std::vector<Candidate>* out) {
       std::vector<PlaneChoice> plane;
       if (plane_wanted(window ? &wt : nullptr) && plane_choices(g, 1, &form, &plane))
         for (int i = 0; i < (int)plane.size(); ++i)
-          add(out, g, variant, plane[i].pl.tile_n, 1, false, kTileM, i, (long long)g.d.N * form.rpi * form.pitch,
+          add(out, g, variant, plane[i].pl.tile_n, 1, false, kTileM, i, plane_rows_issued(g, plane[i].pl),
               ((int)form.units.size() + 1) / 2 * kMmaK);
       continue;
     }

@@ -214,3 +214,15 @@ def test_window_kernel_is_listed_beside_the_plane_kernel(lib, shape):
     issued = es[0].o_mac + N * K * C * R * S * int.__mul__(*b2c.out_shape(b2c.make_desc(N, C, H, W, K, R, S, stride, pad)))
     assert issued % (tile_n * ((C * R * ((S + 3) // 4 * 4) + 31) // 32 * 32)) == 0   # whole words of every filter row
     assert sum(e.variant == b2c.VARIANT_IM2COL_WINDOW for e in es) > 1
+
+
+def test_overhead_of_plane_schedules_counts_the_rows_they_issue(lib):
+    """Schedules with windows of different heights round to whole accumulator tiles differently, and say so in o_mac."""
+    N, C, H, W, K = 315, 64, 56, 56, 64
+    es = [e for e in b2c.enumerate_embeddings(b2c.make_desc(N, C, H, W, K, 3, 3, 1, 1)) if e.variant == b2c.VARIANT_IM2COL_WINDOW]
+    rows = set()
+    for e in es:
+        issued = e.o_mac + N * K * H * W * C * 9
+        assert e.tile_n == 64 and issued % (128 * 64 * C * 9) == 0     # 9 taps of 64 channels: 18 MMAs of 32, nothing padded
+        rows.add(issued // (64 * C * 9))
+    assert len(rows) > 1 and min(rows) >= N * H * (W + 1)              # a grid row has a column of padding more than an image's
