@@ -770,10 +770,13 @@ int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_
   // fastest is kept).  All schedules of the five lowest-overhead (axis map, layout variant)
   // groups are run on scratch tensors.
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  // (Variants of one family count as one candidate: a view and its shift execution, the row unrolls.)
+  // (Variants of one family count as one candidate: a view and its shift execution, the row unrolls.  The plane kernel's
+  // schedules are run beside the five: counted as a family they pushed another out, 1.46 x slower for 8 images of
+  // 93 x 93 x 9 -> 364, 3x3 stride 2, whose space-to-depth form takes 9.4 us and the plane kernel 13.7; or were not run
+  // themselves.)
   std::vector<int> groups;
   for (const Candidate& e : all)
-    if (std::find(groups.begin(), groups.end(), variant_family(e.variant)) == groups.end() && groups.size() < 5)
+    if (e.schedule < 0 && groups.size() < 5 && std::find(groups.begin(), groups.end(), variant_family(e.variant)) == groups.end())
       groups.push_back(variant_family(e.variant));
   size_t ws_max = 0;
   for (const Candidate& e : all) ws_max = std::max(ws_max, (size_t)e.workspace_bytes);
@@ -805,7 +808,7 @@ int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_
   float best_us = 0;
   int first_error = B2C_OK;
   for (size_t i = 0; i < all.size(); ++i) {
-    if (std::find(groups.begin(), groups.end(), variant_family(all[i].variant)) == groups.end()) continue;
+    if (all[i].schedule < 0 && std::find(groups.begin(), groups.end(), variant_family(all[i].variant)) == groups.end()) continue;
     // A candidate that cannot be built or run (a tensor map the driver refuses, an allocation that
     // fails, a device wait that expires) is left out of the selection; the others are still timed.
     b2c_plan* p = nullptr;

@@ -85,6 +85,20 @@ def test_plane_kernel_reads_the_last_incomplete_16_bytes(lib):
 
 
 @pytest.mark.parametrize("case", [
+    # N, C, H, W, K, R, stride, pad: space to depth is a fifth or more faster than the plane kernel, and has a higher overhead
+    (8, 93, 93, 9, 364, 3, 2, 1),
+    (3, 96, 28, 14, 192, 3, 2, 1),
+])
+def test_timed_selection_runs_the_other_families_beside_the_plane_kernel(lib, case):
+    N, C, H, W, K, R, stride, pad = case
+    d = lib.make_desc(N, C, H, W, K, R, R, stride, pad)
+    assert any(e.variant == b2c.VARIANT_IM2COL_WINDOW for e in lib.enumerate_embeddings(d))
+    plan = lib.Plan(d, b2c.POLICY_AUTO_TIMED)
+    assert plan.info().variant == b2c.VARIANT_SPACE_TO_DEPTH
+    plan.destroy()
+
+
+@pytest.mark.parametrize("case", [
     # N, C, H, W, K, groups, R, shift, out_mode
     (40, 64, 28, 28, 64, 64, 3, 5, 3),       # depth-wise: groups merged 16 at a time and more
     (30, 96, 17, 23, 96, 96, 3, 5, 1),       # odd image: every group's channel slice at another alignment
