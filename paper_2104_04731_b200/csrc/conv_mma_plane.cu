@@ -265,7 +265,8 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
       const uint32_t raw = raw_off + (uint32_t)(s * pl.raw_bytes) + kPlaneMargin;
       if (pl.box_bytes > 0) {
         // one tiled copy: box_bytes of every channel of the image from the 16-byte boundary before row lo_a on
-        if (r.rows_a > 0) {
+        if (r.rows_a > 0 && B2C_X_OK(args.dbg, 53, xg + (size_t)r.n_a * args.x_stride_n + r.lo_a * args.W,
+                                     (long long)(args.C - 1) * HW + r.rows_a * args.W)) {
           mbar_arrive_expect_tx(full, (uint32_t)(args.C * pl.box_bytes), leader);
           tma_load_2d(smem_base + raw, &tmap_x, ((r.lo_a * args.W) & ~15) >> 2, r.n_a * pl.img_channels + grp * args.C, full, leader);
         } else {

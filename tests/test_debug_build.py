@@ -2,7 +2,7 @@
 
 It stands in for a memory checker: every address a kernel computes by hand is tested against its
 tensor's range, and the workspace sits between two guard bands.  The GPU test runs the five benchmark
-shapes through every layout variant in that build (a child process, because the binding picks its
+shapes through every layout variant, and every schedule of the window unroll, in that build (a child process, because the binding picks its
 library when it is first loaded): no report, guard bands intact, outputs equal to the oracle's.  It
 then declares every range 64 bytes too short: the accesses to the last elements, which are in range,
 must be reported with their site and skipped, and nothing else may change.  A second child process runs
@@ -34,7 +34,7 @@ for cfg in CONFIGS:
     xd, wd = torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda()
     seen = set()
     for e in b2c.enumerate_embeddings(d):
-        key = (e.variant, e.tile_m, e.map_m, min(e.split_k, 2))
+        key = (e.variant, e.tile_m, e.map_m, min(e.split_k, 2), e.id if e.variant == b2c.VARIANT_IM2COL_WINDOW else 0)
         if key in seen:
             continue
         seen.add(key)
@@ -118,6 +118,15 @@ for N, C, H, W, K, R, S, st, pad, dil in [
         plan.run(xd, y32, y8, torch.zeros(16, dtype=torch.uint8, device="cuda"))
         status = plan.device_status()
         assert status == b2c.OK, (N, C, H, W, K, i, status, plan.debug_info())
+        assert np.array_equal(y32.cpu().numpy(), ref32) and np.array_equal(y8.cpu().numpy(), ref8), (N, C, H, W, K, i)
+        # every range declared 64 bytes short: the last input rows and results are reported, and clean again afterwards
+        b2c.test_shrink_checked_ranges(64)
+        plan.run(xd, y32, y8, torch.zeros(16, dtype=torch.uint8, device="cuda"))
+        status = plan.device_status()
+        b2c.test_shrink_checked_ranges(0)
+        assert status == b2c.E_BOUNDS and plan.debug_info()[0] > 0, (N, C, H, W, K, i, status)
+        plan.run(xd, y32, y8, torch.zeros(16, dtype=torch.uint8, device="cuda"))
+        assert plan.device_status() == b2c.OK
         assert np.array_equal(y32.cpu().numpy(), ref32) and np.array_equal(y8.cpu().numpy(), ref8), (N, C, H, W, K, i)
         plan.destroy()
         runs += 1
