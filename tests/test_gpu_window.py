@@ -53,8 +53,8 @@ def test_bias_vector_and_scalar_loads(lib, K, groups):
     (1, 8, 9, 50, 16, 2, 2, 1, 32, 1, 5),              # padding as wide as the kernel takes
     (60, 8, 7, 7, 8, 3, 3, 1, 1, 1, 7),                # small images: a window spans many (7 rows each)
     (300, 18, 14, 14, 16, 3, 3, 1, 1, 1, 8),           # whole images staged (3528 bytes: two alignments in turn)
-    (30, 3, 225, 223, 16, 5, 5, 2, 2, 1, 7),           # enough rows for every block to walk windows in every schedule
-    (100, 48, 30, 30, 64, 3, 3, 1, 1, 1, 9),           # the same, channel form with moved overlap rows
+    (30, 3, 225, 223, 16, 5, 5, 2, 2, 1, 7),           # segments of one window dealt to the blocks in turn; blocks that walk one segment
+    (100, 48, 30, 30, 64, 3, 3, 1, 1, 1, 9),           # the same in channel form: flat groups, moved overlap rows
     (20, 64, 56, 24, 40, 3, 3, 1, 1, 1, 9),            # one tiled copy for all channels: segments of single images
     (12, 20, 96, 44, 32, 3, 5, 2, (1, 2), 1, 8),       # the same with stride 2; ragged last segment of an image
 ])
@@ -69,6 +69,30 @@ def test_plane_kernel(lib, case, out_layout, out_mode):
     assert ids
     for i in ids:
         check_against_oracle(x, w, stride, pad, dil, shift, out_mode, i, ref=ref, out_layout=out_layout)
+
+
+# ---- blocks that walk several segments of several windows (moved overlap rows, then a fresh segment in the same rings), and
+# accumulator rings of odd length between two sets of epilogue warps: combinations that only larger batches list ----------
+@pytest.mark.parametrize("case", [
+    # N, C, H, W, K, R, stride, out_layout, out_mode
+    (90, 17, 40, 36, 16, 3, 1, 0, 2),      # one tiled copy, flat groups: 180 segments of 20 rows, windows of 10
+    (160, 48, 16, 34, 16, 3, 2, 1, 1),     # one tiled copy, unaligned words, stride 2: 160 segments of 8 rows, windows of 4
+    (150, 48, 42, 44, 16, 3, 2, 0, 2),     # row segments by bulk copies: 150 segments of 22 rows, windows of 11
+    (160, 64, 38, 37, 16, 3, 1, 1, 2),     # two blocks per SM, one window buffer and one raw chunk: 320 segments
+    (160, 16, 40, 35, 96, 3, 1, 0, 3),     # segments across images, ring of five accumulators
+    (300, 5, 29, 30, 96, 3, 1, 0, 1),      # the same in row form
+    (310, 1, 23, 37, 144, 3, 1, 0, 1),     # whole images, row form, ring of three accumulators
+])
+def test_plane_kernel_walks_segments(lib, case):
+    N, C, H, W, K, R, stride, out_layout, out_mode = case
+    x = int8_uniform((N, C, H, W), 1081)
+    w = int8_uniform((K, C, R, R), 1082)
+    ref = oracle.conv2d_int8(x, w, stride, R // 2, 1, 8)
+    d = lib.make_desc(N, C, H, W, K, R, R, stride, R // 2, 1, 8, 0, out_layout, out_mode)
+    ids = [e.id for e in lib.enumerate_embeddings(d) if e.variant == b2c.VARIANT_IM2COL_WINDOW]
+    assert len(ids) > 1
+    for i in ids:
+        check_against_oracle(x, w, stride, R // 2, 1, 8, out_mode, i, ref=ref, out_layout=out_layout)
 
 
 def test_plane_kernel_reads_the_last_incomplete_16_bytes(lib):
@@ -113,6 +137,7 @@ def test_grouped_plane_kernel(lib, case):
     d = lib.make_desc(N, C, H, W, K, R, R, 1, 1, 1, shift, out_mode=out_mode)
     plan = lib.Plan(d, b2c.POLICY_AUTO_TIMED, groups=groups)
     assert plan.info().device_us > 0
+    assert plan.info().variant == b2c.VARIANT_IM2COL_WINDOW   # well ahead of the staged window and of the dense form here
     plan.set_weights(to_dev(w))
     plan.set_activation(to_dev(bias), True)
     y32 = torch.full((N, K, H, W), -7777777, dtype=torch.int32, device="cuda") if out_mode & 1 else None
