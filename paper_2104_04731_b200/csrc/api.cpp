@@ -582,7 +582,7 @@ int create_plan_for(const Geom& g, const b2c_embedding& emb, int schedule, b2c_p
     p->plane.w = reinterpret_cast<const uint8_t*>(p->w_packed);
     p->plane.mma_table = p->mma_table;
     p->ws_total = 0;
-    *out = p;  // (no tensor maps: raw rows and weights travel by plain bulk copies)
+    *out = p;  // (no map of the weights: they travel by a plain bulk copy; the tiled copy of raw rows is encoded per run)
     return B2C_OK;
   }
   p->ws_total = workspace_bytes_for(g, emb.variant, emb.tile_n, emb.split_k, is_swapped(emb));
@@ -1002,10 +1002,11 @@ int b2c_plan_create_grouped_timed(const b2c_conv_desc* desc, int32_t groups, voi
   cudaFree(lane.ws);
   // The other form: every group merged, i.e. the dense convolution with block-diagonal filters through the
   // timed selection of dense plans.  It pays `groups` times the MACs and has the rewrite and the scratch
-  // of its embedding; it is built while those MACs, at 0.62 of the intrinsic's issue rate (the most a path from
-  // NCHW input reaches), would not take longer than the best form in place.
+  // of its embedding; it is built unless those MACs alone, at 2.8 POPS, would take longer than the best form in
+  // place.  (0.62 of the intrinsic's issue rate, well above what a dense path from NCHW input has reached: 1.99
+  // POPS for 1440 images of 256 x 14 x 14.  A form that is cut off could not have won.)
   const long long dense_w = (long long)desc->K * desc->C * desc->R * desc->S;
-  const double dense_us = 2.0 * (double)g.Mg * (double)dense_w / (0.62 * 4.5e9);  // 4.5 POPS
+  const double dense_us = 2.0 * (double)g.Mg * (double)dense_w / (0.62 * 4.5e9);  // issue rate 4.5 POPS
   b2c_plan* dense = nullptr;
   if (us <= 0 || dense_w > (16ll << 20) || dense_us >= us ||  // (a form in place that could not be timed is still the safe choice)
       b2c_plan_create(desc, B2C_POLICY_AUTO_TIMED, cuda_stream, &dense) != B2C_OK || dense->emb.device_us <= 0 ||

@@ -173,7 +173,7 @@ struct ConvArgs {
 };
 
 // Geometry of the window unroll over planes of units (A_PLANE, conv_mma_plane.cu); the kernel takes it beside ConvArgs.
-constexpr int kPlaneMinTiles = 2500;        // accumulator tiles of a problem from which the plane kernel runs it
+constexpr int kPlaneMinTiles = 2500;        // accumulator tiles above which the plane kernel is listed beside the window kernel
 constexpr int kMaxStridePhases = 8;         // strides the window unroll handles
 constexpr int kPlaneMargin = 128;          // readable bytes on either side of the staged raw rows
 constexpr int kMaxAcc = 8;                  // accumulator ring

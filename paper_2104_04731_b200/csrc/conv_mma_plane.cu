@@ -29,8 +29,8 @@
 // resident.
 // What bounds it now: the stores of the results (about 5 cycles of the SM's store path per 128 bytes, 32 lanes from any
 // start) beside the builders' shared-memory traffic.  Before (operand rows written out by builder warps, or a rewrite
-// through memory) and after: 64 images of 3 x 227 x 227, 7x7 stride 2, 64 channels 97 -> 51 us; 32 of 1 x 700 x 161,
-// 20x5 stride 2, 76 -> 33; 15501 of 16 x 14 x 14, 3x3, 124 -> 94; 315 of 64 x 56 x 56, 3x3, 99 -> 81.
+// through memory) and after: 64 images of 3 x 227 x 227, 7x7 stride 2, 64 channels 97 -> 52 us; 32 of 1 x 700 x 161,
+// 20x5 stride 2, 76 -> 30; 15501 of 16 x 14 x 14, 3x3, 125 -> 95; 315 of 64 x 56 x 56, 3x3, 99 -> 80.
 // Copies of window w + 2, units of w + 1, MMAs of w and stores of w - 1 overlap.  Every wait is
 // bounded as in the other kernels.
 #include <algorithm>
