@@ -34,12 +34,13 @@ __device__ __forceinline__ void pack_weights_cp_words(const WeightPack& p, Idx f
     reinterpret_cast<uint32_t*>(p.out)[i] = v;
   }
 }
-// The activation-pack kernels take the weight pack along: the last p.blocks blocks of the x axis do it.
+// The activation-pack kernels take the weight pack along: the last p.blocks blocks of every row of the grid do it.
 __device__ __forceinline__ bool weight_pack_block(const WeightPack& p) {
   const int extra = (int)blockIdx.x - ((int)gridDim.x - p.blocks);
   if (p.blocks == 0 || extra < 0) return false;
   pdl_wait();
-  if (blockIdx.y == 0) pack_weights_cp_words<unsigned>(p, (unsigned)extra * blockDim.x + threadIdx.x, (unsigned)p.blocks * blockDim.x);
+  pack_weights_cp_words<unsigned>(p, (blockIdx.y * (unsigned)p.blocks + (unsigned)extra) * blockDim.x + threadIdx.x,
+                                  gridDim.y * (unsigned)p.blocks * blockDim.x);
   pdl_launch_dependents();
   return true;
 }
@@ -766,10 +767,24 @@ bool weight_pack_rides(const WeightPack& p, const int8_t* x, int N, int C, int H
   return !packs_small_images(x, N, C, HW) && (long long)p.K * p.RS * (p.C_pad / 4) <= kPackWords32;
 }
 
+// Grid of an activation pack with `tiles` x `rows` blocks and the riding weight blocks, dealt to the rows.
+// Every block of the launch takes the activation tile's shared memory, weight blocks too, and where the activations
+// alone fill the machine more than two others on every SM leave no room for the convolution's blocks to start early: 31
+// images of 249 x 52 x 17 -> 87, 5x5, 39.5 us with four, 35.4 with two.  With few activation blocks the weights are the
+// work: up to eight (1 image of 256 x 28 x 28 -> 512, 5x5: two 22.4 us, four 17.8, eight 14.6).
+static dim3 pack_grid(WeightPack* wp, long long tiles, int rows) {
+  if (wp->blocks > 0) {
+    const long long full = ((long long)wp->K * wp->RS * (wp->C_pad / 4) + kPackThreads - 1) / kPackThreads;
+    const long long all = std::min<long long>(full, (tiles * rows >= kNumSMs ? 2 : 8) * kNumSMs);
+    wp->blocks = (int)((all + rows - 1) / rows);  // (of one row)
+  }
+  return dim3((unsigned)tiles + (unsigned)wp->blocks, (unsigned)rows, 1);
+}
+
 cudaError_t launch_pack_activations(const int8_t* x, int8_t* out, int N, int C, int H, int W, int C_pad,
                                     cudaStream_t st, int* status, const Dbg& dbg, const WeightPack* ride) {
   const int HW = H * W;
-  const WeightPack wp = ride ? *ride : WeightPack{nullptr, nullptr, 0, 0, 0, 0, 0};
+  WeightPack wp = ride ? *ride : WeightPack{nullptr, nullptr, 0, 0, 0, 0, 0};
   int CT = C_pad >= 128 ? 128 : 64;
   const bool a16 = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
   if (ride && !weight_pack_rides(*ride, x, N, C, HW)) return cudaErrorInvalidValue;  // (never the previous call's weights)
@@ -788,7 +803,7 @@ cudaError_t launch_pack_activations(const int8_t* x, int8_t* out, int N, int C, 
     // small tensors: narrower channel tiles so that the grid still covers the machine
     while (CT > 32 && (long long)hw_tiles * N * ((C_pad + CT - 1) / CT) < 2 * kNumSMs) CT >>= 1;
     const size_t smem = (size_t)(CT / 16) * (16 * PT + 16);
-    dim3 grid((unsigned)hw_tiles * (unsigned)N + (unsigned)wp.blocks, (C_pad + CT - 1) / CT, 1);
+    const dim3 grid = pack_grid(&wp, (long long)hw_tiles * N, (C_pad + CT - 1) / CT);
     if (row_mode)
       return launch_pdl(pack_activations_bulk_kernel<true>, grid, dim3(kPackThreads), smem, st, x, out, C, HW, C_pad,
                         hw_tiles, CT, PT, wp, status, dbg);
@@ -797,7 +812,7 @@ cudaError_t launch_pack_activations(const int8_t* x, int8_t* out, int N, int C, 
   }
   const int PT = HW > 128 ? 256 : (HW > 64 ? 128 : 64);
   const int hw_tiles = (HW + PT - 1) / PT;
-  dim3 grid((unsigned)hw_tiles * (unsigned)N + (unsigned)wp.blocks, (C_pad + CT - 1) / CT, 1);
+  const dim3 grid = pack_grid(&wp, (long long)hw_tiles * N, (C_pad + CT - 1) / CT);
   if ((HW % 16) == 0 && a16)
     return launch_pdl(pack_activations_kernel<16>, grid, dim3(kPackThreads), 0, st, x, out, C, HW, C_pad, hw_tiles, CT,
                       PT, wp, dbg);

@@ -158,6 +158,8 @@ def test_grouped_plane_kernel(lib, case):
     (2, 48, 14, 14, 72, 3, 1, 1, 1),     # whole images by bulk copies; 48 channels padded to 64
     (3, 33, 9, 11, 40, 3, 2, 1, 1),      # odd image: the loads of the plain pack kernel; 33 channels
     (2, 70, 12, 10, 129, 1, 1, 0, 1),    # 1x1
+    (160, 130, 4, 4, 600, 3, 1, 1, 1),   # as many blocks of activations as SMs: fewer of weights, several words a thread
+    (2, 256, 14, 14, 512, 3, 2, 1, 1),   # eight rows of channel tiles, weight blocks dealt to them
 ])
 def test_one_shot_packs_weights_with_the_activations(lib, case):
     N, C, H, W, K, R, stride, pad, dil = case
