@@ -47,8 +47,8 @@ def kernel_sources_sha1():
     return hashlib.sha1(b"".join(open(os.path.join(ROOT, "paper_2104_04731_b200", "csrc", f), "rb").read()
                                  for f in KERNEL_SOURCES)).hexdigest()
 # (per tile shape "tile_m x tile_n" of the channel-pack map on the headline shape)
-NCU_TRAFFIC = {"conv_mma_sha1": "95b16a2aa406361a918db8f69d45cf816432e3dd",
-               "bytes_per_launch": {"256x256": 2850304, "256x128": 2850048, "128x256": 2859264}}
+NCU_TRAFFIC = {"conv_mma_sha1": "52be1aa19c169acdb65e4122b94d9b46c8b13674",
+               "bytes_per_launch": {"256x256": 2840320, "256x128": 2840448, "128x256": 2859776}}
 
 
 def load_peaks():
@@ -855,7 +855,8 @@ def main():
     ap.add_argument("--no-graph", action="store_true")
     ap.add_argument("--no-cpu", action="store_true")
     ap.add_argument("--headline-only", action="store_true", help="skip the per-shape and scaled-batch series")
-    ap.add_argument("--pick", default=None, help="embedding as variant,tile_n,split_k[,tile_m] (instead of an id)")
+    ap.add_argument("--pick", default=None, help="first embedding with variant,tile_n,split_k[,tile_m] (instead of an id; schedules of the window unroll "
+                         "can agree in all of them: --embedding tells them apart)")
     ap.add_argument("--scaled", action="store_true", help="use the batch-scaled version of the shape as the workload")
     ap.add_argument("--instances", type=int, default=0, help="instances per step (default: enough to exceed L2)")
     ap.add_argument("--min-warm-s", type=float, default=0.2, help="extra time-based warm-up before the timed steps")
