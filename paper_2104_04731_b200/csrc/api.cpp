@@ -964,7 +964,7 @@ int b2c_plan_create_grouped_timed(const b2c_conv_desc* desc, int32_t groups, voi
       sd.K = m * kg;
       Geom sg;
       if (resolve_geom(&sd, &sg) != B2C_OK) continue;
-      for (int nth = 0; nth < 10; ++nth) {
+      for (int nth = 0;; ++nth) {
         PlaneArgs pl;
         if (!plane_plan(sg, groups / m, nth, &pl)) break;
         b2c_embedding e;

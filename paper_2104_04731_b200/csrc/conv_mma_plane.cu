@@ -27,10 +27,11 @@
 // the builder warps turn raw rows into units (byte transposes or unaligned words, zeros outside the image), the
 // epilogue warps drain the accumulators (activation step, shift / clip, NKPQ or NPQK stores).  The weights stay
 // resident.
-// What bounds it now: the stores of the results (about 5 cycles of the SM's store path per 128 bytes, 32 lanes from any
-// start) beside the builders' shared-memory traffic.  Before (operand rows written out by builder warps, or a rewrite
-// through memory) and after: 64 images of 3 x 227 x 227, 7x7 stride 2, 64 channels 97 -> 52 us; 32 of 1 x 700 x 161,
-// 20x5 stride 2, 76 -> 30; 15501 of 16 x 14 x 14, 3x3, 125 -> 95; 315 of 64 x 56 x 56, 3x3, 99 -> 80.
+// What bounds it now: the stores of the results (4 to 5 cycles of the SM's store path per 128 bytes; runs of 32 lanes that start
+// inside a sector cost the memory side more, see plane_sector_rows) beside the builders' shared-memory traffic.  Before (operand
+// rows written out by builder warps, or a rewrite through memory) and after: 64 images of 3 x 227 x 227, 7x7 stride 2, 64 channels 97 -> 52 us; 32 of 1 x 700 x 161,
+// 20x5 stride 2, 76 -> 30; 15501 of 16 x 14 x 14, 3x3, 125 -> 95; 315 of 64 x 56 x 56, 3x3, 99 -> 79; tiles on sector
+// boundaries: 51.6 -> 49.2 and 79.2 -> 73.6 us of these.
 // Copies of window w + 2, units of w + 1, MMAs of w and stores of w - 1 overlap.  Every wait is
 // bounded as in the other kernels.
 #include <algorithm>
@@ -136,6 +137,7 @@ __device__ __forceinline__ ChunkRows chunk_rows(const ConvArgs& args, const Plan
 // segments are those of one image each (spi per image, its P output rows only), else seg_rows rows of the batch.
 struct SegRows {
   int begin, end, windows;
+  int out0;  // (segments of one image) output row of the image at which it begins
 };
 __device__ __forceinline__ SegRows seg_rows(const ConvArgs& args, const PlaneArgs& pl, int seg) {
   SegRows b;
@@ -143,9 +145,11 @@ __device__ __forceinline__ SegRows seg_rows(const ConvArgs& args, const PlaneArg
     const int n = (int)pl.div_spi.div((uint32_t)seg);
     const int r0 = (seg - n * pl.spi) * pl.seg_rows;
     b.begin = n * pl.rpi + r0;
+    b.out0 = r0;
     b.end = n * pl.rpi + min(r0 + pl.seg_rows, args.out_P);
   } else {
     b.begin = seg * pl.seg_rows;
+    b.out0 = 0;
     b.end = min(b.begin + pl.seg_rows, pl.total_rows);
   }
   b.windows = (b.end - b.begin + pl.th - 1) / pl.th;
@@ -153,13 +157,16 @@ __device__ __forceinline__ SegRows seg_rows(const ConvArgs& args, const PlaneArg
 }
 struct WindowSpan {
   int gr0, rows, new0, new1;
+  int lead;  // positions between the start of the first tile and the window's first output
 };
-__device__ __forceinline__ WindowSpan window_span(const PlaneArgs& pl, const SegRows& b, int w) {
+template <bool LEAD>
+__device__ __forceinline__ WindowSpan window_span(const ConvArgs& args, const PlaneArgs& pl, const SegRows& b, int w) {
   WindowSpan s;
   s.gr0 = b.begin + w * pl.th;
   s.rows = min(pl.th, b.end - s.gr0);
   s.new0 = w == 0 ? s.gr0 : s.gr0 + pl.max_ri;
   s.new1 = s.gr0 + s.rows + pl.max_ri;
+  s.lead = LEAD ? ((b.out0 + w * pl.th) * args.out_Q) & pl.lead_mask : 0;
   return s;
 }
 // Bytes of one channel's slot for a segment of `rows` raw rows: any start inside 16 bytes, rounded up.
@@ -168,8 +175,10 @@ __device__ __forceinline__ int segment_bytes(int rows, int W) { return (rows * W
 // RUNW: 0 = channel form, else row form with runs of RUNW words.  VAR: channel form 2 = unit strides and H * W a
 // multiple of 4 (pixels are taken four at a time across row ends, so that any width reads whole words), 1 = every
 // row of every channel starts on a word, 0 = any; row form 1, 2 = the horizontal stride (four neighbouring columns per builder item), 0 = any
-// stride (one column).  KB builder warps, KE epilogue warps, MINB blocks per SM.
-template <int RUNW, int VAR, int KB, int KE, int MINB>
+// stride (one column).  KB builder warps, KE epilogue warps, MINB blocks per SM.  LEAD (row form): tiles may start before
+// their window, so that stores start on sectors.  An instantiation of its own: the few instructions cost layers that have no
+// use for it 5 % (15501 images of 16 x 14 x 14, 95 -> 100 us).
+template <int RUNW, int VAR, int KB, int KE, int MINB, bool LEAD>
 __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
     conv_mma_plane_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvArgs args, const PlaneArgs pl) {
   extern __shared__ uint8_t smem_raw[];
@@ -187,8 +196,8 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
   // shared memory: [windows][raw rows, margins around each stage][weights][A descriptor offsets]
   const uint32_t smem_base = (smem_u32(smem_raw) + 127u) & ~127u;
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
-  const uint32_t win_off = 0;
-  const uint32_t raw_off = (uint32_t)(pl.win_stages * pl.win_bytes);
+  const uint32_t win_off = LEAD ? (uint32_t)(pl.lead_mask + 1) * 16u : 0u;  // a first tile may start before the window
+  const uint32_t raw_off = win_off + (uint32_t)(pl.win_stages * pl.win_bytes);
   const uint32_t w_off = raw_off + (uint32_t)(pl.raw_stages * pl.raw_bytes);
   const uint32_t tab_off = w_off + (uint32_t)pl.w_bytes;
 
@@ -256,7 +265,7 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
     for (int seg = seg_first; seg < seg_end && alive; seg += seg_step) {
     const SegRows blk = seg_rows(args, pl, seg);
     for (int win = 0; win < blk.windows && alive; ++win) {
-      const WindowSpan sp = window_span(pl, blk, win);
+      const WindowSpan sp = window_span<LEAD>(args, pl, blk, win);
       for (int c0 = sp.new0; c0 < sp.new1; c0 += pl.cr) {
       const ChunkRows r = chunk_rows(args, pl, c0, min(pl.cr, sp.new1 - c0));
       alive = __all_sync(0xffffffffu, mbar_wait_sleep(smem_u32(&pc.raw_empty[s]), ph ^ 1u, ctl, args.status, kSleepWindow));
@@ -345,9 +354,9 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
     for (int win = 0; win < blk.windows && alive; ++win) {
       alive = __all_sync(0xffffffffu, mbar_wait(smem_u32(&pc.win_full[s]), ph, ctl, args.status));
       if (!alive) break;
-      const int rows = window_span(pl, blk, win).rows;
-      const int tiles = (rows * pl.pitch + kTileM - 1) / kTileM;
-      uint64_t abase = make_plain_desc(smem_base + win_off + (uint32_t)(s * pl.win_bytes), 0u);
+      const WindowSpan sp = window_span<LEAD>(args, pl, blk, win);
+      const int tiles = (sp.rows * pl.pitch + sp.lead + kTileM - 1) / kTileM;
+      uint64_t abase = make_plain_desc(smem_base + win_off + (uint32_t)(s * pl.win_bytes) - (uint32_t)(sp.lead * 16), 0u);
       for (int t = 0; t < tiles; ++t) {
         alive = __all_sync(0xffffffffu, mbar_wait(smem_u32(&pc.acc_empty[buf]), aph ^ 1u, ctl, args.status));
         if (!alive) break;
@@ -396,7 +405,7 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
     for (int seg = seg_first; seg < seg_end && ok; seg += seg_step) {
     const SegRows blk = seg_rows(args, pl, seg);
     for (int win = 0; win < blk.windows && ok; ++win) {
-      const WindowSpan sp = window_span(pl, blk, win);
+      const WindowSpan sp = window_span<LEAD>(args, pl, blk, win);
       ok = mbar_wait_sleep(smem_u32(&pc.win_empty[ws]), wph ^ 1u, ctl, args.status, kSleepWindow);
       if (!__all_sync(0xffffffffu, ok)) break;
       const uint32_t win_s = win_off + (uint32_t)(ws * pl.win_bytes);
@@ -728,15 +737,19 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
     for (int seg = seg_first; seg < seg_end && ok; seg += seg_step) {
     const SegRows blk = seg_rows(args, pl, seg);
     for (int win = 0; win < blk.windows && ok; ++win) {
-      const WindowSpan sp = window_span(pl, blk, win);
+      const WindowSpan sp = window_span<LEAD>(args, pl, blk, win);
       const int positions = sp.rows * pitch;
-      const int tiles = (positions + kTileM - 1) / kTileM;
-      int j = row_j, q = row_q;  // this lane's grid row and column in the window
+      const int tiles = (positions + sp.lead + kTileM - 1) / kTileM;
+      int j = row_j, q = row_q - sp.lead;  // this lane's grid row and column in the window
+      if constexpr (LEAD)
+        for (; q < 0; q += pitch) --j;
       for (int t = 0; t < tiles; ++t, ++ti) {
         if (kSets == 1 || (ti & (kSets - 1)) == set) {
           const int n = (int)pl.div_rpi.div((uint32_t)(sp.gr0 + j));
           const int i = sp.gr0 + j - n * pl.rpi;
-          const bool row_valid = t * kTileM + row < positions && q < args.out_Q && i < args.out_P;
+          bool row_valid = t * kTileM + row < positions && q < args.out_Q && i < args.out_P;
+          if constexpr (LEAD)  // (one comparison: positions before the window wrap to large values)
+            row_valid = (unsigned)(t * kTileM + row - sp.lead) < (unsigned)positions && q < args.out_Q && i < args.out_P;
           const int out_pq = i * args.out_Q + q;
           ok = mbar_wait(smem_u32(&pc.acc_full[buf]), aph, ctl, args.status);
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -784,20 +797,26 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
   }
 }
 
-template <int RUNW, int VAR, int KB, int KE, int MINB>
+template <int RUNW, int VAR, int KB, int KE, int MINB, bool LEAD>
 cudaError_t launch_one(const CUtensorMap& tmap, const ConvArgs& args, const PlaneArgs& pl, dim3 grid, cudaStream_t st) {
   static std::atomic<unsigned long long> configured{0};
   cudaError_t e =
-      set_max_dynamic_smem_once(configured, (const void*)conv_mma_plane_kernel<RUNW, VAR, KB, KE, MINB>, kPlaneSmemMax);
+      set_max_dynamic_smem_once(configured, (const void*)conv_mma_plane_kernel<RUNW, VAR, KB, KE, MINB, LEAD>, kPlaneSmemMax);
   if (e != cudaSuccess) return e;
-  return launch_pdl(conv_mma_plane_kernel<RUNW, VAR, KB, KE, MINB>, grid, dim3(64 + 32 * (KB + KE)), (size_t)pl.smem, st, tmap, args, pl);
+  return launch_pdl(conv_mma_plane_kernel<RUNW, VAR, KB, KE, MINB, LEAD>, grid, dim3(64 + 32 * (KB + KE)), (size_t)pl.smem, st, tmap, args, pl);
 }
 
+template <int RUNW, int VAR, bool LEAD>
+cudaError_t launch_blocks(const CUtensorMap& tmap, const ConvArgs& args, const PlaneArgs& pl, dim3 grid, cudaStream_t st) {
+  // One block per SM: eight builder and eight epilogue warps; two blocks: four of each.
+  if (pl.per_sm == 1) return launch_one<RUNW, VAR, 8, 8, 1, LEAD>(tmap, args, pl, grid, st);
+  return launch_one<RUNW, VAR, 4, 4, 2, LEAD>(tmap, args, pl, grid, st);
+}
 template <int RUNW, int VAR>
 cudaError_t launch_form(const CUtensorMap& tmap, const ConvArgs& args, const PlaneArgs& pl, dim3 grid, cudaStream_t st) {
-  // One block per SM: eight builder and eight epilogue warps; two blocks: four of each.
-  if (pl.per_sm == 1) return launch_one<RUNW, VAR, 8, 8, 1>(tmap, args, pl, grid, st);
-  return launch_one<RUNW, VAR, 4, 4, 2>(tmap, args, pl, grid, st);
+  if constexpr (RUNW > 0)
+    if (pl.lead_mask) return launch_blocks<RUNW, VAR, true>(tmap, args, pl, grid, st);
+  return launch_blocks<RUNW, VAR, false>(tmap, args, pl, grid, st);
 }
 template <int RUNW>
 cudaError_t launch_row_form(const CUtensorMap& tmap, const ConvArgs& args, const PlaneArgs& pl, dim3 grid, cudaStream_t st) {

@@ -392,7 +392,7 @@ struct PlaneForm {
   std::vector<Unit> units;
 };
 
-bool plane_form(const Geom& g, bool row_form, PlaneForm* f) {
+bool plane_form(const Geom& g, bool row_form, bool whole_sectors, PlaneForm* f) {
   const b2c_conv_desc& d = g.d;
   const int sh = d.stride_h, sw = d.stride_w;
   if (sh > kMaxStridePhases || sw > kMaxStridePhases) return false;
@@ -476,8 +476,27 @@ bool plane_form(const Geom& g, bool row_form, PlaneForm* f) {
   const int share_w = (row_form || sw != 1) ? 0 : std::max(0, std::min(std::min(d.pad_w, f->max_si), cols - (d.W + d.pad_w)));
   const int share_h = sh != 1 ? 0 : std::max(0, std::min(std::min(d.pad_h, f->max_ri), rows - (d.H + d.pad_h)));
   f->pitch = cols - share_w;
+  // (the added columns stay zero)
+  if (whole_sectors) f->pitch = g.Q + round_up(f->pitch - g.Q, (d.out_mode & B2C_OUT_I32) ? kSectorOutputs : 4 * kSectorOutputs);
   f->rpi = rows - share_h;
   return true;
+}
+
+// Grid rows after which NKPQ results start on a memory sector again (1: every row does; 0: no schedule can keep to sectors).
+// The channel form takes windows of so many rows; the row form's tiles start before a window that does not start on a boundary.
+// A grid row's outputs are one run of memory, and the next row's follow without a gap; so where the row's overhang is a
+// multiple of a sector's outputs, a warp's 32 positions lie the same way to the sectors all through a window, and windows
+// that start on a boundary keep every store on it.  Stores of 32 int32 results from any start took 67 us for 253 MB, from sector
+// boundaries 47: the memory side pays for the two partly written sectors, not the SM.  H * W of the results decides how many
+// channels start on a boundary: all (a multiple of 8; 32 for int8), or every other one (4, 16); fewer are not worth it.
+int plane_sector_rows(const Geom& g, int pitch) {
+  const b2c_conv_desc& d = g.d;
+  if (d.out_layout != B2C_LAYOUT_NCHW) return 0;
+  const int outputs = (d.out_mode & B2C_OUT_I32) ? kSectorOutputs : 4 * kSectorOutputs;
+  if ((pitch - g.Q) % outputs != 0 || g.PQ % (outputs / 2) != 0) return 0;
+  int rows = 1;
+  while ((long long)rows * g.Q % outputs != 0) rows <<= 1;
+  return rows;
 }
 
 // Schedule of one form with per_sm blocks per SM, windows of min_tiles to max_tiles accumulator tiles, dealt one by one
@@ -487,7 +506,7 @@ bool plane_form(const Geom& g, bool row_form, PlaneForm* f) {
 // MMA, the store path) and takes the slowest role per window, the way of the first window to its MMAs and the stores
 // of the last one.
 double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm, bool dealt, int min_tiles, int max_tiles, int stages,
-                      PlaneArgs* pl) {
+                      bool whole_sectors, PlaneArgs* pl) {
   const b2c_conv_desc& d = g.d;
   const int HW = d.H * d.W;
   const long long total_rows = (long long)d.N * f.rpi;
@@ -496,7 +515,10 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
   const int n16 = round_up(d.K, 16);
   const int nruns = d.C * f.ndh, ncb = (d.C + 15) / 16;
   const double out_bytes = (d.out_mode & B2C_OUT_I32 ? 4.0 : 0.0) + (d.out_mode & B2C_OUT_I8 ? 1.0 : 0.0);
-  const double out_cost = (d.out_mode & B2C_OUT_I32 ? 5.0 : 0.0) + (d.out_mode & B2C_OUT_I8 ? 3.0 : 0.0);
+  const int step = whole_sectors ? plane_sector_rows(g, f.pitch) : 1;  // rows of windows and segments come in multiples of it
+  const int outputs = (d.out_mode & B2C_OUT_I32) ? kSectorOutputs : 4 * kSectorOutputs;
+  const int max_lead = f.runw > 0 && plane_sector_rows(g, f.pitch) > 1 ? outputs - 1 : 0;
+  const double out_cost = (d.out_mode & B2C_OUT_I32 ? (whole_sectors ? 4.0 : 5.0) : 0.0) + (d.out_mode & B2C_OUT_I8 ? 3.0 : 0.0);
   const int kb = per_sm == 2 ? 4 : 8, sets = per_sm == 2 ? 1 : 2;  // builder warps; sets of four epilogue warps
   const int smem_max = per_sm == 2 ? 110 * 1024 : kPlaneSmemMax;
   double best = -1;
@@ -521,12 +543,13 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
     while (tmem_cols < nbuf * tile_n) tmem_cols <<= 1;
     const int places = (int)std::max<long long>(1, (long long)kNumSMs * per_sm / ((long long)cols * groups));
     for (int th = 1; th <= 128; th += 1 + th / 16) {
-      const int tiles = (th * f.pitch + kTileM - 1) / kTileM;
+      const int tiles = (th * f.pitch + kTileM - 1) / kTileM;  // (the estimate leaves out what a lead can add)
+      if (th % step != 0) continue;
       if (th > 1 && (tiles > max_tiles || th > total_rows)) break;
       if (tiles < min_tiles) continue;
       const int wr = th + f.max_ri;
       const long long plane_units = (long long)wr * f.pitch;
-      const long long last_read = (long long)tiles * kTileM + (long long)f.max_ri * f.pitch + f.max_si + 1;
+      const long long last_read = (long long)(th * f.pitch + max_lead + kTileM - 1) / kTileM * kTileM + (long long)f.max_ri * f.pitch + f.max_si + 1;
       const long long win_bytes = (((f.planes - 1) * plane_units + std::max(plane_units, last_read)) * 16 + 127) / 128 * 128;
       if (win_bytes > 200 * 1024) break;
       // Segments: single windows; or a block's share of all rows, cut further when the outputs that are being written
@@ -545,6 +568,9 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
         spi = (int)((g.P + share - 1) / share);
         blocks = (int)std::min<long long>(places, (long long)d.N * spi);
       }
+      if (whole_sectors && (spi == 0 ? g.Q % kSectorOutputs != 0 : spi > 1 && share % step != 0)) continue;
+      // (a window in the middle of an image that does not start on a boundary)
+      const int lead_mask = spi > 0 && max_lead > 0 && ((long long)th * g.Q % outputs != 0 || share * g.Q % outputs != 0) ? max_lead : 0;
       const double active = (double)blocks * share * f.pitch * d.K * groups * out_bytes;
       if (spi == 0 && active > 100e6 && share > th) {
         const int parts = (int)std::min<double>((double)((share + th - 1) / th), std::ceil(active / 100e6));
@@ -599,7 +625,7 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
           const int ws = st < 2 ? 2 : 1, rs = (single && whole_first) ? 1 : (st < 1 ? 2 : 1);
           if (single && st < 2) continue;
           if (ws == 1 && !dealt && !single && th < f.max_ri) continue;  // the overlap rows are moved inside the buffer
-          const long long smem = 128 + ws * win_bytes + rs * raw_bytes + w_bytes + 8LL * round_up(num_mma, 4);
+          const long long smem = 128 + (lead_mask ? (lead_mask + 1) * 16 : 0) + ws * win_bytes + rs * raw_bytes + w_bytes + 8LL * round_up(num_mma, 4);
           if (smem > smem_max) continue;
           // one buffer between two roles makes them take turns
           double chain = rs == 1 ? copy + build_lat : std::max(copy, build_lat);
@@ -631,6 +657,7 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
           pl->c_pitch = tiled ? box : round_up(raw_rows * d.W, 16) + 64;
           pl->box_bytes = tiled ? box : 0;
           pl->spi = spi;
+          pl->lead_mask = lead_mask;
           pl->raw_bytes = (int)raw_bytes;
           pl->win_stages = ws;
           pl->raw_stages = rs;
@@ -644,8 +671,9 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
 }
 
 // Form and schedules of the plane kernel, the lowest estimate first: the best one for each number of blocks per SM,
-// way of dealing windows, range of window heights and number of buffers (their order depends on how the store path, the builders and DRAM share the time, which
-// the estimate knows to 10 to 25 %; the timed selection tries them all).
+// way of dealing windows, range of window heights and number of buffers, rows as narrow as can be or widened to whole sectors
+// (their order depends on how the store path, the builders and DRAM share the time, which the estimate knows to 10 to
+// 25 %; the timed selection tries them all).
 struct PlaneChoice {
   double t;
   PlaneArgs pl;
@@ -677,22 +705,29 @@ bool plane_choices(const Geom& g, int groups, PlaneForm* form, std::vector<Plane
   double best = -1;
   for (int f = 0; f < 2; ++f) {
     PlaneForm cand;
-    if (!plane_form(g, f == 1, &cand)) continue;
     std::vector<PlaneChoice> list;
     // blocks per SM, dealt, fewest and most tiles of a window, buffers (2: two windows and two raw chunks, 1: two and
     // one, 0: one of each; fewer are often better although no role waits less: they leave the L1 more room)
     static const int kStyles[10][5] = {{1, 1, 4, 5, 0}, {1, 1, 5, 8, 1}, {1, 1, 4, 8, 2},  {1, 1, 9, 16, 2}, {2, 1, 1, 4, 2},
                                        {2, 1, 5, 16, 0}, {2, 1, 5, 8, 1}, {2, 1, 9, 16, 1}, {2, 0, 5, 16, 2}, {1, 0, 1, 16, 2}};
-    for (const int* style : kStyles) {
-      PlaneChoice c;
-      std::memset(&c.pl, 0, sizeof(c.pl));
-      c.t = plane_schedule(g, groups, cand, style[0], style[1] != 0, style[2], style[3], style[4], &c.pl);
-      if (c.t < 0) continue;
-      bool same = false;
-      for (const PlaneChoice& o : list)
-        same |= o.pl.per_sm == c.pl.per_sm && o.pl.th == c.pl.th && o.pl.seg_rows == c.pl.seg_rows && o.pl.tile_n == c.pl.tile_n &&
-                o.pl.win_stages == c.pl.win_stages && o.pl.raw_stages == c.pl.raw_stages;
-      if (!same) list.push_back(c);
+    int narrow = 0;
+    for (int whole_sectors = 0; whole_sectors < 2; ++whole_sectors) {
+      if (!plane_form(g, f == 1, whole_sectors != 0, &cand)) break;
+      // Rows widened to whole sectors are listed beside the others where they cost little: every tile of 128 positions then holds
+      // fewer outputs (57 -> 64 positions, 315 images of 64 x 56 x 56, 79 us -> 74; 29 -> 36, depth-wise on 28 x 28, no gain).
+      if (whole_sectors && (cand.pitch == narrow || cand.pitch * 20 > narrow * 23 || plane_sector_rows(g, cand.pitch) == 0)) break;
+      narrow = cand.pitch;
+      for (const int* style : kStyles) {
+        PlaneChoice c;
+        std::memset(&c.pl, 0, sizeof(c.pl));
+        c.t = plane_schedule(g, groups, cand, style[0], style[1] != 0, style[2], style[3], style[4], whole_sectors != 0, &c.pl);
+        if (c.t < 0) continue;
+        bool same = false;
+        for (const PlaneChoice& o : list)
+          same |= o.pl.pitch == c.pl.pitch && o.pl.per_sm == c.pl.per_sm && o.pl.th == c.pl.th && o.pl.seg_rows == c.pl.seg_rows &&
+                  o.pl.tile_n == c.pl.tile_n && o.pl.win_stages == c.pl.win_stages && o.pl.raw_stages == c.pl.raw_stages;
+        if (!same) list.push_back(c);
+      }
     }
     if (list.empty()) continue;
     std::stable_sort(list.begin(), list.end(), [](const PlaneChoice& a, const PlaneChoice& b) { return a.t < b.t; });
@@ -718,6 +753,7 @@ bool plane_plan(const Geom& g, int groups, int nth, PlaneArgs* pl, std::vector<u
   if (!plane_choices(g, groups, &f, &list)) return false;
   if (nth < 0 || nth >= (int)list.size()) return false;
   *pl = list[nth].pl;
+  f.pitch = pl->pitch;  // (the form was searched with rows of two widths)
   const int HW = d.H * d.W;
   pl->runw = f.runw;
   pl->sh = d.stride_h;
@@ -782,6 +818,13 @@ static bool plane_wanted(const WindowTile* wt) { return wt == nullptr || wt->mto
 // Accumulator rows that a schedule of the plane kernel issues: whole tiles of every window, the taps' overhang among
 // them (see seg_rows and window_span in conv_mma_plane.cu).
 long long plane_rows_issued(const Geom& g, const PlaneArgs& pl) {
+  if (pl.lead_mask) {
+    long long sum = 0;  // of one image, window by window: a window's tiles start up to lead_mask positions before it
+    for (int r0 = 0; r0 < g.P; r0 += pl.seg_rows)
+      for (int r = r0; r < std::min(r0 + pl.seg_rows, g.P); r += pl.th)
+        sum += ((long long)std::min(pl.th, std::min(r0 + pl.seg_rows, g.P) - r) * pl.pitch + ((long long)r * g.Q & pl.lead_mask) + kTileM - 1) / kTileM;
+    return sum * g.d.N * kTileM;
+  }
   auto tiles = [&](long long rows) {  // of a segment
     const long long full = ((long long)pl.th * pl.pitch + kTileM - 1) / kTileM;
     return rows / pl.th * full + (rows % pl.th * pl.pitch + kTileM - 1) / kTileM;

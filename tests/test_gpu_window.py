@@ -95,6 +95,28 @@ def test_plane_kernel_walks_segments(lib, case):
         check_against_oracle(x, w, stride, R // 2, 1, 8, out_mode, i, ref=ref, out_layout=out_layout)
 
 
+# ---- NKPQ stores from sector boundaries: tiles that start before their window (row form), rows widened to whole sectors ----------
+@pytest.mark.parametrize("case", [
+    # N, C, H, W, K, R, stride, pad, out_mode
+    (20, 3, 60, 92, 16, 7, 2, 3, 1),       # row form, rows of 46: windows start at every even distance from a boundary
+    (7, 2, 96, 100, 24, 3, 1, 1, 2),       # int8 alone: sectors of 32 results, up to 28 positions of lead
+    (9, 17, 64, 54, 33, 3, 1, 1, 3),       # channel form, rows widened from 55 to 62 positions
+    (40, 64, 56, 56, 48, 3, 1, 1, 1),      # 57 to 64: every row starts on a boundary
+    (11, 20, 52, 50, 16, 3, 1, 1, 1),      # rows of 50 widened to 58, segments of several windows
+    (3, 1, 82, 30, 16, 5, 1, 2, 1),        # a short last window with a lead
+])
+def test_plane_kernel_aligned_stores(lib, case):
+    N, C, H, W, K, R, stride, pad, out_mode = case
+    x = int8_uniform((N, C, H, W), 1091)
+    w = int8_uniform((K, C, R, R), 1092)
+    ref = oracle.conv2d_int8(x, w, stride, pad, 1, 8)
+    d = lib.make_desc(N, C, H, W, K, R, R, stride, pad, 1, 8, out_mode=out_mode)
+    ids = [e.id for e in lib.enumerate_embeddings(d) if e.variant == b2c.VARIANT_IM2COL_WINDOW]
+    assert len(ids) > 1
+    for i in ids:
+        check_against_oracle(x, w, stride, pad, 1, 8, out_mode, i, ref=ref)
+
+
 def test_plane_kernel_reads_the_last_incomplete_16_bytes(lib):
     """The tensor ends inside a 16-byte unit: its last bytes are copied one by one, nothing behind them is read."""
     N, C, H, W, K = 3, 3, 29, 31, 16                     # 8091 bytes, 11 past the last whole unit
