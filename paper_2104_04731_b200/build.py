@@ -10,7 +10,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 SO = os.path.join(HERE, "libb2conv.so")
 SO_DEBUG = os.path.join(HERE, "libb2conv_debug.so")  # -DB2C_DEBUG_BOUNDS: bounds-checked kernels, workspace guard bands
-SOURCES = ["api.cpp", "planner.cpp", "tma.cpp", "layout.cu", "conv_mma.cu", "conv_mma_pair.cu", "mma_rate.cu", "conv_mma_window.cu", "conv_mma_plane.cu"]
+SOURCES = ["api.cpp", "planner.cpp", "tma.cpp", "layout.cu", "conv_mma.cu", "conv_mma_pair.cu", "mma_rate.cu", "conv_mma_window.cu", "conv_mma_plane.cu", "conv_mma_stream.cu"]
 
 
 def _nvcc() -> str:

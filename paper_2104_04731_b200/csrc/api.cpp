@@ -23,6 +23,7 @@ struct b2c_plan {
   int32_t* table32 = nullptr;    // device, plan-owned (offsets into the staged window)
   WindowGeom win = {0, 0, 0, 0, 0};
   PlaneArgs plane = {};          // plane kernel: geometry and device tables (plane.num_mma > 0: this plan runs it)
+  StreamArgs stream = {};        // stream kernel: the same (stream.taps > 0)
   uint64_t* mma_table = nullptr; // device, plan-owned: A descriptors of the plane kernel, then its weight indices
   const int32_t* plane_wsrc = nullptr;
   TmaView view = {};             // geometry handed to the im2col-mode-TMA kernel (TMA-view variants)
@@ -265,6 +266,14 @@ void fill_common_args(b2c_plan* p) {
       a.out_pad_h = d.pad_h;
       a.out_pad_w = d.pad_w;
     }
+  } else if (p->stream.taps > 0) {
+    p->amode = A_STREAM;
+    a.tile_n = p->stream.tile_n;
+    a.tmem_cols = p->stream.tmem_cols;
+    a.num_kb = p->stream.ncb * p->stream.taps;
+    a.split_k = 1;
+    a.cluster_split = 0;
+    return;
   } else if (p->plane.num_mma > 0) {
     p->amode = A_PLANE;
     a.tile_n = p->plane.tile_n;
@@ -442,7 +451,8 @@ int create_plan_for(const Geom& g, const b2c_embedding& emb, int schedule, b2c_p
   if (cudaMemset(p->status, 0, kStatusWords * sizeof(int)) != cudaSuccess) return fail(B2C_E_CUDA);
   std::vector<uint64_t> mma;
   std::vector<int32_t> wsrc;
-  const bool plane = schedule >= 0;
+  const bool stream = schedule == kStreamSchedule, plane = schedule >= 0 && !stream;
+  if (stream && !stream_plan(g, emb.tile_n, &p->stream, &mma, &wsrc)) return fail(B2C_E_UNSUPPORTED);
   if (plane && !plane_plan(g, group_count, schedule, &p->plane, &mma, &wsrc)) return fail(B2C_E_UNSUPPORTED);
   if (is_tma_view_variant(emb.variant)) {
     if (!tma_view_for(g, emb.variant, &p->view)) return fail(B2C_E_UNSUPPORTED);
@@ -501,8 +511,9 @@ int create_plan_for(const Geom& g, const b2c_embedding& emb, int schedule, b2c_p
       if (cudaMemcpy(p->wtable, wt.data(), wt.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess)
         return fail(B2C_E_CUDA);
     }
-  } else if (plane) {
-    p->w_packed_bytes = (size_t)group_count * p->plane.cols * p->plane.w_bytes;
+  } else if (plane || stream) {
+    p->w_packed_bytes = stream ? (size_t)p->stream.cols * p->stream.tile_n * p->stream.ncb * p->stream.taps * kMmaK
+                               : (size_t)group_count * p->plane.cols * p->plane.w_bytes;
     // both tables in one buffer: the A descriptors, then the weight indices
     std::vector<uint64_t> tables = mma;
     tables.resize(mma.size() + (wsrc.size() + 1) / 2);
@@ -583,6 +594,16 @@ int create_plan_for(const Geom& g, const b2c_embedding& emb, int schedule, b2c_p
     p->plane.mma_table = p->mma_table;
     p->ws_total = 0;
     *out = p;  // (no map of the weights: they travel by a plain bulk copy; the tiled copy of raw rows is encoded per run)
+    return B2C_OK;
+  }
+  if (p->amode == A_STREAM) {
+    p->stream.mma_table = p->mma_table;
+    p->stream.pairs = stream_resident_pairs(p->stream);
+    p->ws_total = 0;
+    // the packed weights as rows of 1 KB (plan-owned memory, so the map is encoded once)
+    const int rc = encode_tiled_channels(&p->tmap_b, p->w_packed, (long long)(p->w_packed_bytes / 1024), 1024, p->stream.b_stage_bytes / 1024, 1024);
+    if (rc != B2C_OK) return fail(rc);
+    *out = p;
     return B2C_OK;
   }
   p->ws_total = workspace_bytes_for(g, emb.variant, emb.tile_n, emb.split_k, is_swapped(emb));
@@ -1087,6 +1108,10 @@ static int set_weights_one(b2c_plan* p, const int8_t* w, cudaStream_t st) {
   else if (p->amode == A_PLANE)
     CUDA_TRY(launch_pack_weights_plane(w, p->w_packed, p->group_count, d.K, p->g.Kg, p->plane.tile_n, p->plane.cols,
                                        p->plane.num_mma, p->plane_wsrc, st));
+  else if (p->amode == A_STREAM)
+    // (a block of the pair reads half of a column tile, one run of memory: the plane pack with tiles of that width)
+    CUDA_TRY(launch_pack_weights_plane(w, p->w_packed, 1, d.K, p->g.Kg, p->stream.tile_n / 2, 2 * p->stream.cols,
+                                       p->stream.ncb * p->stream.taps, p->plane_wsrc, st));
   else if (is_tma_view_variant(p->emb.variant))
     CUDA_TRY(launch_pack_weights_table(w, p->w_packed, d.K, p->g.Kg, p->view.R * p->view.S * p->view.C, p->wtable, st));
   else
@@ -1199,6 +1224,11 @@ static int run_convolve(b2c_plan* p, const int8_t* x, int32_t* y32, int8_t* y8, 
       rc = encode_tiled_channels(&tmap_a, x, (long long)d.N * p->plane.img_channels, d.H * d.W, d.C, p->plane.box_bytes);
       if (rc != B2C_OK) return rc;
     }
+  } else if (p->amode == A_STREAM) {
+    if (p->stream.box_bytes > 0) {
+      rc = encode_tiled_channels(&tmap_a, x, (long long)d.N * d.C, d.H * d.W, 32, p->stream.box_bytes);
+      if (rc != B2C_OK) return rc;
+    }
   } else if (p->amode == A_WINDOW) {
     if (a.wn_linear) {
       tmap_a = p->tmap_b;  // the images arrive by plain bulk copies; any valid map
@@ -1237,6 +1267,8 @@ static int run_convolve(b2c_plan* p, const int8_t* x, int32_t* y32, int8_t* y8, 
     PlaneArgs pl = p->plane;
     pl.x_bytes = (long long)(d.N - 1) * a.x_stride_n + (long long)d.C * d.H * d.W * a.groups;
     CUDA_TRY(launch_conv_mma_plane(tmap_a, a, pl, st));
+  } else if (p->amode == A_STREAM) {
+    CUDA_TRY(launch_conv_mma_stream(tmap_a, p->tmap_b, a, p->stream, st));
   } else if (p->amode == A_WINDOW) {
     CUDA_TRY(launch_conv_mma_window(&tmap_a, &p->tmap_b, a, st));
   } else

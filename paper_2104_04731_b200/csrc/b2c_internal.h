@@ -78,7 +78,7 @@ struct Dbg {
   int* status = nullptr;         // [0] status word, [1] site, [2..3] byte offset of the first bad access from its range start
 };
 
-enum AMode { A_TILED = 0, A_IM2COL_TMA = 1, A_GATHER = 2, A_STAGED = 3, A_SHIFT = 4, A_WINDOW = 5, A_PLANE = 6 };
+enum AMode { A_TILED = 0, A_IM2COL_TMA = 1, A_GATHER = 2, A_STAGED = 3, A_SHIFT = 4, A_WINDOW = 5, A_PLANE = 6, A_STREAM = 7 };
 
 // Everything the MMA kernel needs besides its two tensor maps.
 struct ConvArgs {
@@ -206,6 +206,26 @@ struct PlaneArgs {
   // Row form: a window's tiles start (index of its first output & lead_mask) positions before it.  (The last field: among the
   // others it moved those the builders and epilogues read, 32 images of 1 x 700 x 161 30.8 -> 32.8 us.)
   int lead_mask;
+};
+
+// Geometry of the window unroll with streamed weights (A_STREAM, conv_mma_stream.cu).
+constexpr int kStreamMaxStages = 12;         // ring of weight stages
+constexpr int kStreamSmemMax = 224 * 1024;   // dynamic shared memory of one block
+constexpr int kStreamSchedule = 1000;        // Candidate::schedule of this kernel
+struct StreamArgs {
+  int stride, words;                         // both axes; H * W is a multiple of 4
+  int ndh, ndw, max_dh;                      // row and column stride phases the taps use, largest row phase
+  int8_t row_phase[2], row_index[2], col_index[2];  // phase of an index; index of a phase, -1 if no tap uses it
+  int pitch, rpi, total_rows, max_ri, images;  // grid as in PlaneArgs
+  int th;                                    // grid rows of a block's tile
+  int plane_bytes, win_bytes, win_stages;
+  int ncb, taps;                             // blocks of 32 channels, MMAs of each
+  int b_group, b_stage_bytes, b_stages, w_steps, w_run_rows;  // MMAs of a weight stage; stages of a tile; 1 KB rows of a half column tile
+  int max_images, img_slot, img_groups, box_bytes;  // images of a tile with rows; raw bytes and builder items of one; tiled copies: bytes per channel
+  int raw_bytes, raw_stages;
+  int num_tiles, cols, tile_n, tmem_cols, pairs, smem;
+  FastDiv div_rpi, div_pitch, div_w, div_groups, div_cols;
+  const uint64_t* mma_table;                 // A descriptor of every tap relative to the window, as in PlaneArgs
 };
 
 // Programmatic dependent launch: a kernel launched through launch_pdl may start while the previous
@@ -409,6 +429,8 @@ bool window_tile_geom(const Geom& g, WindowTile* wt);
 bool plane_plan(const Geom& g, int groups, int nth, PlaneArgs* pl, std::vector<uint64_t>* table = nullptr,
                 std::vector<int32_t>* wsrc = nullptr);
 long long plane_rows_issued(const Geom& g, const PlaneArgs& pl);
+// The stream kernel with column tiles of tile_n channels; false if it does not apply.  Tables as for plane_plan.
+bool stream_plan(const Geom& g, int tile_n, StreamArgs* sa, std::vector<uint64_t>* table = nullptr, std::vector<int32_t>* wsrc = nullptr);
 
 // --- tma.cpp -----------------------------------------------------------------------------------
 // Tensor-map encoders obtained through cudaGetDriverEntryPoint (no link-time libcuda dependency).
@@ -475,6 +497,9 @@ size_t conv_mma_pair_smem_bytes(const ConvArgs& args);
 cudaError_t launch_conv_mma_window(const CUtensorMap* tmap_x, const CUtensorMap* tmap_b, const ConvArgs& args, cudaStream_t st);
 size_t conv_mma_window_smem_bytes(const ConvArgs& args);
 cudaError_t launch_conv_mma_plane(const CUtensorMap& tmap, const ConvArgs& args, const PlaneArgs& pl, cudaStream_t st);
+cudaError_t launch_conv_mma_stream(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w, const ConvArgs& args, const StreamArgs& sa,
+                                   cudaStream_t st);
+int stream_resident_pairs(const StreamArgs& sa);
 // Geometry of the fused activation pack; false when the tensor has no bulk-copy form.
 bool fused_pack_geometry(int C, int H, int W, int C_pad, int* ct, int* pt, int* hw_tiles, int* ctiles, int* smem);
 cudaError_t launch_bounded_wait_selftest(int* status, cudaStream_t st);

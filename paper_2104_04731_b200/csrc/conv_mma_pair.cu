@@ -21,82 +21,11 @@
 // in the one-SM kernel.
 #include <algorithm>
 
-#include "conv_mma_common.cuh"
+#include "conv_mma_cluster.cuh"
 
 namespace b2c {
 
 namespace {
-
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// Address of the same shared-memory location in block `rank` of the cluster.
-__device__ __forceinline__ uint32_t map_to_rank(uint32_t local, uint32_t rank) {
-  uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
-  return remote;
-}
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// Waits that pair with arrivals from the other block of the cluster.
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(done)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-__device__ __noinline__ bool mbar_wait_cluster_slow(uint32_t bar, uint32_t parity, SharedCtl* ctl, int* status) {
-  const unsigned long long t0 = global_ns();
-  while (true) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    if (ctl->abort_flag) return false;
-    if (global_ns() - t0 > kWaitLimitNs) {
-      ctl->abort_flag = 1;
-      atomicCAS(status, 0, B2C_E_TIMEOUT);
-      return false;
-    }
-  }
-}
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, SharedCtl* ctl, int* status) {
-#pragma unroll 1
-  for (int i = 0; i < 32; ++i)
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-  return mbar_wait_cluster_slow(bar, parity, ctl, status);
-}
-
-// TMA loads of a block of the pair: destination in the executing block's shared memory, completion
-// on `bar`, a shared::cluster address that may lie in either block of the pair (.cta_group::2).
-__device__ __forceinline__ void tma_pair_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar,
-                                                 uint32_t on) {
-  asm volatile(
-      "{\n.reg .pred q;\nsetp.ne.b32 q, %5, 0;\n"
-      "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, %3}], "
-      "[%4];\n}" ::"r"(dst),
-      "l"(map), "r"(c0), "r"(c1), "r"(bar), "r"(on)
-      : "memory");
-}
-__device__ __forceinline__ void tma_pair_load_im2col_4d(uint32_t dst, const CUtensorMap* map, int c, int w, int h, int n,
-                                                        uint32_t bar, uint16_t off_w, uint16_t off_h, uint32_t on) {
-  asm volatile(
-      "{\n.reg .pred q;\nsetp.ne.b32 q, %9, 0;\n"
-      "@q cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, "
-      "%3, %4, %5}], [%6], {%7, %8};\n}" ::"r"(dst),
-      "l"(map), "r"(c), "r"(w), "r"(h), "r"(n), "r"(bar), "h"(off_w), "h"(off_h), "r"(on)
-      : "memory");
-}
-
-// Instruction descriptor of the two-SM MMA: as make_idesc_i8, with M = 256 (128 rows per block).
-__device__ __forceinline__ uint32_t make_idesc_i8_pair(int n) {
-  return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
-}
 
 // One reduction block of the pair: `ksteps` (1..4) two-SM MMAs over consecutive 32-byte slices.
 __device__ __forceinline__ void mma_i8_pair_block(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
@@ -125,16 +54,6 @@ __device__ __forceinline__ void mma_i8_pair_block(uint32_t d_tmem, uint64_t ades
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(on), "r"(ksteps)
       : "memory");
 }
-// Arrives on the barrier at this shared-memory offset in both blocks of the pair once every MMA
-// issued so far has completed.
-__device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint32_t on) {
-  asm volatile(
-      "{\n.reg .pred q;\n.reg .b16 m;\nsetp.ne.b32 q, %1, 0;\nmov.b16 m, 3;\n"
-      "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], m;\n}" ::"r"(bar),
-      "r"(on)
-      : "memory");
-}
-
 constexpr int kPackWarps = 4;  // warps 10..13 of the fused form: activation pack
 constexpr int kPackGroup = 32 * kPackWarps;
 

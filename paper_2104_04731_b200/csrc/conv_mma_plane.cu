@@ -53,12 +53,6 @@ struct __align__(8) PlaneCtl {
   SharedCtl base;  // abort flag and tensor-memory base (the bounded waits take this)
 };
 
-// Operand descriptor without swizzle: `half` bytes between the two 16-byte halves of the reduction slice,
-// row groups of 8 contiguous (128 bytes apart), descriptor version 1.
-__device__ __forceinline__ uint64_t make_plain_desc(uint32_t addr, uint32_t half) {
-  return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)(half >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) | ((uint64_t)1 << 46);
-}
-
 // Up to four MMAs from a list of A descriptors; the B descriptor advances by a constant step.
 __device__ __forceinline__ void mma_i8_list4(uint32_t d_tmem, uint64_t a0, uint64_t a1, uint64_t a2, uint64_t a3,
                                              uint64_t bdesc, uint64_t b_step, uint32_t idesc, uint32_t accumulate,
@@ -83,25 +77,6 @@ __device__ __forceinline__ void mma_i8_list4(uint32_t d_tmem, uint64_t a0, uint6
       "}" ::"r"(d_tmem),
       "l"(a0), "l"(a1), "l"(a2), "l"(a3), "l"(bdesc), "l"(b_step), "r"(idesc), "r"(accumulate), "r"(on), "r"(count)
       : "memory");
-}
-
-// Bounded wait with back-off: polling a barrier takes the same shared-memory pipe as the builders' and the
-// epilogue's loads and stores, and most warps of this kernel wait for whole windows (microseconds), so a warp that
-// finds its barrier not ready sleeps between polls.  (Waits for a tile poll: sleeping there costs 2 to 5 us a call.)
-__device__ __forceinline__ bool mbar_wait_sleep(uint32_t bar, uint32_t parity, SharedCtl* ctl, int* status, unsigned ns) {
-  if (mbar_try_wait(bar, parity)) return true;
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
-  while (true) {
-    __nanosleep(ns);
-    if (mbar_try_wait(bar, parity)) return true;
-    if (ctl->abort_flag) return false;
-    if (global_ns() - t0 > kWaitLimitNs) {
-      ctl->abort_flag = 1;
-      atomicCAS(status, 0, B2C_E_TIMEOUT);
-      return false;
-    }
-  }
 }
 
 // Debug build: is the unit at this offset in shared memory inside the window of `bytes` bytes at `lo`?

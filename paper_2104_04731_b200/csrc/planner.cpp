@@ -806,6 +806,118 @@ bool plane_plan(const Geom& g, int groups, int nth, PlaneArgs* pl, std::vector<u
   return true;
 }
 
+bool stream_plan(const Geom& g, int tile_n, StreamArgs* sa, std::vector<uint64_t>* table, std::vector<int32_t>* wsrc) {
+  const b2c_conv_desc& d = g.d;
+  std::memset(sa, 0, sizeof(*sa));
+  const int HW = d.H * d.W;
+  if (d.in_layout != B2C_LAYOUT_NCHW || d.stride_h != d.stride_w || d.stride_h > 2 || d.W < 4 || d.pad_h > 32 || d.pad_w > 32) return false;
+  // (bulk copies of a channel block start and end on 16 bytes)
+  if ((long long)d.C * HW % 16 != 0 || (long long)d.C * HW > (1 << 26) || d.K > 4096) return false;
+  // the grid and the units of a block of 32 channels
+  Geom block = g;
+  block.d.C = 32;
+  PlaneForm f;
+  if (!plane_form(block, false, false, &f) || f.pitch > kTileM) return false;
+  const long long total_rows = (long long)d.N * f.rpi;
+  if (total_rows > 0x3FFFFFF0 / f.pitch) return false;
+  const int sh = d.stride_h;
+  sa->stride = sh;
+  sa->words = HW % 4 == 0 ? 1 : 0;
+  sa->ndh = f.ndh;
+  sa->ndw = f.ndw;
+  sa->max_dh = f.max_dh;
+  for (int p = 0; p < 2; ++p) {
+    sa->row_phase[p] = f.row_phase[p];
+    sa->row_index[p] = -1;
+    sa->col_index[p] = f.col_phase[p];
+  }
+  for (int i = 0; i < f.ndh; ++i) sa->row_index[f.row_phase[i]] = (int8_t)i;
+  sa->pitch = f.pitch;
+  sa->rpi = f.rpi;
+  sa->total_rows = (int)total_rows;
+  sa->max_ri = f.max_ri;
+  sa->images = d.N;
+  sa->th = kTileM / f.pitch;
+  sa->ncb = (d.C + 31) / 32;
+  sa->taps = d.R * d.S;
+  const int wr = sa->th + f.max_ri;
+  const int plane_units = wr * f.pitch;
+  const int last_read = kTileM + f.max_ri * f.pitch + f.max_si;
+  sa->plane_bytes = plane_units * 16;
+  sa->win_bytes = (((f.planes - 1) * plane_units + std::max(plane_units, last_read)) * 16 + 127) / 128 * 128;
+  if ((long long)f.ndh * f.ndw * plane_units > 16000) return false;  // (14 bits of the descriptor)
+  // images of a tile whose rows it needs, and the most raw rows of one (as tile_rows and raw_rows of the kernel; the
+  // tiles repeat after rpi of them)
+  int raw_rows = 0;
+  const long long tiles_m = (total_rows + sa->th - 1) / sa->th;
+  for (long long t = 0; t < std::min<long long>(tiles_m, f.rpi); ++t) {
+    const int r0 = (int)(t * sa->th), n_a = r0 / f.rpi;
+    const int last = (int)std::min<long long>(r0 + sa->th, total_rows) - 1, n_l = last / f.rpi;
+    const int end = std::max(r0, n_l * f.rpi + std::min(last - n_l * f.rpi, g.P - 1) + f.max_ri + 1);
+    for (int n = n_a; n * f.rpi < end; ++n) {
+      const int lo = std::max(0, (r0 - n * f.rpi) * sh - d.pad_h);
+      const int hi = std::min(d.H, (end - 1 - n * f.rpi) * sh + f.max_dh - d.pad_h + 1);
+      if (hi <= lo) continue;
+      sa->max_images = std::max(sa->max_images, n - n_a + 1);
+      raw_rows = std::max(raw_rows, hi - lo);
+    }
+  }
+  if (sa->max_images < 1 || sa->max_images > 32) return false;
+  // raw rows: whole images of a channel block, one bulk copy each, or one tiled copy per image of the rows needed
+  const int box = round_up(raw_rows * d.W + 15, 16);
+  const bool tiled = HW % 16 == 0 && box <= 1024 && (long long)box < HW;
+  if (!tiled && 32LL * HW * sa->max_images > 40 * 1024) return false;
+  sa->box_bytes = tiled ? box : 0;
+  sa->img_slot = round_up(32 * (tiled ? box : HW), 128);
+  sa->img_groups = tiled ? (raw_rows * d.W + 6) / 4 : (std::min(HW, raw_rows * d.W) + 6) / 4;
+  sa->raw_bytes = sa->img_slot * sa->max_images;
+  sa->tile_n = tile_n;
+  sa->cols = (d.K + tile_n - 1) / tile_n;
+  sa->tmem_cols = 2 * tile_n;
+  sa->num_tiles = (int)((tiles_m + 1) / 2) * sa->cols;
+  // weights: 16 KB a stage and block; the run of a half column tile is read in 1 KB rows
+  sa->b_group = 1024 / tile_n;
+  sa->b_stage_bytes = sa->b_group * tile_n * 16;
+  const int total_mma = sa->ncb * sa->taps;
+  sa->w_steps = (total_mma + sa->b_group - 1) / sa->b_group;
+  sa->w_run_rows = total_mma * tile_n / 64;
+  const int table_bytes = 8 * (round_up(sa->taps, 4) + 4);
+  // rings: four windows and raw blocks where they leave room for six weight stages, else fewer
+  static const int kRings[6][3] = {{4, 4, 6}, {4, 3, 5}, {3, 3, 5}, {3, 3, 4}, {2, 2, 4}, {2, 2, 3}};
+  int ring = 0;
+  for (; ring < 6; ++ring) {
+    sa->win_stages = kRings[ring][0];
+    sa->raw_stages = kRings[ring][1];
+    const int rest = kStreamSmemMax - 128 - table_bytes - sa->win_stages * sa->win_bytes - sa->raw_stages * sa->raw_bytes;
+    sa->b_stages = rest < 0 ? 0 : std::min(std::min(kStreamMaxStages, sa->w_steps + 1), rest / sa->b_stage_bytes);
+    if (sa->b_stages >= std::min(kRings[ring][2], sa->w_steps + 1)) break;
+  }
+  if (ring == 6) return false;
+  sa->smem = 128 + table_bytes + sa->win_stages * sa->win_bytes + sa->raw_stages * sa->raw_bytes + sa->b_stages * sa->b_stage_bytes;
+  sa->pairs = kNumSMs / 2;
+  sa->div_rpi = make_fastdiv((uint32_t)f.rpi);
+  sa->div_pitch = make_fastdiv((uint32_t)f.pitch);
+  sa->div_w = make_fastdiv((uint32_t)d.W);
+  sa->div_groups = make_fastdiv((uint32_t)sa->img_groups);
+  sa->div_cols = make_fastdiv((uint32_t)sa->cols);
+  if (table && wsrc) {
+    // one MMA per tap: the two 16-channel blocks at one position
+    table->clear();
+    wsrc->assign((size_t)total_mma * 32, -1);
+    const int half = f.ndh * f.ndw * plane_units;
+    for (int r = 0; r < d.R; ++r)
+      for (int s = 0; s < d.S; ++s) {
+        const PlaneForm::Unit& u = f.units[r * d.S + s];  // (of the first 16 channels)
+        table->push_back((uint64_t)(u.plane * plane_units + u.ri * f.pitch + u.si) | ((uint64_t)half << 16));
+        for (int cb = 0; cb < sa->ncb; ++cb)
+          for (int c = 0; c < 32 && cb * 32 + c < d.C; ++c)
+            (*wsrc)[((size_t)cb * sa->taps + r * d.S + s) * 32 + c] = ((cb * 32 + c) * d.R + r) * d.S + s;
+      }
+    while (table->size() % 4 != 0) table->push_back(table->back());
+  }
+  return true;
+}
+
 // The plane kernel builds every input row once per window and needs windows of several tiles to pay for the rows the
 // taps reach below; the window kernel's tiles are independent of each other and spread a small problem over more
 // blocks.  Up to kPlaneMinTiles accumulator tiles a problem that the window kernel takes is listed for it alone; above,
@@ -923,6 +1035,18 @@ void enumerate_embeddings(const Geom& g, std::vector<Candidate>* out) {
         for (int i = 0; i < (int)plane.size(); ++i)
           add(out, g, variant, plane[i].pl.tile_n, 1, false, kTileM, i, plane_rows_issued(g, plane[i].pl),
               ((int)form.units.size() + 1) / 2 * kMmaK);
+      // Stream kernel: more channels than the plane kernel takes, taps enough to pay for the building of the units, and tiles for
+      // more than a few pairs of SMs.  The widest column tile builds the units least often; half of it where it leaves half
+      // of the pairs without a tile (16 images of 192 x 28 x 28 -> 192, 3x3: 12.7 us, half the tile 15.2).
+      if (d.C >= 48 && d.R * d.S >= 4) {
+        int wide = 64;
+        while (wide < d.K && wide < 256) wide <<= 1;
+        StreamArgs sa;
+        for (int t = wide; t >= std::max(64, wide / 2); t >>= 1) {
+          if (!stream_plan(g, t, &sa) || sa.num_tiles < 8 || (t < wide && sa.num_tiles >= kNumSMs / 2)) break;
+          add(out, g, variant, t, 1, false, kTileM, kStreamSchedule, (long long)sa.num_tiles / sa.cols * 2 * kTileM, sa.ncb * sa.taps * kMmaK);
+        }
+      }
       continue;
     }
     int num_kb;

@@ -130,6 +130,31 @@ def test_plane_kernel_reads_the_last_incomplete_16_bytes(lib):
             check_against_oracle(x, w, 1, 1, 1, 5, 3, e.id, ref=ref)
 
 
+# ---- units built while the weights stream (two SMs): staging forms, ragged blocks, walks of several tiles -------------------------
+@pytest.mark.parametrize("case", [
+    # N, C, H, W, K, R, S, stride, pad, dil, shift
+    (37, 256, 14, 14, 130, 3, 3, 2, 1, 1, 11),      # whole images, four phase planes, ragged column tile, a pair with an empty half
+    (130, 64, 7, 7, 64, 3, 3, 1, 1, 1, 9),          # H * W odd: unaligned words
+    (21, 80, 28, 28, 96, 3, 3, 1, 1, 1, 10),        # one tiled copy per image part; ragged last block of 16 channels
+    (9, 96, 44, 40, 70, 5, 5, 2, 2, 1, 11),         # 25 MMAs a block: weight stages that end inside one
+    (11, 64, 30, 52, 300, 2, 3, 1, (0, 1), 3, 9),   # dilation 3, six taps, padding on one axis
+    (60, 48, 12, 20, 256, 4, 1, 1, 2, 1, 9),        # half a block of channels, padding wider than the taps need
+    (400, 64, 14, 14, 512, 3, 3, 2, 1, 1, 10),      # several tiles a pair: both accumulators, rings that run on
+    (2, 48, 112, 126, 64, 3, 3, 1, 1, 1, 9),        # one grid row of 127 positions a tile
+])
+@pytest.mark.parametrize("out_layout,out_mode", [(0, 3), (1, 2)])
+def test_stream_kernel(lib, case, out_layout, out_mode):
+    N, C, H, W, K, R, S, stride, pad, dil, shift = case
+    x = int8_uniform((N, C, H, W), 1095)
+    w = int8_uniform((K, C, R, S), 1096)
+    ref = oracle.conv2d_int8(x, w, stride, pad, dil, shift)
+    d = lib.make_desc(N, C, H, W, K, R, S, stride, pad, dil, shift, 0, out_layout, out_mode)
+    ids = [e.id for e in lib.enumerate_embeddings(d) if e.variant == b2c.VARIANT_IM2COL_WINDOW and e.tile_n >= 64]
+    assert ids
+    for i in ids:
+        check_against_oracle(x, w, stride, pad, dil, shift, out_mode, i, ref=ref, out_layout=out_layout)
+
+
 @pytest.mark.parametrize("case", [
     # N, C, H, W, K, R, stride, pad: space to depth is a fifth or more faster than the plane kernel, and has a higher overhead
     (8, 93, 93, 9, 364, 3, 2, 1),
