@@ -1260,7 +1260,7 @@ static int run_convolve(b2c_plan* p, const int8_t* x, int32_t* y32, int8_t* y8, 
       a.pk_src = x;
       a.pk_dst = reinterpret_cast<int8_t*>(wsb);
       a.pk_ctl = reinterpret_cast<int*>(wsb + p->ws_ctl_offset);
-      CUDA_TRY(cudaMemsetAsync(a.pk_ctl, 0, (size_t)(d.N + 1) * sizeof(int), st));
+      CUDA_TRY(launch_zero_words(a.pk_ctl, d.N + 1, st));
     }
     CUDA_TRY(launch_conv_mma_pair(p->amode, &tmap_a, &p->tmap_b, a, st));
   } else if (p->amode == A_PLANE) {

@@ -473,6 +473,7 @@ cudaError_t launch_pack_weights_rows(const int8_t* w, int8_t* out, int K, int Kg
 // = filter element wsrc[(2m + u) * 16 + b] (zero where that is -1 and for channels past K).
 cudaError_t launch_pack_weights_plane(const int8_t* w, int8_t* out, int groups, int K, int Kg, int tile_n, int cols, int num_mma,
                                        const int32_t* wsrc, cudaStream_t st);
+cudaError_t launch_zero_words(int* p, int n, cudaStream_t st);
 cudaError_t launch_im2col(const int8_t* x, int8_t* a, const GatherEntry* table, long long Mg, int PQ, int Q, int H,
                           int W, int stride_h, int stride_w, int pad_h, int pad_w, long long x_stride_n,
                           int x_stride_h, int x_stride_w, int K_pad, cudaStream_t st, const Dbg& dbg = Dbg());

@@ -409,6 +409,14 @@ __global__ void pack_weights_rows_kernel(const int8_t* __restrict__ w, int8_t* _
   pdl_launch_dependents();
 }
 
+// Work counters of the activation pack inside the two-SM kernel.  A kernel instead of a memset so that launches overlap: the
+// convolution's block set-up runs beside it, and it starts while the kernel before it drains.
+__global__ void __launch_bounds__(256) zero_words_kernel(int* p, int n) {
+  pdl_launch_dependents();
+  pdl_wait();
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0;
+}
+
 // Weights of the plane kernel, in the order its MMAs read them: [group][column tile][MMA][half][channel][16].
 __global__ void pack_weights_plane_kernel(const int8_t* __restrict__ w, int8_t* __restrict__ out, int groups, int K, int Kg,
                                            int tile_n, int cols, int num_mma, const int32_t* __restrict__ wsrc) {
@@ -875,6 +883,10 @@ cudaError_t launch_pack_weights_plane(const int8_t* w, int8_t* out, int groups, 
   const long long total = (long long)groups * cols * num_mma * 32 * tile_n;
   return launch_pdl(pack_weights_plane_kernel, dim3(grid_for(total, 256)), dim3(256), 0, st, w, out, groups, K, Kg, tile_n, cols, num_mma,
                     wsrc);
+}
+
+cudaError_t launch_zero_words(int* p, int n, cudaStream_t st) {
+  return launch_pdl(zero_words_kernel, dim3(std::min((n + 255) / 256, kNumSMs)), dim3(256), 0, st, p, n);
 }
 
 cudaError_t launch_im2col(const int8_t* x, int8_t* a, const GatherEntry* table, long long Mg, int PQ, int Q, int H,
