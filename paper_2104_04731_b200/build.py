@@ -34,7 +34,7 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
         return so
     cmd = [
         _nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-        "-Xcompiler", "-fPIC", "-shared", "-cudart", "static", "-x", "cu",
+        "-Xcompiler", "-fPIC", "-shared", "-cudart", "static", "-x", "cu", "--threads", "0",
         "-I", os.path.join(ROOT, "include"), "-I", CSRC,
     ]
     if verbose:
