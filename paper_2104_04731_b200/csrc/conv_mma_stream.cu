@@ -26,6 +26,7 @@
 #include <algorithm>
 
 #include "conv_mma_cluster.cuh"
+#include "stream_tile.h"
 
 namespace b2c {
 
@@ -76,36 +77,6 @@ __device__ __forceinline__ void mma_i8_pair_list4(uint32_t d_tmem, uint64_t a0, 
 #else
 #define B2C_WINDOW_OK(d, site, lo, bytes, at) true
 #endif
-
-// Grid rows [r0, end) that a block's tile needs units of: its th output rows and what their taps reach below, up to the
-// last row that a valid output reads (the overhang rows of an image are no outputs).
-struct TileRows {
-  int r0, end, n_a;  // n_a: image of row r0
-};
-__device__ __forceinline__ TileRows tile_rows(const ConvArgs& args, const StreamArgs& sa, int r0) {
-  TileRows t;
-  t.r0 = r0;
-  t.end = r0;
-  t.n_a = sa.images;
-  if (r0 >= sa.total_rows) return t;
-  t.n_a = (int)sa.div_rpi.div((uint32_t)r0);
-  const int last = min(r0 + sa.th, sa.total_rows) - 1;
-  const int n_l = (int)sa.div_rpi.div((uint32_t)last);
-  const int i_l = min(last - n_l * sa.rpi, args.out_P - 1);
-  t.end = max(r0, n_l * sa.rpi + i_l + sa.max_ri + 1);
-  return t;
-}
-// Raw rows [lo, hi) of image n that those grid rows need (none: hi <= lo).
-struct RawRows {
-  int lo, hi;
-};
-template <int STRIDE>
-__device__ __forceinline__ RawRows raw_rows(const ConvArgs& args, const StreamArgs& sa, const TileRows& t, int n) {
-  RawRows r;
-  r.lo = max(0, (t.r0 - n * sa.rpi) * STRIDE - args.pad_h);
-  r.hi = min(args.H, (t.end - 1 - n * sa.rpi) * STRIDE + sa.max_dh - args.pad_h + 1);
-  return r;
-}
 
 // STRIDE 1 or 2 on both axes.  WORDS: H * W is a multiple of 4, so four consecutive pixels of a channel are one word.
 template <int STRIDE, bool WORDS>
@@ -273,11 +244,11 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     for (int t = tile_first; t < tile_end && alive; t += tile_step) {
       B2C_STREAM_TILE(t)
       (void)ct;
-      const TileRows tr = tile_rows(args, sa, r0);
+      const TileRows tr = stream_tile_rows(args, sa, r0);
       // lane p copies image n_a + p
       const int n = tr.n_a + lane;
       RawRows rr = {0, 0};
-      if (tr.end > tr.r0 && lane < sa.max_images && n < sa.images && n * sa.rpi < tr.end) rr = raw_rows<STRIDE>(args, sa, tr, n);
+      if (tr.end > tr.r0 && lane < sa.max_images && n < sa.images && n * sa.rpi < tr.end) rr = stream_raw_rows(args, sa, tr, n, STRIDE);
       const bool mine = rr.hi > rr.lo;
       for (int cb = 0; cb < sa.ncb; ++cb) {
         alive = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sc.raw_empty[s]), ph ^ 1u, ctl, args.status));
@@ -328,54 +299,18 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       }
     };
     const int per_row = sa.ndh * sa.ndw;      // planes of 16 channels
-    const uint32_t c_step = (uint32_t)(sa.box_bytes > 0 ? sa.box_bytes : HW);
+    const uint32_t c_step = stream_channel_step(args, sa);
     // An item's places in the raw rows and in the window are worked out once for a tile (once in all where every tile
     // starts an image) and used for its ncb channel blocks: with the divisions of every pixel in every block the builders
     // took most of the SM's issue slots (115 us, so 80).
-    struct Item {
-      uint32_t src;     // byte offset of channel 0 of the group in the raw rows
-      uint32_t dst[2];  // units of the four pixels in the window, 16 bits each, kNoUnit: not stored
-    };
-    constexpr uint32_t kNoUnit = 0xFFFFu;
     constexpr int kKept = 3;  // items a thread keeps; further ones are worked out anew
-    const int items = sa.max_images * 2 * sa.img_groups;
+    const int items = stream_items(sa);
     // Store t of a lane takes pixel t ^ y, with y from the lane, so that the eight lanes of a store phase (their groups are 64
     // bytes apart, 32 with stride 2) hit eight different 16-byte bank groups; the transposes' selectors do the exchange.
     const int y = STRIDE == 1 ? (lane >> 1) & 3 : ((lane >> 2) & 1) * 2;
     const uint32_t sel_a = (y & 2) ? 0x7362u : 0x5140u, sel_b = (y & 2) ? 0x5140u : 0x7362u;
     const uint32_t sel_c = (y & 1) ? 0x7632u : 0x5410u, sel_d = (y & 1) ? 0x5410u : 0x7632u;
-    // item e = (image of the tile, block of 16 channels, four consecutive pixels); false: nothing to store
-    auto make_item = [&](const TileRows& tr, int e, Item* it) -> bool {
-      const int iu = (int)sa.div_groups.div((uint32_t)e);
-      const int p = iu >> 1, u = iu & 1;
-      const int n = tr.n_a + p;
-      if (e >= items || n >= sa.images || n * sa.rpi >= tr.end) return false;
-      const RawRows rr = raw_rows<STRIDE>(args, sa, tr, n);
-      const int f0 = rr.lo * args.W, f1 = rr.hi * args.W;
-      const int f = ((f0 >> 2) + e - iu * sa.img_groups) * 4;
-      if (f >= f1) return false;
-      it->src = (uint32_t)(p * sa.img_slot) + (uint32_t)(u * 16) * c_step + (uint32_t)(f - (sa.box_bytes > 0 ? (f0 & ~15) : 0));
-      const int h0 = (int)sa.div_w.div((uint32_t)f);
-      const int w0 = f - h0 * args.W;
-      const int row0 = n * sa.rpi - tr.r0;  // window row of the image's grid row 0
-      const int plane_units = sa.plane_bytes >> 4;
-      uint32_t d[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int q = k ^ y;
-        // (W >= 4: a group crosses one row end at most)
-        const bool wrap = w0 + q >= args.W;
-        const int hp = h0 + (wrap ? 1 : 0) + args.pad_h, wp = w0 + q - (wrap ? args.W : 0) + args.pad_w;
-        const int ra = STRIDE == 1 ? 0 : (int)sa.row_index[hp & 1], cbi = STRIDE == 1 ? 0 : (int)sa.col_index[wp & 1];
-        const int j = row0 + (STRIDE == 1 ? hp : hp >> 1), jc = STRIDE == 1 ? wp : wp >> 1;
-        const bool stored = f + q >= f0 && f + q < f1 && jc < sa.pitch && (STRIDE == 1 || (ra >= 0 && cbi >= 0)) && j < tr.end - tr.r0;
-        d[k] = stored ? (uint32_t)((u * per_row + ra * sa.ndw + cbi) * plane_units + j * sa.pitch + jc) : kNoUnit;
-      }
-      it->dst[0] = d[0] | (d[1] << 16);
-      it->dst[1] = d[2] | (d[3] << 16);
-      return true;
-    };
-    auto build_item = [&](const Item& it, uint32_t raw_s, uint32_t win_s) {
+    auto build_item = [&](const StreamItem& it, uint32_t raw_s, uint32_t win_s) {
       const uint32_t a = raw_s + it.src;
       uint32_t px[4][4];
 #pragma unroll
@@ -402,24 +337,23 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       for (int q = 0; q < 4; ++q) {
         const uint32_t unit = (it.dst[q >> 1] >> (16 * (q & 1))) & 0xFFFFu;
         const uint32_t at = win_s + unit * 16u;
-        if (unit != kNoUnit && B2C_WINDOW_OK(args.dbg, 59, win_s, sa.win_bytes, at))
+        if (unit != kStreamNoUnit && B2C_WINDOW_OK(args.dbg, 59, win_s, sa.win_bytes, at))
           *reinterpret_cast<uint4*>(smem + at) = make_uint4(px[q][0], px[q][1], px[q][2], px[q][3]);
       }
     };
-    // Tiles that all start an image have their rows outside the images at the same places: zero from the start, never written.
-    const bool same_rows = sa.th % sa.rpi == 0;
-    Item kept[kKept];
+    const bool same_rows = stream_same_rows(sa);
+    StreamItem kept[kKept];
     uint32_t live = 0;  // bit i: kept[i] stores something
     for (int t = tile_first; t < tile_end && ok; t += tile_step) {
       B2C_STREAM_TILE(t)
       (void)ct;
-      const TileRows tr = tile_rows(args, sa, r0);
+      const TileRows tr = stream_tile_rows(args, sa, r0);
       const int rows = tr.end - tr.r0;
       // (then the places are those of the first tile; a tile that ends behind the batch builds units of outputs that do not exist)
       if (t == tile_first || !same_rows) live = 0;
 #pragma unroll
       for (int i = 0; i < kKept; ++i)
-        if ((t == tile_first || !same_rows) && make_item(tr, tid + i * kGroupWarps * 32, &kept[i])) live |= 1u << i;
+        if ((t == tile_first || !same_rows) && stream_item(args, sa, tr, tid + i * kGroupWarps * 32, y, STRIDE, &kept[i])) live |= 1u << i;
       for (int cb = 0; cb < sa.ncb; ++cb, next_window()) {
         if (turn != group) continue;
         ok = mbar_wait(smem_u32(&sc.win_empty[ws]), wph ^ 1u, ctl, args.status);
@@ -448,8 +382,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         for (int i = 0; i < kKept; ++i)
           if ((live >> i) & 1u) build_item(kept[i], raw_s, win_s);
         for (int e = tid + kKept * kGroupWarps * 32; e < items; e += kGroupWarps * 32) {
-          Item it;
-          if (make_item(tr, e, &it)) build_item(it, raw_s, win_s);
+          StreamItem it;
+          if (stream_item(args, sa, tr, e, y, STRIDE, &it)) build_item(it, raw_s, win_s);
         }
         // the raw rows have been read; the units are visible to the tensor cores' async proxy
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

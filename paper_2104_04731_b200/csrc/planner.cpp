@@ -14,6 +14,7 @@
 #include <utility>
 
 #include "b2c_internal.h"
+#include "stream_tile.h"
 
 namespace b2c {
 
@@ -846,20 +847,21 @@ bool stream_plan(const Geom& g, int tile_n, StreamArgs* sa, std::vector<uint64_t
   sa->plane_bytes = plane_units * 16;
   sa->win_bytes = (((f.planes - 1) * plane_units + std::max(plane_units, last_read)) * 16 + 127) / 128 * 128;
   if ((long long)f.ndh * f.ndw * plane_units > 16000) return false;  // (14 bits of the descriptor)
-  // images of a tile whose rows it needs, and the most raw rows of one (as tile_rows and raw_rows of the kernel; the
-  // tiles repeat after rpi of them)
+  // images of a tile whose rows it needs, and the most raw rows of one (the tiles repeat after rpi of them)
+  sa->div_rpi = make_fastdiv((uint32_t)f.rpi);
+  ConvArgs rows = {};  // (what the row functions read of it)
+  rows.H = d.H;
+  rows.pad_h = d.pad_h;
+  rows.out_P = g.P;
   int raw_rows = 0;
   const long long tiles_m = (total_rows + sa->th - 1) / sa->th;
   for (long long t = 0; t < std::min<long long>(tiles_m, f.rpi); ++t) {
-    const int r0 = (int)(t * sa->th), n_a = r0 / f.rpi;
-    const int last = (int)std::min<long long>(r0 + sa->th, total_rows) - 1, n_l = last / f.rpi;
-    const int end = std::max(r0, n_l * f.rpi + std::min(last - n_l * f.rpi, g.P - 1) + f.max_ri + 1);
-    for (int n = n_a; n * f.rpi < end; ++n) {
-      const int lo = std::max(0, (r0 - n * f.rpi) * sh - d.pad_h);
-      const int hi = std::min(d.H, (end - 1 - n * f.rpi) * sh + f.max_dh - d.pad_h + 1);
-      if (hi <= lo) continue;
-      sa->max_images = std::max(sa->max_images, n - n_a + 1);
-      raw_rows = std::max(raw_rows, hi - lo);
+    const TileRows tr = stream_tile_rows(rows, *sa, (int)(t * sa->th));
+    for (int n = tr.n_a; n * f.rpi < tr.end; ++n) {
+      const RawRows r = stream_raw_rows(rows, *sa, tr, n, sh);
+      if (r.hi <= r.lo) continue;
+      sa->max_images = std::max(sa->max_images, n - tr.n_a + 1);
+      raw_rows = std::max(raw_rows, r.hi - r.lo);
     }
   }
   if (sa->max_images < 1 || sa->max_images > 32) return false;
@@ -895,7 +897,6 @@ bool stream_plan(const Geom& g, int tile_n, StreamArgs* sa, std::vector<uint64_t
   if (ring == 6) return false;
   sa->smem = 128 + table_bytes + sa->win_stages * sa->win_bytes + sa->raw_stages * sa->raw_bytes + sa->b_stages * sa->b_stage_bytes;
   sa->pairs = kNumSMs / 2;
-  sa->div_rpi = make_fastdiv((uint32_t)f.rpi);
   sa->div_pitch = make_fastdiv((uint32_t)f.pitch);
   sa->div_w = make_fastdiv((uint32_t)d.W);
   sa->div_groups = make_fastdiv((uint32_t)sa->img_groups);

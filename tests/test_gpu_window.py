@@ -156,6 +156,28 @@ def test_stream_kernel(lib, case, out_layout, out_mode):
 
 
 @pytest.mark.parametrize("case", [
+    # N, C, H, W, K, R, S, pad, dil: stride 2, the last row of every image is read by no output
+    (64, 64, 15, 15, 128, 2, 2, 0, 1),
+    (64, 128, 13, 12, 128, 2, 2, 0, 1),
+    (60, 64, 17, 22, 96, 4, 3, (0, 1), 1),
+    (40, 96, 27, 20, 70, 6, 3, (0, 1), 1),
+    (50, 64, 21, 26, 64, 2, 2, 0, (3, 1)),
+])
+def test_stream_kernel_unread_last_row(lib, case):
+    """It belongs to no grid row of its image; stored, it would lie on the next image's first row."""
+    N, C, H, W, K, R, S, pad, dil = case
+    x = int8_uniform((N, C, H, W), 1097)
+    w = int8_uniform((K, C, R, S), 1098)
+    ref = oracle.conv2d_int8(x, w, 2, pad, dil, 9)
+    d = lib.make_desc(N, C, H, W, K, R, S, 2, pad, dil, 9, 0, 0, 3)
+    ids = [e.id for e in lib.enumerate_embeddings(d) if e.variant == b2c.VARIANT_IM2COL_WINDOW and e.tile_n >= 64]
+    assert ids
+    for i in ids:
+        for _ in range(3):
+            check_against_oracle(x, w, 2, pad, dil, 9, 3, i, ref=ref)
+
+
+@pytest.mark.parametrize("case", [
     # N, C, H, W, K, R, stride, pad: space to depth is a fifth or more faster than the plane kernel, and has a higher overhead
     (8, 93, 93, 9, 364, 3, 2, 1),
     (3, 96, 28, 14, 192, 3, 2, 1),
