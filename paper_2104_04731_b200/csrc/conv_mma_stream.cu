@@ -32,8 +32,8 @@ namespace b2c {
 
 namespace {
 
-constexpr int kGroups = 3, kGroupWarps = 4;  // builder groups, each with every third window
-constexpr int kBuilders = kGroups * kGroupWarps, kEpilogue = 8;
+constexpr int kGroupWarps = 4;  // of a builder group; stream_groups of the groups take windows in turn
+constexpr int kBuilders = kStreamGroups * kGroupWarps, kEpilogue = 8;
 constexpr int kFirstBuilder = 3, kFirstEpilogue = kFirstBuilder + kBuilders;
 constexpr int kStreamThreads = 32 * (kFirstEpilogue + kEpilogue);
 
@@ -283,12 +283,13 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     // groups of four warps work on consecutive windows side by side (1440 images of 256 x 14 x 14 -> 512, 3x3 stride 2, cool GPU:
     // one group of eight 222 us, three of four 115, and 80 with the items kept; two of six 92, three of five 82).
     const int group = (warp - kFirstBuilder) / kGroupWarps, bw = (warp - kFirstBuilder) % kGroupWarps, tid = bw * 32 + lane;
+    const int groups = stream_groups(sa);  // (a group past them takes no window)
     int turn = 0;  // the group whose window is next
     int rs = 0, ws = 0;
     uint32_t rph = 0, wph = 0;
     bool ok = true;
     auto next_window = [&]() {
-      if (++turn == kGroups) turn = 0;
+      if (++turn == groups) turn = 0;
       if (++rs == sa.raw_stages) {
         rs = 0;
         rph ^= 1u;

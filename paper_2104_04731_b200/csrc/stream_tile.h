@@ -47,6 +47,13 @@ B2C_HOST_DEVICE RawRows stream_raw_rows(const ConvArgs& args, const StreamArgs& 
   return r;
 }
 
+// Builder groups that take the windows in turn: no more than the ring has windows.  A wait tells the phases of a barrier apart
+// by parity only, so a group must not come to a buffer two uses ahead of the MMAs.  Window w, in a ring of S, waits for the
+// MMAs of w - S; that those of w - 2 S are through is known from the group's own last window, w - groups, which waited for
+// those of w - groups - S.  (With three groups and two buffers, a group overwrote windows that were still to be read.)
+constexpr int kStreamGroups = 3;
+B2C_HOST_DEVICE int stream_groups(const StreamArgs& sa) { return stream_min(kStreamGroups, sa.win_stages); }
+
 // The work of one builder thread on a window: four consecutive pixels of 16 channels.
 struct StreamItem {
   uint32_t src;     // byte offset of channel 0 of the group in the raw rows

@@ -1,8 +1,11 @@
 // Replays where the stream kernel's builder threads put the pixels of a layer, tile by tile, with the functions that the
 // kernel itself uses, and reports layers in which two threads store to one unit of a window or a tap reads anything
-// but its pixel (or, outside the image, zero).  Arguments: the number of random layers, then nothing; or one layer.
+// but its pixel (or, outside the image, zero).  Arguments: the number of random layers, or one layer.  "rings" instead runs
+// the waits of the window and raw rings in random orders.
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
+#include <map>
 #include <vector>
 
 #include "stream_tile.h"
@@ -103,33 +106,121 @@ int replay(const b2c_conv_desc& d, int tile_n) {
   return right ? 1 : 2;
 }
 
+unsigned long long g_random = 88172645463325252ull;  // xorshift64
+int pick(int lo, int hi) {
+  g_random ^= g_random << 13, g_random ^= g_random >> 7, g_random ^= g_random << 17;
+  return lo + (int)(g_random % (unsigned long long)(hi - lo + 1));
+}
+b2c_conv_desc random_layer() {
+  b2c_conv_desc d = {};
+  d.out_mode = B2C_OUT_I32;
+  d.N = pick(1, 40), d.C = 16 * pick(3, 8), d.H = pick(2, 60), d.W = pick(4, 60), d.K = pick(16, 64), d.R = pick(1, 6), d.S = pick(1, 5);
+  d.stride_h = d.stride_w = pick(1, 2);
+  d.pad_h = pick(0, 3), d.pad_w = pick(0, 3), d.dil_h = pick(1, 3), d.dil_w = pick(1, 3);
+  return d;
+}
+
+// A barrier as the waits see it: a wait for a parity passes when the phase in progress has the other one.
+struct Phases {
+  long long done = 0;
+  bool passes(long long use) const { return (done & 1) != (use & 1); }
+};
+
+// Windows of a block in the order of its roles, which advance in random order: the raw producer, the loads in flight, the
+// builder groups and the MMA warp.  False if a role gets past a wait before the phase that it waits for is complete.
+bool ring_waits_hold(const StreamArgs& sa) {
+  const int windows = 40, S = sa.win_stages, R = sa.raw_stages, groups = stream_groups(sa);
+  Phases win_full[4], win_empty[4], raw_full[4], raw_empty[4];
+  std::vector<int> loads;                       // windows whose raw rows are in flight
+  std::vector<int> next(groups), state(groups);  // window of each group; 0: waits for its buffer, 1: for its rows, 2: builds
+  for (int g = 0; g < groups; ++g) next[g] = g;
+  int produced = 0, consumed = 0;
+  std::vector<int> commits;  // windows whose MMAs are in flight
+  for (int step = 0; step < 4000 && consumed < windows; ++step) {
+    const int role = pick(0, groups + 3);
+    if (role < groups) {
+      const int g = role, w = next[g];
+      if (w >= windows) continue;
+      if (state[g] == 0) {
+        if (!win_empty[w % S].passes(w / S - 1)) continue;
+        if (win_empty[w % S].done < w / S) return false;
+        state[g] = 1;
+      } else if (state[g] == 1) {
+        if (!raw_full[w % R].passes(w / R)) continue;
+        if (raw_full[w % R].done < w / R + 1) return false;
+        state[g] = 2;
+      } else {
+        ++raw_empty[w % R].done;
+        ++win_full[w % S].done;
+        next[g] = w + groups;
+        state[g] = 0;
+      }
+    } else if (role == groups) {
+      const int w = produced;
+      if (w >= windows || !raw_empty[w % R].passes(w / R - 1)) continue;
+      if (raw_empty[w % R].done < w / R) return false;
+      loads.push_back(w);
+      ++produced;
+    } else if (role == groups + 1) {
+      if (loads.empty()) continue;
+      const int i = pick(0, (int)loads.size() - 1);  // copies complete in any order
+      ++raw_full[loads[i] % R].done;
+      loads.erase(loads.begin() + i);
+    } else if (role == groups + 2) {
+      const int w = consumed;
+      if (!win_full[w % S].passes(w / S)) continue;
+      if (win_full[w % S].done < w / S + 1) return false;
+      commits.push_back(w);
+      ++consumed;
+    } else if (!commits.empty()) {
+      ++win_empty[commits.front() % S].done;
+      commits.erase(commits.begin());
+    }
+  }
+  return consumed == windows;
+}
+
+// Every pair of ring lengths that the planner gives to random layers.
+int rings() {
+  std::map<std::pair<int, int>, StreamArgs> seen;
+  for (int i = 0; i < 50000; ++i) {
+    const b2c_conv_desc d = random_layer();
+    Geom g;
+    StreamArgs sa;
+    if (resolve_geom(&d, &g) == B2C_OK && stream_plan(g, 64 << pick(0, 2), &sa)) seen[{sa.win_stages, sa.raw_stages}] = sa;
+  }
+  int wrong = 0;
+  for (const auto& s : seen) {
+    bool holds = true;
+    for (int i = 0; i < 20000 && holds; ++i) holds = ring_waits_hold(s.second);
+    std::printf("%d windows, %d raw buffers, %d groups: %s\n", s.first.first, s.first.second, stream_groups(s.second),
+                holds ? "every wait holds" : "a wait passes early");
+    wrong += !holds;
+  }
+  return wrong || seen.size() < 3 ? 1 : 0;
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
+  if (argc == 2 && !std::strcmp(argv[1], "rings")) return rings();
   int seen[3] = {0, 0, 0};
-  b2c_conv_desc d = {};
-  d.out_mode = B2C_OUT_I32;
-  auto layer = [&](int N, int C, int H, int W, int K, int R, int S, int stride, int ph, int pw, int dh, int dw) {
-    d.N = N, d.C = C, d.H = H, d.W = W, d.K = K, d.R = R, d.S = S;
-    d.stride_h = d.stride_w = stride;
-    d.pad_h = ph, d.pad_w = pw, d.dil_h = dh, d.dil_w = dw;
+  auto layer = [&](const b2c_conv_desc& d) {
     int tile_n = 64;
-    while (tile_n < K && tile_n < 256) tile_n <<= 1;
+    while (tile_n < d.K && tile_n < 256) tile_n <<= 1;
     ++seen[replay(d, tile_n)];
   };
   if (argc == 13) {
     int v[12];
     for (int i = 0; i < 12; ++i) v[i] = std::atoi(argv[i + 1]);
-    layer(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8], v[9], v[10], v[11]);
+    b2c_conv_desc d = {};
+    d.out_mode = B2C_OUT_I32;
+    d.N = v[0], d.C = v[1], d.H = v[2], d.W = v[3], d.K = v[4], d.R = v[5], d.S = v[6];
+    d.stride_h = d.stride_w = v[7];
+    d.pad_h = v[8], d.pad_w = v[9], d.dil_h = v[10], d.dil_w = v[11];
+    layer(d);
   } else {
-    unsigned long long x = 88172645463325252ull;  // xorshift64
-    auto pick = [&](int lo, int hi) {
-      x ^= x << 13, x ^= x >> 7, x ^= x << 17;
-      return lo + (int)(x % (unsigned long long)(hi - lo + 1));
-    };
-    for (int i = argc > 1 ? std::atoi(argv[1]) : 1000; i > 0; --i)
-      layer(pick(1, 40), 16 * pick(3, 8), pick(2, 60), pick(4, 60), pick(16, 64), pick(1, 6), pick(1, 5), pick(1, 2), pick(0, 3), pick(0, 3), pick(1, 3),
-            pick(1, 3));
+    for (int i = argc > 1 ? std::atoi(argv[1]) : 1000; i > 0; --i) layer(random_layer());
   }
   std::printf("layers: %d right, %d wrong, %d of other kernels\n", seen[1], seen[2], seen[0]);
   return seen[2] ? 1 : 0;

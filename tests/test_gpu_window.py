@@ -141,6 +141,7 @@ def test_plane_kernel_reads_the_last_incomplete_16_bytes(lib):
     (60, 48, 12, 20, 256, 4, 1, 1, 2, 1, 9),        # half a block of channels, padding wider than the taps need
     (400, 64, 14, 14, 512, 3, 3, 2, 1, 1, 10),      # several tiles a pair: both accumulators, rings that run on
     (2, 48, 112, 126, 64, 3, 3, 1, 1, 1, 9),        # one grid row of 127 positions a tile
+    (34, 112, 44, 40, 32, 5, 5, 2, 2, 1, 11),       # rings of two windows, several tiles of four windows each
 ])
 @pytest.mark.parametrize("out_layout,out_mode", [(0, 3), (1, 2)])
 def test_stream_kernel(lib, case, out_layout, out_mode):

@@ -1,5 +1,6 @@
 """The stream kernel's placement of pixels (csrc/stream_tile.h), replayed on the host for random layers: no unit of a window
-has two writers, and every tap of every output reads its pixel, or zero outside the image."""
+has two writers, and every tap of every output reads its pixel, or zero outside the image.  And the waits of its rings,
+whose barriers tell phases apart by parity only, with the roles in random order."""
 import os
 import subprocess
 
@@ -37,3 +38,8 @@ def test_random_layers(replay):
 def test_even_filters_with_stride_two(replay, layer):
     r = replay(*layer)
     assert r.returncode == 0 and "1 right" in r.stdout, r.stdout + r.stderr
+
+
+def test_ring_waits(replay):
+    r = replay("rings")
+    assert r.returncode == 0 and "2 windows" in r.stdout, r.stdout + r.stderr
