@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
       const uint32_t row_off = (uint32_t)row * 128u;
       const uint32_t xr = (uint32_t)(row & 7);
       for (int kb = kb_begin; kb < kb_end; ++kb) {
-        if (!mbar_wait(smem_u32(&ctl.empty[s]), ph ^ 1u, &ctl, args.status)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl.empty[s]), ph ^ 1u, &ctl, args.status))) {
           ok = false;
           break;
         }
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
       const uint32_t row_off = (uint32_t)row * 128u;
       const uint32_t xr = (uint32_t)(row & 7);
       for (int kb = kb_begin; kb < kb_end; ++kb) {
-        if (!mbar_wait(smem_u32(&ctl.empty[s]), ph ^ 1u, &ctl, args.status)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl.empty[s]), ph ^ 1u, &ctl, args.status))) {
           ok = false;
           break;
         }
@@ -631,7 +631,7 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
     // ---- epilogue ----
     const int buf = persistent ? (ti & (nbuf - 1)) : 0;
     const uint32_t use = persistent ? (uint32_t)(ti >> nbuf_log2) : 0u;
-    if (ok) ok = mbar_wait(smem_u32(&ctl.tmem_full[buf]), use & 1u, &ctl, args.status);
+    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl.tmem_full[buf]), use & 1u, &ctl, args.status));
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (ok) {
       // Output index of (m, k): NKPQ -> (n*K + k)*PQ + pq ; NPQK -> m*K + k.

@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(PACK ? kThreads + kPackGroup : kThreads, PERSI
       }
       const int buf = persistent ? (ti & (nbuf - 1)) : 0;
       const uint32_t use = persistent ? (uint32_t)(ti / nbuf) : 0u;
-      ok = mbar_wait(smem_u32(&ctl.tmem_full[buf]), use & 1u, &ctl, args.status);
+      ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl.tmem_full[buf]), use & 1u, &ctl, args.status));
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (ok) {
         const long long base_nkpq = (long long)out_img * args.y_stride_n + out_pq;

@@ -377,9 +377,12 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
       sph ^= 1u;
       return met;
     };
-    for (int seg = seg_first; seg < seg_end && ok; seg += seg_step) {
+    // After a wait that gave up, a warp leaves a window by vote and the role where a segment begins, so that its lanes stay
+    // together; what it still builds and arrives on is of no use to anyone, and harmless.  (ok is a lane's own.)
+    for (int seg = seg_first; seg < seg_end; seg += seg_step) {
+    if (__any_sync(0xffffffffu, ctl->abort_flag != 0)) break;
     const SegRows blk = seg_rows(args, pl, seg);
-    for (int win = 0; win < blk.windows && ok; ++win) {
+    for (int win = 0; win < blk.windows; ++win) {
       const WindowSpan sp = window_span<LEAD>(args, pl, blk, win);
       ok = mbar_wait_sleep(smem_u32(&pc.win_empty[ws]), wph ^ 1u, ctl, args.status, kSleepWindow);
       if (!__all_sync(0xffffffffu, ok)) break;
@@ -685,7 +688,6 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
         rph ^= 1u;
       }
       }
-      if (!ok) break;
       // the units are visible to the tensor core's async proxy
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
@@ -706,12 +708,13 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
     const int pitch = pl.pitch;
     const int step_j = kTileM / pitch, step_q = kTileM - step_j * pitch;  // a tile further: rows and columns
     const int row_j = (int)pl.div_pitch.div((uint32_t)row), row_q = row - row_j * pitch;
-    bool ok = true;
     int buf = 0, ti = 0;
     uint32_t aph = 0;
-    for (int seg = seg_first; seg < seg_end && ok; seg += seg_step) {
+    // (As the builders; tiles after a wait that gave up are drained as they are, and the status says so.)
+    for (int seg = seg_first; seg < seg_end; seg += seg_step) {
+    if (__any_sync(0xffffffffu, ctl->abort_flag != 0)) break;
     const SegRows blk = seg_rows(args, pl, seg);
-    for (int win = 0; win < blk.windows && ok; ++win) {
+    for (int win = 0; win < blk.windows; ++win) {
       const WindowSpan sp = window_span<LEAD>(args, pl, blk, win);
       const int positions = sp.rows * pitch;
       const int tiles = (positions + sp.lead + kTileM - 1) / kTileM;
@@ -726,9 +729,8 @@ __global__ void __launch_bounds__(64 + 32 * (KB + KE), MINB)
           if constexpr (LEAD)  // (one comparison: positions before the window wrap to large values)
             row_valid = (unsigned)(t * kTileM + row - sp.lead) < (unsigned)positions && q < args.out_Q && i < args.out_P;
           const int out_pq = i * args.out_Q + q;
-          ok = mbar_wait(smem_u32(&pc.acc_full[buf]), aph, ctl, args.status);
+          (void)mbar_wait(smem_u32(&pc.acc_full[buf]), aph, ctl, args.status);
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          if (!ok) break;
           const long long base_nkpq = (long long)n * args.y_stride_n + out_pq + (long long)grp * args.K * args.out_PQ;
           const long long base_npqk = ((long long)n * args.out_PQ + out_pq) * args.K;
           const uint32_t taddr = tmem_acc + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * args.tile_n);

@@ -357,8 +357,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         if ((t == tile_first || !same_rows) && stream_item(args, sa, tr, tid + i * kGroupWarps * 32, y, STRIDE, &kept[i])) live |= 1u << i;
       for (int cb = 0; cb < sa.ncb; ++cb, next_window()) {
         if (turn != group) continue;
-        ok = mbar_wait(smem_u32(&sc.win_empty[ws]), wph ^ 1u, ctl, args.status);
-        if (!__all_sync(0xffffffffu, ok)) break;
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sc.win_empty[ws]), wph ^ 1u, ctl, args.status));
+        if (!ok) break;
         const uint32_t win_s = (uint32_t)(ws * sa.win_bytes);
         // rows outside the image (a buffer's later windows of the tile find them cleared)
         if (!same_rows && cb < sa.win_stages) {
@@ -376,8 +376,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
                 }
           }
         }
-        ok = mbar_wait(smem_u32(&sc.raw_full[rs]), rph, ctl, args.status);
-        if (!__all_sync(0xffffffffu, ok)) break;
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sc.raw_full[rs]), rph, ctl, args.status));
+        if (!ok) break;
         const uint32_t raw_s = raw_off + (uint32_t)(rs * sa.raw_bytes);
 #pragma unroll
         for (int i = 0; i < kKept; ++i)
@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       const bool row_valid = j < sa.th && q < args.out_Q && i < args.out_P && n < sa.images;
       const int out_pq = i * args.out_Q + q;
       const int buf = ti & 1;
-      ok = mbar_wait(smem_u32(&sc.acc_full[buf]), (uint32_t)((ti >> 1) & 1), ctl, args.status);
+      ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sc.acc_full[buf]), (uint32_t)((ti >> 1) & 1), ctl, args.status));
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (!ok) break;
       const long long base_nkpq = (long long)n * args.y_stride_n + out_pq;

@@ -232,8 +232,8 @@ __global__ void __launch_bounds__(kWinThreads, 2)
     for (int t = tile_first; t < tile_end && ok; t += tile_step, ++ti) {
       const int ab = ti & (kABufs - 1);
       const uint32_t a_use = (uint32_t)(ti / kABufs);
-      ok = mbar_wait_relaxed(smem_u32(&wc.a_empty[ab]), (a_use & 1u) ^ 1u, ctl, args.status);
-      if (ok) ok = mbar_wait_relaxed(smem_u32(&wc.win_full[s]), ph, ctl, args.status);
+      ok = __all_sync(0xffffffffu, mbar_wait_relaxed(smem_u32(&wc.a_empty[ab]), (a_use & 1u) ^ 1u, ctl, args.status));
+      if (ok) ok = __all_sync(0xffffffffu, mbar_wait_relaxed(smem_u32(&wc.win_full[s]), ph, ctl, args.status));
       if (!ok) break;
       if (LINEAR) {
         // this row's pixel (n, p, q); rows past the last pixel build from the window's first image (never stored)
@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(kWinThreads, 2)
       }
       const int tb = ti & (nbuf - 1);
       const uint32_t t_use = (uint32_t)(ti >> nbuf_log2);
-      ok = mbar_wait_relaxed(smem_u32(&wc.tmem_full[tb]), t_use & 1u, ctl, args.status);
+      ok = __all_sync(0xffffffffu, mbar_wait_relaxed(smem_u32(&wc.tmem_full[tb]), t_use & 1u, ctl, args.status));
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (!ok) break;
       const long long base_nkpq = (long long)img * args.y_stride_n + out_pq;
