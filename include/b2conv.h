@@ -369,6 +369,14 @@ int b2c_test_shrink_checked_ranges(long long bytes);
  * needed it returns B2C_E_CUDA); n = 0 disarms.  Nothing on the device is touched. */
 int b2c_test_fail_nth_encode(int n);
 
+/* Test hook (no counterpart in the paper): which kernel runs embedding `id` of the enumeration, where
+ * its fields do not tell.  *kernel = B2C_KERNEL_*; INVALID_ARG for an id that is not listed. */
+#define B2C_KERNEL_OTHER 0      /* the variant's own kernel                                                */
+#define B2C_KERNEL_PLANE 1      /* window unroll from planes of 16-byte units                              */
+#define B2C_KERNEL_PLANE_LEAD 2 /* the same, tiles begin before their window so that stores start a sector */
+#define B2C_KERNEL_STREAM 3     /* the same units on two SMs, weights streamed                             */
+int b2c_test_kernel_of(const b2c_conv_desc* desc, int32_t id, int32_t* kernel);
+
 const char* b2c_status_string(int status);
 
 /* The last CUDA error code (cudaError_t or CUresult as int) seen by this thread's failing call. */

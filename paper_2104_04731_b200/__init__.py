@@ -35,7 +35,7 @@ EXPORTS = [
     "b2c_plan_device_status", "b2c_selftest_bounded_wait", "b2c_plan_destroy", "b2c_pack_activations", "b2c_im2col", "b2c_im2col_noalloc",
     "b2c_status_string",
     "b2c_last_cuda_error", "b2c_oneshot_status", "b2c_oneshot_cache_clear", "b2c_test_fail_nth_encode", "b2c_selftest_pack_wait", "b2c_measure_mma_rate", "b2c_measure_mma_rate_pair", "b2c_debug_build", "b2c_plan_debug_info",
-    "b2c_plan_check_canaries", "b2c_test_shrink_checked_ranges",
+    "b2c_plan_check_canaries", "b2c_test_shrink_checked_ranges", "b2c_test_kernel_of",
 ]
 
 
@@ -119,6 +119,7 @@ def load():
     lib.b2c_measure_mma_rate_pair.argtypes = [i32, i32, ctypes.POINTER(ctypes.c_float), ctypes.POINTER(ctypes.c_float), vp]
     lib.b2c_oneshot_cache_clear.argtypes = []
     lib.b2c_test_fail_nth_encode.argtypes = [i32]
+    lib.b2c_test_kernel_of.argtypes = [pd, i32, pi32]
     for name in EXPORTS:
         fn = getattr(lib, name)
         if name not in ("b2c_plan_destroy", "b2c_status_string"):
@@ -345,6 +346,16 @@ def oneshot_cache_clear():
 def test_fail_nth_encode(n: int):
     """Host-side fault injection: the n-th tensor-map encode from now on fails (0 disarms)."""
     _check(load().b2c_test_fail_nth_encode(n), "b2c_test_fail_nth_encode")
+
+
+KERNEL_OTHER, KERNEL_PLANE, KERNEL_PLANE_LEAD, KERNEL_STREAM = 0, 1, 2, 3
+
+
+def test_kernel_of(desc: ConvDesc, emb_id: int) -> int:
+    """Test hook: the kernel (KERNEL_*) that runs embedding ``emb_id`` of the enumeration."""
+    k = ctypes.c_int32()
+    _check(load().b2c_test_kernel_of(ctypes.byref(desc), emb_id, ctypes.byref(k)), "b2c_test_kernel_of")
+    return k.value
 
 
 def conv2d_int8_host(x, w, stride=1, pad=0, dilation=1, shift=0, y32=None, y8=None):

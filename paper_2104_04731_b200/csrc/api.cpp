@@ -815,6 +815,24 @@ int b2c_enumerate(const b2c_conv_desc* desc, b2c_embedding* out, int32_t cap, in
   return all.empty() ? B2C_E_UNSUPPORTED : B2C_OK;
 }
 
+int b2c_test_kernel_of(const b2c_conv_desc* desc, int32_t id, int32_t* kernel) {
+  if (!desc || !kernel) return B2C_E_INVALID_ARG;
+  Geom g;
+  const int rc = resolve_geom(desc, &g);
+  if (rc != B2C_OK) return rc;
+  std::vector<Candidate> all;
+  enumerate_legal(g, &all);
+  if (id < 0 || id >= (int)all.size()) return B2C_E_INVALID_ARG;
+  const int schedule = all[id].schedule;
+  PlaneArgs pl;
+  *kernel = B2C_KERNEL_OTHER;
+  if (schedule == kStreamSchedule)
+    *kernel = B2C_KERNEL_STREAM;
+  else if (schedule >= 0 && plane_plan(g, 1, schedule, &pl))
+    *kernel = pl.lead_mask ? B2C_KERNEL_PLANE_LEAD : B2C_KERNEL_PLANE;
+  return B2C_OK;
+}
+
 int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_stream, b2c_plan** out) {
   if (!desc || !out) return B2C_E_INVALID_ARG;
   *out = nullptr;

@@ -113,6 +113,8 @@ def test_plane_kernel_aligned_stores(lib, case):
     d = lib.make_desc(N, C, H, W, K, R, R, stride, pad, 1, 8, out_mode=out_mode)
     ids = [e.id for e in lib.enumerate_embeddings(d) if e.variant == b2c.VARIANT_IM2COL_WINDOW]
     assert len(ids) > 1
+    # (the row form, fewer than 8 channels, begins tiles before their windows)
+    assert (C < 8) == any(lib.test_kernel_of(d, i) == b2c.KERNEL_PLANE_LEAD for i in ids)
     for i in ids:
         check_against_oracle(x, w, stride, pad, 1, 8, out_mode, i, ref=ref)
 
@@ -137,7 +139,7 @@ def test_plane_kernel_reads_the_last_incomplete_16_bytes(lib):
     (130, 64, 7, 7, 64, 3, 3, 1, 1, 1, 9),          # H * W odd: unaligned words
     (21, 80, 28, 28, 96, 3, 3, 1, 1, 1, 10),        # one tiled copy per image part; ragged last block of 16 channels
     (9, 96, 44, 40, 70, 5, 5, 2, 2, 1, 11),         # 25 MMAs a block: weight stages that end inside one
-    (11, 64, 30, 52, 300, 2, 3, 1, (0, 1), 3, 9),   # dilation 3, six taps, padding on one axis
+    (11, 64, 28, 52, 300, 2, 3, 1, (0, 1), 3, 9),   # dilation 3, six taps, padding on one axis (30 rows are no form of this kernel)
     (60, 48, 12, 20, 256, 4, 1, 1, 2, 1, 9),        # half a block of channels, padding wider than the taps need
     (400, 64, 14, 14, 512, 3, 3, 2, 1, 1, 10),      # several tiles a pair: both accumulators, rings that run on
     (2, 48, 112, 126, 64, 3, 3, 1, 1, 1, 9),        # one grid row of 127 positions a tile
@@ -151,7 +153,7 @@ def test_stream_kernel(lib, case, out_layout, out_mode):
     ref = oracle.conv2d_int8(x, w, stride, pad, dil, shift)
     d = lib.make_desc(N, C, H, W, K, R, S, stride, pad, dil, shift, 0, out_layout, out_mode)
     ids = [e.id for e in lib.enumerate_embeddings(d) if e.variant == b2c.VARIANT_IM2COL_WINDOW and e.tile_n >= 64]
-    assert ids
+    assert any(lib.test_kernel_of(d, i) == b2c.KERNEL_STREAM for i in ids)
     for i in ids:
         check_against_oracle(x, w, stride, pad, dil, shift, out_mode, i, ref=ref, out_layout=out_layout)
 
@@ -171,7 +173,7 @@ def test_stream_kernel_unread_last_row(lib, case):
     w = int8_uniform((K, C, R, S), 1098)
     ref = oracle.conv2d_int8(x, w, 2, pad, dil, 9)
     d = lib.make_desc(N, C, H, W, K, R, S, 2, pad, dil, 9, 0, 0, 3)
-    ids = [e.id for e in lib.enumerate_embeddings(d) if e.variant == b2c.VARIANT_IM2COL_WINDOW and e.tile_n >= 64]
+    ids = [e.id for e in lib.enumerate_embeddings(d) if lib.test_kernel_of(d, e.id) == b2c.KERNEL_STREAM]
     assert ids
     for i in ids:
         for _ in range(3):
