@@ -71,11 +71,11 @@ __device__ __forceinline__ void mma_i8_pair_list4(uint32_t d_tmem, uint64_t a0, 
       : "memory");
 }
 
-// Debug build: is the unit at this offset in shared memory inside the window of `bytes` bytes at `lo`?
+// Debug build: do the n bytes at this offset in shared memory lie inside the `bytes` bytes at `lo`?
 #ifdef B2C_DEBUG_BOUNDS
-#define B2C_WINDOW_OK(d, site, lo, bytes, at) b2c_dbg_in_range((d).status, site, smem + (lo), bytes, smem + (at), 16)
+#define B2C_SMEM_OK(d, site, lo, bytes, at, n) b2c_dbg_in_range((d).status, site, smem + (lo), bytes, smem + (at), n)
 #else
-#define B2C_WINDOW_OK(d, site, lo, bytes, at) true
+#define B2C_SMEM_OK(d, site, lo, bytes, at, n) true
 #endif
 
 // STRIDE 1 or 2 on both axes.  WORDS: H * W is a multiple of 4, so four consecutive pixels of a channel are one word.
@@ -258,7 +258,10 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         const int channels = min(32, args.C - cb * 32);
         const int8_t* src = args.x + (size_t)n * args.x_stride_n + (size_t)(cb * 32) * HW;
         bool copy = mine;
-        if (mine && !B2C_X_OK(args.dbg, 57, src + rr.lo * args.W, (long long)(channels - 1) * HW + (rr.hi - rr.lo) * args.W)) copy = false;
+        // (what the copy reads: whole channels, or the rows and what their tensor map clips)
+        if (mine && !(sa.box_bytes > 0 ? B2C_X_OK(args.dbg, 57, src + rr.lo * args.W, (long long)(channels - 1) * HW + (rr.hi - rr.lo) * args.W)
+                                       : B2C_X_OK(args.dbg, 57, src, (long long)channels * HW)))
+          copy = false;
         const uint32_t bytes = !copy ? 0u : (uint32_t)(sa.box_bytes > 0 ? 32 * sa.box_bytes : channels * HW);
         const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
         mbar_arrive_expect_tx(full, total, leader_lane);
@@ -313,6 +316,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     const uint32_t sel_c = (y & 1) ? 0x7632u : 0x5410u, sel_d = (y & 1) ? 0x5410u : 0x7632u;
     auto build_item = [&](const StreamItem& it, uint32_t raw_s, uint32_t win_s) {
       const uint32_t a = raw_s + it.src;
+      // (the second word of an unaligned pixel group may lie behind the stage: it is read, not used)
+      if (!B2C_SMEM_OK(args.dbg, 60, raw_s, sa.raw_bytes + 8, a & ~3u, 15 * c_step + (WORDS ? 4u : 8u))) return;
       uint32_t px[4][4];
 #pragma unroll
       for (int k4 = 0; k4 < 4; ++k4) {
@@ -338,7 +343,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       for (int q = 0; q < 4; ++q) {
         const uint32_t unit = (it.dst[q >> 1] >> (16 * (q & 1))) & 0xFFFFu;
         const uint32_t at = win_s + unit * 16u;
-        if (unit != kStreamNoUnit && B2C_WINDOW_OK(args.dbg, 59, win_s, sa.win_bytes, at))
+        if (unit != kStreamNoUnit && B2C_SMEM_OK(args.dbg, 59, win_s, sa.win_bytes, at, 16))
           *reinterpret_cast<uint4*>(smem + at) = make_uint4(px[q][0], px[q][1], px[q][2], px[q][3]);
       }
     };
@@ -372,7 +377,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
               for (int b = 0; b < sa.ndw; ++b)
                 for (int q = lane; q < sa.pitch; q += 32) {
                   const uint32_t at = win_s + (uint32_t)((u * per_row + a * sa.ndw + b) * sa.plane_bytes) + (uint32_t)(j * sa.pitch + q) * 16u;
-                  if (B2C_WINDOW_OK(args.dbg, 58, win_s, sa.win_bytes, at)) *reinterpret_cast<uint4*>(smem + at) = make_uint4(0, 0, 0, 0);
+                  if (B2C_SMEM_OK(args.dbg, 58, win_s, sa.win_bytes, at, 16)) *reinterpret_cast<uint4*>(smem + at) = make_uint4(0, 0, 0, 0);
                 }
           }
         }
