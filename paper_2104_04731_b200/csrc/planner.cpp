@@ -569,7 +569,7 @@ double plane_schedule(const Geom& g, int groups, const PlaneForm& f, int per_sm,
         spi = (int)((g.P + share - 1) / share);
         blocks = (int)std::min<long long>(places, (long long)d.N * spi);
       }
-      if (whole_sectors && (spi == 0 ? g.Q % kSectorOutputs != 0 : spi > 1 && share % step != 0)) continue;
+      if (whole_sectors && (spi == 0 ? g.Q % outputs != 0 : spi > 1 && share % step != 0)) continue;
       // (a window in the middle of an image that does not start on a boundary)
       const int lead_mask = spi > 0 && max_lead > 0 && ((long long)th * g.Q % outputs != 0 || share * g.Q % outputs != 0) ? max_lead : 0;
       const double active = (double)blocks * share * f.pitch * d.K * groups * out_bytes;
