@@ -101,25 +101,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, SharedC
   return mbar_wait_slow(bar, parity, ctl, status);
 }
 
-// Bounded wait with back-off: polling a barrier takes the same shared-memory pipe as the builders' and the
-// epilogue's loads and stores, and most warps of the plane kernels wait for whole windows (microseconds), so a warp that
-// finds its barrier not ready sleeps between polls.  (Waits for a tile poll: sleeping there costs 2 to 5 us a call.)
-__device__ __forceinline__ bool mbar_wait_sleep(uint32_t bar, uint32_t parity, SharedCtl* ctl, int* status, unsigned ns) {
-  if (mbar_try_wait(bar, parity)) return true;
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
-  while (true) {
-    __nanosleep(ns);
-    if (mbar_try_wait(bar, parity)) return true;
-    if (ctl->abort_flag) return false;
-    if (global_ns() - t0 > kWaitLimitNs) {
-      ctl->abort_flag = 1;
-      atomicCAS(status, 0, B2C_E_TIMEOUT);
-      return false;
-    }
-  }
-}
-
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar,
                                             uint32_t on) {
   asm volatile(

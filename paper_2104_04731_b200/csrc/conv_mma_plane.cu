@@ -79,6 +79,25 @@ __device__ __forceinline__ void mma_i8_list4(uint32_t d_tmem, uint64_t a0, uint6
       : "memory");
 }
 
+// Bounded wait with back-off: polling a barrier takes the same shared-memory pipe as the builders' and the
+// epilogue's loads and stores, and most warps of this kernel wait for whole windows (microseconds), so a warp that
+// finds its barrier not ready sleeps between polls.  (Waits for a tile poll: sleeping there costs 2 to 5 us a call.)
+__device__ __forceinline__ bool mbar_wait_sleep(uint32_t bar, uint32_t parity, SharedCtl* ctl, int* status, unsigned ns) {
+  if (mbar_try_wait(bar, parity)) return true;
+  if (mbar_try_wait(bar, parity)) return true;
+  const unsigned long long t0 = global_ns();
+  while (true) {
+    __nanosleep(ns);
+    if (mbar_try_wait(bar, parity)) return true;
+    if (ctl->abort_flag) return false;
+    if (global_ns() - t0 > kWaitLimitNs) {
+      ctl->abort_flag = 1;
+      atomicCAS(status, 0, B2C_E_TIMEOUT);
+      return false;
+    }
+  }
+}
+
 // Debug build: is the unit at this offset in shared memory inside the window of `bytes` bytes at `lo`?
 #ifdef B2C_DEBUG_BOUNDS
 #define B2C_WINDOW_OK(d, site, lo, bytes, at) b2c_dbg_in_range((d).status, site, smem + (lo), bytes, smem + (at), 16)
