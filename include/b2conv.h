@@ -95,7 +95,10 @@ typedef struct {
                                       * dilation): the input becomes planes of 16-byte units in shared memory and a tap is a
                                       * start address into them; listed once per schedule worth timing (entries that may differ in
                                       * no field but the id), beside the first form where both apply.
-                                      * Weights stay resident in shared memory */
+                                      * Weights stay resident in shared memory in both.  From 48 channels and four taps on (NCHW,
+                                      * stride 1 or 2) the same units are also built 32 channels at a time by a pair of SMs that
+                                      * share a tile of 256 positions (tile_m is 128, the rows of one block), with weights
+                                      * that stream; one or two entries */
 
 typedef struct {
   int32_t id;       /* index in the enumeration for this descriptor; pass to b2c_plan_create      */

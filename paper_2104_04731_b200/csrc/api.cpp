@@ -60,8 +60,8 @@ struct b2c_plan {
   long long x_stride_n_whole = 0, y_stride_n_whole = 0;  // sub-plans: batch strides of the whole tensors
   struct HostPipe* pipe = nullptr;  // streaming host-buffer calls: created by the first b2c_plan_run_host_async
   // The two-SM persistent channel-pack schedule can run the activation pack inside the MMA kernel
-  // (NCHW input whose rows have a bulk-copy form): run then launches one kernel, preceded by a memset
-  // of the work counters, which live in the workspace after the rewritten operand.
+  // (NCHW input whose rows have a bulk-copy form): run then launches one kernel, preceded by a small
+  // one that zeroes the work counters, which live in the workspace after the rewritten operand.
   bool fused_pack = false;
   size_t ws_ctl_offset = 0;  // bytes from the workspace start to the counters [1 + N] int
   int dbg_site = 0;          // debug build: site and byte offset of the last reported out-of-range access
@@ -434,7 +434,7 @@ void enumerate_legal(const Geom& g, std::vector<Candidate>* all) {
   for (size_t i = 0; i < all->size(); ++i) (*all)[i].id = (int)i;
 }
 
-// schedule: that of the plane kernel if it is the one to run the embedding, else -1.
+// schedule: as Candidate::schedule.
 int create_plan_for(const Geom& g, const b2c_embedding& emb, int schedule, b2c_plan** out, int group_count = 1) {
   b2c_plan* p = new (std::nothrow) b2c_plan();
   if (!p) return B2C_E_INVALID_ARG;

@@ -370,7 +370,7 @@ int cp_block_bytes(int C_pad);       // reduction bytes per block for the channe
 int im2col_k_pad(int Kg);            // padded reduction length for the stencil-unroll maps
 // An embedding and, for the window unroll, which kernel runs it.
 struct Candidate : b2c_embedding {
-  int schedule;  // plane kernel: index of its schedule (plane_plan); -1: any other kernel, the window kernel among them
+  int schedule;  // plane kernel: index of its schedule (plane_plan); kStreamSchedule: stream kernel; -1: any other, the window kernel among them
 };
 void enumerate_embeddings(const Geom& g, std::vector<Candidate>* out);
 int pick_by_policy(const std::vector<Candidate>& all, int policy);  // index or -1

@@ -29,9 +29,9 @@
 // resident.
 // What bounds it now: the stores of the results (4 to 5 cycles of the SM's store path per 128 bytes; runs of 32 lanes that start
 // inside a sector cost the memory side more, see plane_sector_rows) beside the builders' shared-memory traffic.  Before (operand
-// rows written out by builder warps, or a rewrite through memory) and after: 64 images of 3 x 227 x 227, 7x7 stride 2, 64 channels 97 -> 52 us; 32 of 1 x 700 x 161,
-// 20x5 stride 2, 76 -> 30; 15501 of 16 x 14 x 14, 3x3, 125 -> 95; 315 of 64 x 56 x 56, 3x3, 99 -> 79; tiles on sector
-// boundaries: 51.6 -> 49.2 and 79.2 -> 73.6 us of these.
+// rows written out by builder warps, or a rewrite through memory) and after: 64 images of 3 x 227 x 227, 7x7 stride 2, 64 channels 97 -> 49 us; 32 of 1 x 700 x 161,
+// 20x5 stride 2, 76 -> 30; 15501 of 16 x 14 x 14, 3x3, 125 -> 95; 315 of 64 x 56 x 56, 3x3, 99 -> 74 (of the first and the last,
+// tiles on sector boundaries gave 51.6 -> 49.2 and 79.2 -> 73.6).
 // Copies of window w + 2, units of w + 1, MMAs of w and stores of w - 1 overlap.  Every wait is
 // bounded as in the other kernels.
 #include <algorithm>

@@ -8,10 +8,11 @@
 // a clock from there, the pair schedule needs 64 per MMA clock), and the rewrite's stores disturb those loads.  Here the
 // input is read once per column tile, as it lies in memory, and only the weights stream: 32 bytes per MMA clock, 11 more
 // for the raw rows.  What it pays is the overhang of the position grid (7 x 7 outputs with stride 2: 49 of 64 positions).
-// Measured, channel pack and its pair schedules before, this kernel now: 128 images of 256 x 7 x 7 -> 512, 3x3, 19.5 -> 13.7 us;
-// 40 of 160 x 20 x 44 -> 130, 5x5, 64.7 -> 38.8; 64 of 96 x 28 x 28 -> 192, 5x5, 43.4 -> 30.2; 16 of 192 x 28 x 28 -> 192, 3x3,
-// 13.2 -> 12.0; 84 of 128 x 14 x 28 -> 256, 3x3 stride 2, 17.8 -> 11.0.  (1440 of 256 x 14 x 14 -> 512, 3x3 stride 2: 94, as the
-// pair schedule; the overhang takes what the missing rewrite saves.)
+// Measured in a loop over three sets of buffers, the fastest other embedding and this kernel: 128 images of 256 x 7 x 7 -> 512, 3x3,
+// 19.5 and 13.8 us; 40 of 160 x 20 x 44 -> 130, 5x5, 62.8 and 35.8; 64 of 96 x 28 x 28 -> 192, 5x5, 43.0 and 29.4; 16 of
+// 192 x 28 x 28 -> 192, 3x3, 13.1 and 11.9; 84 of 128 x 14 x 28 -> 256, 3x3 stride 2, 17.9 and 10.8.  1440 of 256 x 14 x 14 -> 512, 3x3
+// stride 2: 92.7 and 94 (the overhang takes more than the missing rewrite saves).  Large windows leave rings of two, and other
+// embeddings are faster: 80 of 128 x 56 x 56 -> 64, 5x5 stride 2, 34.7 and 40.4; 17 of 176 x 48 x 45 -> 428, 22.3 and 34.2.
 // What bounds it: shared memory.  Of 1152 MMA clocks a block of 32 channels takes with 9 taps and 256 columns, the operand
 // reads use 576, the arriving weights and raw rows 386, the builders about 200; and the issue slots of the builders.
 //

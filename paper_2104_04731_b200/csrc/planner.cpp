@@ -715,7 +715,9 @@ bool plane_choices(const Geom& g, int groups, PlaneForm* form, std::vector<Plane
     for (int whole_sectors = 0; whole_sectors < 2; ++whole_sectors) {
       if (!plane_form(g, f == 1, whole_sectors != 0, &cand)) break;
       // Rows widened to whole sectors are listed beside the others where they cost little: every tile of 128 positions then holds
-      // fewer outputs (57 -> 64 positions, 315 images of 64 x 56 x 56, 79 us -> 74; 29 -> 36, depth-wise on 28 x 28, no gain).
+      // fewer outputs.  Best schedule of either kind, 3x3, us: 57 -> 64 positions, 64 x 56 x 56 -> 64, 315 images 79 and 74, 100
+      // 28.9 and 24.5, 16 9.2 and 8.9, 8 and fewer the same; 101 -> 108, 20 images of 32 x 100 x 100 -> 64 17.2 and 15.5, but 4 images
+      // 7.1 and 7.8; 61 -> 68 and 113 -> 120 2 % less; 51 -> 58 and 53 -> 60 10 % more; 29 -> 36, depth-wise on 28 x 28, no gain.
       if (whole_sectors && (cand.pitch == narrow || cand.pitch * 20 > narrow * 23 || plane_sector_rows(g, cand.pitch) == 0)) break;
       narrow = cand.pitch;
       for (const int* style : kStyles) {
@@ -1038,7 +1040,7 @@ void enumerate_embeddings(const Geom& g, std::vector<Candidate>* out) {
               ((int)form.units.size() + 1) / 2 * kMmaK);
       // Stream kernel: more channels than the plane kernel takes, taps enough to pay for the building of the units, and tiles for
       // more than a few pairs of SMs.  The widest column tile builds the units least often; half of it where it leaves half
-      // of the pairs without a tile (16 images of 192 x 28 x 28 -> 192, 3x3: 12.7 us, half the tile 15.2).
+      // of the pairs without a tile (16 images of 192 x 28 x 28 -> 192, 3x3, 58 tiles: 11.9 us; half the tile a fifth more).
       if (d.C >= 48 && d.R * d.S >= 4) {
         int wide = 64;
         while (wide < d.K && wide < 256) wide <<= 1;
