@@ -20,6 +20,19 @@ namespace b2c {
 
 namespace {
 
+// Barrier `id` of `threads` threads; true if all of them brought true.
+__device__ __forceinline__ bool barrier_and(int id, int threads, bool mine) {
+  uint32_t all;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.u32 q, %3, 0;\n"
+      "barrier.cta.red.and.pred p, %1, %2, q;\n"
+      "selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(all)
+      : "r"(id), "r"(threads), "r"((uint32_t)mine)
+      : "memory");
+  return all != 0;
+}
+
 // PERSIST: 0 = one tile per block; 1 = persistent, one block per SM (wide tiles, deep stage ring);
 // 2 = persistent, three blocks per SM (narrow tiles: short main loops, several epilogues in flight).
 template <int AMODE, int PERSIST>
@@ -412,7 +425,8 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
     const int tile_w_log2 = remap == 3 ? 31 - __clz(args.sh_wps) : 0;
     const int tile_h3 = kTileM >> tile_w_log2;
     const int row_in_tile = row >> tile_w_log2, col_in_tile = row & ((1 << tile_w_log2) - 1);
-    for (int t = tile_first; t < tile_end && ok; t += tile_step, ++ti) {
+    // (a staged-window warp whose wait gave up leaves with the others, where they meet)
+    for (int t = tile_first; t < tile_end && (ok || AMODE == A_STAGED); t += tile_step, ++ti) {
     if (alternate && (ti & 1) != half) continue;
     B2C_TILE_ORIGIN(t)
     const unsigned m = (unsigned)m0 + (unsigned)row;
@@ -511,8 +525,9 @@ __global__ void __launch_bounds__(kThreads, PERSIST == 1 ? 1 : 3) conv_mma_kerne
       // (rows outside the image and the left/right margins are zeros, so the gather below needs no
       // bounds tests); then each thread forms half a row of the A tile per stage from that window.
       const int tg = (int)threadIdx.x - 64;
-      // (persistent blocks: every thread must be done reading the previous tile's window)
-      if (ti > 0) asm volatile("bar.sync 1, %0;" ::"n"(kGatherWarps * 32) : "memory");
+      // (persistent blocks: every thread must be done reading the previous tile's window; and the warps hear whether
+      // one of them has given up a wait, since none may wait at this barrier for a warp that has left)
+      if (ti > 0 && !barrier_and(1, kGatherWarps * 32, ok)) break;
       const unsigned m_last = min((unsigned)m0 + (unsigned)kTileM - 1u, (unsigned)args.Mg - 1u);
       const int img0 = (int)args.div_pq.div((uint32_t)m0);
       const int p_first = (int)args.div_q.div((uint32_t)(m0 - img0 * args.PQ));

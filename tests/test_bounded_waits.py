@@ -29,3 +29,12 @@ def test_results_of_waits_are_voted():
         if own:  # then nothing but the vote looks at it
             assert not re.search(r"&& ok\b", "\n".join(lines)), os.path.basename(path)
     assert waits > 20
+
+
+def test_staged_window_warps_leave_together():
+    """They meet at a barrier in every tile after the first; a warp whose wait gave up still comes there, with its word for it."""
+    source = open(os.path.join(CSRC, "conv_mma.cu")).read()
+    role = source[source.index("gather + epilogue warps"):]
+    assert "(ok || AMODE == A_STAGED)" in role.split("B2C_TILE_ORIGIN", 1)[0]
+    first = re.search(r'if \(ti > 0[^\n]*', role).group(0)
+    assert "!barrier_and(1, kGatherWarps * 32, ok)) break;" in first
