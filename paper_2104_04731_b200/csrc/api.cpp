@@ -643,36 +643,29 @@ struct LaneBuffers {
   int8_t* y8;
   void* ws;
 };
-// Copies of the activations and results that successive runs of a timing take in turn.  A program's next pass comes with
-// other buffers, and a layer whose tensors fill most of L2 then reads and writes memory, where a replay on one set stays
-// in L2: 32 images of 1 x 700 x 161, 20x5 stride 2 (114 MB), two schedules on one set 28.7 and 29.0 us, on three 32.0
-// and 29.6.  Below a third of L2 the passes of a program may stay there as well, and above twice its size one set is enough.
-struct RunSets {
+// Copies of the results that successive runs of a timing take in turn.  A program's next pass comes with other buffers, and a
+// layer whose tensors fill most of L2 then writes memory, where a replay on one set stays in L2: 32 images of
+// 1 x 700 x 161, 20x5 stride 2 (114 MB), two schedules on one set 28.7 and 29.1 us, on three 31.9 and 29.9.  Below a third of
+// L2 the passes of a program may stay there as well; one and a half times its size is enough.
+struct ResultSets {
   int n;
-  size_t x_step, y_step;  // elements from one copy to the next
+  size_t step;  // elements from one copy to the next
 };
-RunSets run_sets(const Geom& g) {
-  const size_t l2 = 126u << 20;
-  const size_t bytes = (size_t)g.x_elems + (size_t)g.y_elems * ((g.d.out_mode & B2C_OUT_I32 ? 4 : 0) + (g.d.out_mode & B2C_OUT_I8 ? 1 : 0));
-  RunSets s = {1, 0, 0};
-  if (bytes >= l2 / 3 && bytes < 2 * l2) s.n = (int)((2 * l2 + bytes - 1) / bytes);
-  if (s.n > 1) {
-    s.x_step = ((size_t)g.x_elems + 255) & ~(size_t)255;
-    s.y_step = ((size_t)g.y_elems + 255) & ~(size_t)255;
-  }
-  return s;
+ResultSets result_sets(const Geom& g) {
+  const size_t l2 = 126u << 20, enough = l2 + l2 / 2, x = (size_t)g.x_elems;
+  const size_t y = (size_t)g.y_elems * ((g.d.out_mode & B2C_OUT_I32 ? 4 : 0) + (g.d.out_mode & B2C_OUT_I8 ? 1 : 0));
+  if (x + y < l2 / 3 || x + y >= enough) return ResultSets{1, 0};
+  return ResultSets{(int)std::min<size_t>(4, (enough - x + y - 1) / y), ((size_t)g.y_elems + 255) & ~(size_t)255};
 }
-// Allocates them: the activations, and the results of each lane that the layer has; one copy where there is no room for more.
-bool alloc_tensors(const Geom& g, LaneBuffers* lane, int lanes, RunSets* sets, int8_t** x) {
+// Allocates the results that the layer has, for each lane; one copy where there is no room for more.
+bool alloc_results(const Geom& g, LaneBuffers* lane, int lanes, ResultSets* sets) {
   while (true) {
-    const size_t x_more = (sets->n - 1) * sets->x_step, y_more = (sets->n - 1) * sets->y_step;
-    bool ok = cudaMalloc(x, g.x_elems + x_more + 256) == cudaSuccess;
+    const size_t elems = g.y_elems + (sets->n - 1) * sets->step;
+    bool ok = true;
     for (int l = 0; l < lanes && ok; ++l)
-      ok = ((g.d.out_mode & B2C_OUT_I8) == 0 || cudaMalloc(&lane[l].y8, g.y_elems + y_more + 256) == cudaSuccess) &&
-           ((g.d.out_mode & B2C_OUT_I32) == 0 || cudaMalloc(&lane[l].y32, (g.y_elems + y_more) * 4 + 256) == cudaSuccess);
+      ok = ((g.d.out_mode & B2C_OUT_I8) == 0 || cudaMalloc(&lane[l].y8, elems + 256) == cudaSuccess) &&
+           ((g.d.out_mode & B2C_OUT_I32) == 0 || cudaMalloc(&lane[l].y32, elems * 4 + 256) == cudaSuccess);
     if (ok || sets->n == 1) return ok;
-    cudaFree(*x);
-    *x = nullptr;
     for (int l = 0; l < lanes; ++l) {
       cudaFree(lane[l].y8);
       cudaFree(lane[l].y32);
@@ -680,11 +673,11 @@ bool alloc_tensors(const Geom& g, LaneBuffers* lane, int lanes, RunSets* sets, i
       lane[l].y32 = nullptr;
     }
     (void)cudaGetLastError();
-    *sets = RunSets{1, 0, 0};
+    *sets = ResultSets{1, 0};
   }
 }
 
-int time_plan(b2c_plan* p, const int8_t* x, const LaneBuffers* lane, int lanes, const RunSets& sets, float* us) {
+int time_plan(b2c_plan* p, const int8_t* x, const LaneBuffers* lane, int lanes, const ResultSets& sets, float* us) {
   const int iters = 10, replays = 5;
   cudaStream_t st[kMaxLanes] = {};
   cudaEvent_t e0 = nullptr, e1 = nullptr, fork = nullptr, join[kMaxLanes] = {};
@@ -713,8 +706,8 @@ int time_plan(b2c_plan* p, const int8_t* x, const LaneBuffers* lane, int lanes, 
       for (int i = 0; i < iters && rc == B2C_OK && e == cudaSuccess; ++i)
         for (int l = 0; l < lanes && rc == B2C_OK; ++l) {
           const LaneBuffers& b = lane[l];
-          const size_t c = (size_t)(i % sets.n);
-          rc = b2c_conv2d_int8_run(p, x + c * sets.x_step, b.y32 ? b.y32 + c * sets.y_step : nullptr, b.y8 ? b.y8 + c * sets.y_step : nullptr, b.ws, st[l]);
+          const size_t at = (size_t)(i % sets.n) * sets.step;
+          rc = b2c_conv2d_int8_run(p, x, b.y32 ? b.y32 + at : nullptr, b.y8 ? b.y8 + at : nullptr, b.ws, st[l]);
         }
       for (int l = 1; l < lanes && e == cudaSuccess; ++l) {
         e = cudaEventRecord(join[l], st[l]);
@@ -874,17 +867,16 @@ int b2c_plan_create(const b2c_conv_desc* desc, int32_t policy_or_id, void* cuda_
       cudaFree(lane[l].ws);
     }
   };
-  // (sixteen lanes have tensors enough)
-  RunSets sets = lanes == 1 ? run_sets(g) : RunSets{1, 0, 0};
-  bool alloc_ok = cudaMalloc(&w, g.w_elems + 256) == cudaSuccess;
+  ResultSets sets = lanes == 1 ? result_sets(g) : ResultSets{1, 0};  // (sixteen lanes have results enough)
+  bool alloc_ok = cudaMalloc(&x, g.x_elems + 256) == cudaSuccess && cudaMalloc(&w, g.w_elems + 256) == cudaSuccess &&
+                  alloc_results(g, lane, lanes, &sets);
   for (int l = 0; l < lanes && alloc_ok; ++l) alloc_ok = cudaMalloc(&lane[l].ws, ws_max + 1024) == cudaSuccess;
-  alloc_ok = alloc_ok && alloc_tensors(g, lane, lanes, &sets, &x);
   if (!alloc_ok) {
     set_last_cuda_error((int)cudaGetLastError());
     cleanup();
     return B2C_E_CUDA;
   }
-  cudaMemsetAsync(x, 1, g.x_elems + (sets.n - 1) * sets.x_step, st);
+  cudaMemsetAsync(x, 1, g.x_elems, st);
   cudaMemsetAsync(w, 1, g.w_elems, st);
   cudaStreamSynchronize(st);
   int best = -1;
@@ -1020,8 +1012,9 @@ int b2c_plan_create_grouped_timed(const b2c_conv_desc* desc, int32_t groups, voi
   int8_t *x = nullptr, *w = nullptr;
   LaneBuffers lane = {};
   const size_t w_bytes = (size_t)desc->K * (desc->C / groups) * desc->R * desc->S;
-  RunSets sets = run_sets(g);
-  bool ok = cudaMalloc(&w, w_bytes + 256) == cudaSuccess && cudaMalloc(&lane.ws, 1024) == cudaSuccess && alloc_tensors(g, &lane, 1, &sets, &x);
+  ResultSets sets = result_sets(g);
+  bool ok = cudaMalloc(&x, g.x_elems + 256) == cudaSuccess && cudaMalloc(&w, w_bytes + 256) == cudaSuccess && alloc_results(g, &lane, 1, &sets) &&
+            cudaMalloc(&lane.ws, 1024) == cudaSuccess;
   float us = -1;
   auto timed = [&](b2c_plan* q, float* t) {
     const bool good = b2c_plan_set_weights(q, w, st) == B2C_OK && cudaStreamSynchronize(st) == cudaSuccess &&
@@ -1031,7 +1024,7 @@ int b2c_plan_create_grouped_timed(const b2c_conv_desc* desc, int32_t groups, voi
     return good;
   };
   if (ok) {
-    cudaMemsetAsync(x, 1, g.x_elems + (sets.n - 1) * sets.x_step, st);
+    cudaMemsetAsync(x, 1, g.x_elems, st);
     cudaMemsetAsync(w, 1, w_bytes, st);
     if (!timed(inplace, &us)) us = -1;
     inplace->emb.device_us = us;
