@@ -13,8 +13,10 @@
 // 192 x 28 x 28 -> 192, 3x3, 13.1 and 11.9; 84 of 128 x 14 x 28 -> 256, 3x3 stride 2, 17.9 and 10.8.  1440 of 256 x 14 x 14 -> 512, 3x3
 // stride 2: 92.7 and 94 (the overhang takes more than the missing rewrite saves).  Large windows leave rings of two, and other
 // embeddings are faster: 80 of 128 x 56 x 56 -> 64, 5x5 stride 2, 34.7 and 40.4; 17 of 176 x 48 x 45 -> 428, 22.3 and 34.2.
-// What bounds it: shared memory.  Of 1152 MMA clocks a block of 32 channels takes with 9 taps and 256 columns, the operand
-// reads use 576, the arriving weights and raw rows 386, the builders about 200; and the issue slots of the builders.
+// What bounds it: no unit is full (1536 images of the last shape under ncu: tensor pipe 58 % of the time, issue slots 45, L1 41);
+// a window's way through the builders, whose waits and fences take the most issue opportunities, and at the boards' power limit the
+// clock.  By count, of 1152 MMA clocks that a block of 32 channels takes with 9 taps and 256 columns, shared memory is busy for all:
+// operand reads 576, arriving weights and raw rows 386, builders about 200.
 //
 // A tile is th grid rows of the whole batch per block (th x pitch <= 128 positions), so that both blocks' operands start
 // at the same address, which the pair's one descriptor needs.  Grid, phases and units are those of the plane kernel's channel
